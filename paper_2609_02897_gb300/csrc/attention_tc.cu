@@ -399,7 +399,13 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
     if (valid < kKeys) {
       // ragged tile: V rows past the last valid key may hold anything; zero
       // them so that 0 * V stays 0, once the V tile has landed (it comes
-      // through its own ring and may still be in flight)
+      // through its own ring and may still be in flight).  The slot's previous
+      // tile must have been consumed first: S runs up to three tiles ahead of
+      // P.V, so with a late V ring that tile may not even have landed, and the
+      // parity of its phase would then pass for this tile's.
+      const int pt = t - G::kVStages;
+      if (!bad && pt >= 0 && !wait_all(&pv_done[pt % kSBufs], (pt / kSBufs) & 1, budget))
+        bad = true;
       if (!bad && wait_all(&v_full[t % G::kVStages], (t / G::kVStages) & 1, budget)) {
         uint8_t* vt = gbase + G::kVOff + (t % G::kVStages) * G::kTileBytes;
         constexpr int kChunksPerRow = G::kNH * 8;
