@@ -144,7 +144,10 @@ typedef struct asd_dims {
 /* Bytes of device workspace that the calls below need for `total_nodes`
  * nodes with these dims on the current device (depends on its SM count).
  * Returns 0 if the dims are invalid.  The workspace needs no initialisation;
- * its address must be 256-byte aligned. */
+ * its address must be 256-byte aligned.  The last part of it, up to about
+ * 10 MB (bf16 dims), holds the partial results of an attention whose contexts
+ * are cut into chunks: with a workspace that ends before it, as one sized for
+ * other dims may, the calls work and split less. */
 size_t asd_workspace_bytes(const asd_dims* dims, int32_t total_nodes);
 
 /*
@@ -313,12 +316,16 @@ int32_t asd_abi_version(void);
 int32_t asd_lm_head_variant(const asd_dims* dims, int32_t total_nodes, const void* w_lm);
 
 /*
- * Which tree-attention kernel a call with these dims and node count runs (a
- * diagnostic query; no counterpart in the paper; nothing is launched): 1 the
+ * Which tree-attention kernel a verify step with these dims and node count runs
+ * (a diagnostic query; no counterpart in the paper; nothing is launched): 1 the
  * bf16 split-KV kernel beside the LM head (up to 128 nodes), 2 the tensor-core
  * kernel with one 128-row query tile per CTA, 3 the tensor-core kernel with two
  * query tiles per CTA in ping-pong (when its 256-row items fill at least two
  * waves of CTAs), 4 the fp32 kernel, 0 for invalid arguments.
+ * asd_tree_attention by itself has no LM head to share the SMs with and runs
+ * form 2 where a step runs form 1 (same semantics, other roundings).  Form 2
+ * may cut long contexts into chunks, whose length follows the batch's context
+ * lengths.
  */
 int32_t asd_attention_variant(const asd_dims* dims, int32_t total_nodes);
 

@@ -173,6 +173,24 @@ WsLayout layout(const asd_dims& d, int T, int nsm) {
     L.lz_h = off;      off = align256(off + 2 * 2 * static_cast<size_t>(L.lz_cap) * d.hidden);
   }
   L.total = off;
+  // The split attention's partial rows come last and are optional: with a
+  // workspace that ends before them (one sized for another batch) the
+  // attention splits as far as they fit, or not at all.  An every-row
+  // workspace stays within ASD_NOALLOC_SCRATCH_BYTES wherever it would without
+  // them, so that asd_workspace_bytes still tells what the allocation-free
+  // LM head accepts.
+  L.at_part = L.full = off;
+  const long long rows = d.dtype == ASD_BF16
+                             ? nsm * std::min<long long>(kAttnTcRows, static_cast<long long>(d.max_nodes) * G)
+                             : 0;
+  if (rows > 0) {
+    const size_t want = align256(sizeof(int2) * static_cast<size_t>(d.batch)) +
+                        static_cast<size_t>(rows) * (sizeof(float2) + 4 * static_cast<size_t>(d.head_dim));
+    const size_t room = d.lm_head_schedule == ASD_LM_LAZY_LEVELS ? want
+                        : off < ASD_NOALLOC_SCRATCH_BYTES        ? ASD_NOALLOC_SCRATCH_BYTES - off
+                                                                 : 0;
+    L.full = off + std::min(want, room);
+  }
   return L;
 }
 
@@ -189,6 +207,7 @@ struct Ctx {
   int T;
   cudaStream_t st;
   void* ws;
+  size_t ws_bytes;
 };
 
 // Wait budget (SM clock cycles) that asd_debug_set_wait_cycles set for the
@@ -210,6 +229,7 @@ asd_status begin_call(const asd_dims* dims, int32_t total_nodes, void* ws, size_
   if (ws_bytes < c->L.total) return ASD_ERR_WORKSPACE;
   c->st = static_cast<cudaStream_t>(stream);
   c->ws = ws;
+  c->ws_bytes = ws_bytes;
   if (cudaMemsetAsync(ws_at<int>(ws, c->L.status), 0, 16, c->st) != cudaSuccess)
     return ASD_ERR_CUDA;
   // a test's shorter wait budget rides in words 2-3 of the status block
@@ -246,7 +266,7 @@ PrepParams prep_params(const Ctx& c, const int32_t* parent, const int32_t* token
 asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const void* v_cache,
                          const int32_t* page_table, const int32_t* ctx_len, const void* tree_k,
                          const void* tree_v, const int32_t* parent, const int32_t* cu,
-                         void* out) {
+                         void* out, bool in_step) {
   const asd_dims& d = c.d;
   AttnParams a{};
   a.q = q;
@@ -276,7 +296,11 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
   a.max_nodes = d.max_nodes;
   a.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(d.head_dim)));
   cudaError_t err;
-  if (c.L.attn_tc) {
+  // up to 128 nodes the mma.sync kernel runs beside the LM head of a verify
+  // step; with the SMs to itself the tensor-core kernel is the faster one at
+  // every size
+  const int tc = c.L.attn_tc ? c.L.attn_tc : (d.dtype == ASD_BF16 && !in_step ? 1 : 0);
+  if (tc) {
     CUtensorMap tk, tv, ttk, ttv, tq;
     uint64_t rows;
     uint32_t box_rows;
@@ -300,7 +324,22 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
       if (!make_q_tmap_bf16(&tq, q, d.head_dim, d.num_q_heads, c.T, a.G)) return ASD_ERR_CUDA;
       a.q_tma = 1;
     }
-    err = launch_attention_tc(a, tk, tv, ttk, ttv, tq, c.L.attn_tc == 2, c.st);
+    a.nsm = device_sm_count();
+    if (tc == 1) {
+      // a standalone call has no use for the LM head's partials either
+      const size_t at = in_step ? c.L.at_part : c.L.lm_part;
+      const size_t rows_at = at + align256(sizeof(int2) * static_cast<size_t>(d.batch));
+      const size_t row_bytes = sizeof(float2) + 4 * static_cast<size_t>(d.head_dim);
+      const size_t end = std::min(c.ws_bytes, c.L.full);
+      if (end > rows_at) {
+        a.part_cap = std::min<long long>(attention_split_rows(d, c.T, a.nsm),
+                                         static_cast<long long>((end - rows_at) / row_bytes) & ~63LL);
+        a.plan = ws_at<int2>(c.ws, at);
+        a.part_ml = ws_at<float2>(c.ws, rows_at);
+        a.part_o = ws_at<float>(c.ws, rows_at + sizeof(float2) * static_cast<size_t>(a.part_cap));
+      }
+    }
+    err = launch_attention_tc(a, tk, tv, ttk, ttv, tq, tc == 2, c.st);
   } else if (d.dtype == ASD_BF16) {
     CUtensorMap tk, tv;
     uint64_t rows;
@@ -564,7 +603,7 @@ size_t asd_workspace_bytes(const asd_dims* dims, int32_t total_nodes) {
   if (!dims_ok(dims) || !nodes_ok(dims, total_nodes)) return 0;
   const int nsm = device_sm_count();
   if (nsm <= 0) return 0;
-  return layout(*dims, total_nodes, nsm).total;
+  return layout(*dims, total_nodes, nsm).full;
 }
 
 asd_status asd_tree_attention(const asd_dims* dims, const void* q, const void* k_cache,
@@ -587,7 +626,7 @@ asd_status asd_tree_attention(const asd_dims* dims, const void* q, const void* k
       cudaSuccess)
     return ASD_ERR_CUDA;
   return run_attention(c, q, k_cache, v_cache, page_table, ctx_len, tree_k, tree_v, parent,
-                       cu_nodes, out);
+                       cu_nodes, out, false);
 }
 
 asd_status asd_lmhead_margin(const asd_dims* dims, const void* hidden, const void* w_lm,
@@ -719,7 +758,7 @@ asd_status asd_verify_step(const asd_dims* dims, const asd_verify_args* a, void*
   if (st != ASD_OK) return st;
   record(a->stage_events[2], c.st);
   st = run_attention(c, a->q, a->k_cache, a->v_cache, a->page_table, a->ctx_len, a->tree_k,
-                     a->tree_v, a->parent, a->cu_nodes, a->attn_out);
+                     a->tree_v, a->parent, a->cu_nodes, a->attn_out, true);
   if (st != ASD_OK) return st;
   record(a->stage_events[3], c.st);
   TailParams t = tail_params(c, (lazy ? 0 : kTailFinalize) | kTailWalk | kTailCompact);

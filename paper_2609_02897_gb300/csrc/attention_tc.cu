@@ -1,14 +1,26 @@
 // Tree attention (Sec. 2 "Verify": the target scores every drafted node in
-// one forward pass) on the 5th-generation tensor cores, for steps where the
-// attention kernel has the SMs to itself (more than 128 tree nodes: the LM
-// head then takes most of an SM's shared memory and runs first).  bf16 in,
-// fp32 accumulate.
+// one forward pass) on the 5th-generation tensor cores, where the attention
+// kernel has the SMs to itself: a standalone attention call, or a step of more
+// than 128 tree nodes (the LM head then takes most of an SM's shared memory
+// and runs first).  bf16 in, fp32 accumulate.
 //
-// Work item (one CTA): 128 query rows of one (sequence, KV head) pair, the
-// whole context; the CTAs take the sequences in decreasing order of work, so
-// the longest items start first.  The rows of a pair are its N nodes times
-// the G query heads that share the KV head, node-major (row r -> node r / G,
-// head g*G + r % G); row r lives in TMEM lane r.  Keys come in tiles of 128,
+// Measured, a whole asd_tree_attention call: one sequence, 8 nodes, context
+// 32768 in a cache of 40960 slots 186.5 -> 36.9 us (134 MB of K/V; the
+// mma.sync kernel in 8 splits of the cache's capacity before), 4 sequences of
+// 60 nodes, contexts 901 to 3625 41.0 -> 32.4 us (unsplit before).
+//
+// Work item (one CTA): 128 query rows of one (sequence, KV head) pair and a
+// chunk of its keys: the whole context, or, when the items would leave SMs
+// idle, one of up to kMaxChunks equal runs of key tiles.  The chunk length is
+// one for the whole step and is chosen in-kernel from the context lengths
+// (chunk_length: the host knows the cache's capacity only, which says little
+// about them), so a cache sized for many times the context splits like a tight
+// one.  A chunk leaves its unnormalised O, reference max and row sum in the
+// workspace, and attn_merge_kernel, a warp per query row, combines them.  The
+// CTAs take the chunks in decreasing order of work, so the longest start
+// first.  The rows of a pair are its N nodes times the G query heads that
+// share the KV head, node-major (row r -> node r / G, head g*G + r % G); row r
+// lives in TMEM lane r.  Keys come in tiles of 128,
 // K and V through TMA rings of their own (128-byte swizzle; paged caches one
 // box per page; the tree K/V through a 3D map over [T, Hkv, D]), so a K slot
 // is refilled as soon as its S MMA is done rather than after the tile's P.V;
@@ -33,10 +45,12 @@
 // TMEM (512 columns): O [0, D), S/P [128, 256), [256, 384), [384, 512).
 // Shared memory: Q, a 3-stage K ring and a V ring (160 KB of rings for D =
 // 128).
-// Warp roles (384 threads): warp 0 K producer, warp 1 TMEM allocator and
-// issuer of the S MMAs, warps 2-9 softmax and epilogue, two per TMEM lane
-// quarter, each on one half of every tile's keys, warp 10 issuer of the P.V
-// MMAs, warp 11 V producer.
+// Warp roles (384 threads): warp 0 K producer, warp 1 issuer of the S MMAs,
+// warps 2-9 softmax and epilogue, two per TMEM lane quarter, each on one half
+// of every tile's keys, warp 10 TMEM allocator and issuer of the P.V MMAs,
+// warp 11 V producer.
+#include <algorithm>
+
 #include "kernels.h"
 #include "tc.cuh"
 
@@ -112,7 +126,10 @@ __device__ __forceinline__ bool aborted_warp(volatile int* s_abort) {
 
 struct Item {
   int b, g, s0, n, r0, nrows, R;
-  int ctx, nctx, ntree, ntiles;
+  int key_base;              // first context key of the chunk (a multiple of kKeys)
+  int ctx;                   // context length past key_base
+  int nctx, ntree, ntiles;   // context, tree and all key tiles of the chunk
+  int chunks, chunk, part0;  // chunks of the sequence, this one, the sequence's partial rows
 };
 
 constexpr int kOrderMax = 256;   // batches ordered by work in-kernel (larger ones: index order)
@@ -145,26 +162,177 @@ __device__ __forceinline__ int sequence_of_rank(const AttnParams& p, int r, int*
   return *s_b;
 }
 
-// blockIdx.y = (r, g): KV head g of the sequence of rank r (sequence_of_rank);
-// blockIdx.x: the item's block of query rows.
-__device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, int* s_work, int* s_b) {
-  const int rb = blockIdx.x, bg = blockIdx.y;
-  const int r = bg / p.Hkv;
-  it.b = sequence_of_rank(p, r, s_work, s_b);
-  it.g = bg - r * p.Hkv;
-  it.s0 = p.cu_nodes[it.b];
-  it.n = p.cu_nodes[it.b + 1] - it.s0;
+constexpr int kMaxChunks = 32;   // chunks per sequence: one lane of the merging warp each
+constexpr float kMergeOverhead = 3.f;   // cost of the merge in key tiles of ~1 us
+
+// Shared-memory scratch of make_item, one entry per sequence.
+struct PlanSmem {
+  int s0[kOrderMax], n[kOrderMax], ctx[kOrderMax];   // first node, nodes, context length
+  int tiles[kOrderMax];    // key tiles (0: no query rows)
+  int items[kOrderMax];    // query row blocks x KV heads, then CTAs
+  int key[kOrderMax];      // key tiles of the longest chunk
+  int part[kOrderMax];     // partial rows (0: one chunk)
+  float cost[kMaxChunks];  // of cutting the longest sequence into 1, 2, ... chunks
+  int seq, first, part0;   // the sequence of this CTA, its first CTA and partial row
+};
+
+// ceil(t / len) for 0 <= t from inv ~ 1 / len, for quotients up to kMaxChunks
+// (the estimate is then off by one at most).
+__device__ __forceinline__ int ceil_div_est(int t, int len, float inv) {
+  int c = static_cast<int>(static_cast<float>(t) * inv);
+  c -= (c - 1) * len >= t ? 1 : 0;
+  c += c * len < t ? 1 : 0;
+  c += c * len < t ? 1 : 0;
+  return c;
+}
+
+// Key tiles per chunk.  Warp w weighs cutting the longest sequence into w + 1,
+// w + 1 + warps, ... chunks (and the others into chunks no longer than its),
+// its lanes summing over the sequences.  The chunks run at once, one CTA per
+// SM (a second wave would pay a CTA's overhead again), so a step takes its
+// longest chunk: the shortest length that fits, unless the merge costs more
+// than the cut saves.  Every thread of the CTA calls it (it synchronises the
+// CTA) and returns the same length.
+__device__ __forceinline__ int chunk_length(const AttnParams& p, PlanSmem& s) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int longest = 1, items = 0;
+  for (int q = lane; q < p.B; q += 32) {
+    longest = max(longest, s.tiles[q]);
+    items += s.items[q];
+  }
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  items = __reduce_add_sync(0xffffffffu, items);
+  if (items == 0 || items > p.nsm) return longest;   // uniform over the CTA
+  for (int k = warp; k < kMaxChunks; k += kThreads / 32) {
+    const int len = (longest + k) / (k + 1);
+    const float inv = 1.f / static_cast<float>(len);
+    int ctas = 0, part = 0;
+    for (int q = lane; q < p.B; q += 32) {
+      const int c = ceil_div_est(s.tiles[q], len, inv);
+      ctas += s.items[q] * c;
+      part += c > 1 ? s.n[q] * p.Hq * c : 0;
+    }
+    ctas = __reduce_add_sync(0xffffffffu, ctas);
+    part = __reduce_add_sync(0xffffffffu, part);
+    // one chunk each (k = 0) is always possible
+    if (lane == 0)
+      s.cost[k] = k > 0 && (part > p.part_cap || ctas > p.nsm)
+                      ? INFINITY
+                      : static_cast<float>(len) + (part > 0 ? kMergeOverhead : 0.f);
+  }
+  __syncthreads();
+  static_assert(kMaxChunks == 32, "a lane per candidate");
+  const float cost = s.cost[lane];
+  float best = cost;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+  const int k = __ffs(__ballot_sync(0xffffffffu, cost == best)) - 1;
+  return (longest + k) / (k + 1);
+}
+
+// The chunk of CTA blockIdx.x: sequences in decreasing order of their chunks'
+// length (ties by index), within one its KV heads, its chunks, its blocks of
+// query rows (which read the same keys) innermost.  False when the CTA has
+// none.  Every thread of the CTA calls it (it synchronises the CTA).
+__device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSmem& s) {
+  const int idx = blockIdx.x;
+  int local, ctx;
+  if (p.B > kOrderMax) {   // index order, unsplit
+    const int rbmax = (p.max_nodes * p.G + kRows - 1) / kRows;
+    it.b = idx / (rbmax * p.Hkv);
+    if (it.b >= p.B) {
+      __syncthreads();
+      return false;
+    }
+    local = idx - it.b * rbmax * p.Hkv;
+    it.g = local / rbmax;
+    it.r0 = (local - it.g * rbmax) * kRows;
+    it.chunks = 1;
+    it.chunk = 0;
+    it.part0 = 0;
+    it.s0 = p.cu_nodes[it.b];
+    it.n = p.cu_nodes[it.b + 1] - it.s0;
+    ctx = min(max(p.ctx_len[it.b], 0), p.ctx_max);
+    __syncthreads();
+  } else {
+    // sequence extents and context lengths are caller inputs (the tree
+    // preparation reports bad ones): a malformed sequence gets no CTA
+    if (threadIdx.x == 0) s.seq = -1;
+    for (int q = threadIdx.x; q < p.B; q += blockDim.x) {
+      const int s0 = p.cu_nodes[q], n = p.cu_nodes[q + 1] - s0;
+      const int c = min(max(p.ctx_len[q], 0), p.ctx_max);
+      const bool okq = n > 0 && n <= kMaxNodes && s0 >= 0 && s0 + n <= p.T;
+      s.s0[q] = s0;
+      s.n[q] = n;
+      s.ctx[q] = c;
+      s.tiles[q] = okq ? (c + kKeys - 1) / kKeys + (n + kKeys - 1) / kKeys : 0;
+      s.items[q] = okq ? (n * p.G + kRows - 1) / kRows * p.Hkv : 0;
+      s.key[q] = s.tiles[q];
+      s.part[q] = 0;
+    }
+    __syncthreads();
+    int len = 0x3fffffff;
+    if (p.part_cap > 0) {
+      len = chunk_length(p, s);
+      __syncthreads();   // every warp has read s.items
+      for (int q = threadIdx.x; q < p.B; q += blockDim.x) {
+        const int t = s.tiles[q], c = (t + len - 1) / len;
+        if (c > 1) {
+          s.items[q] *= c;
+          s.key[q] = (t + c - 1) / c;
+          s.part[q] = s.n[q] * p.Hq * c;
+        }
+      }
+      __syncthreads();
+    }
+    // a warp per sequence, its lanes summing the CTAs and partial rows before it
+    const int lane = threadIdx.x & 31;
+    for (int q = threadIdx.x >> 5; q < p.B; q += kThreads / 32) {
+      const int key = s.key[q];
+      int first = 0, part = 0;
+      for (int j = lane; j < p.B; j += 32) {
+        const int kj = s.key[j];
+        const bool before = kj > key || (kj == key && j < q);
+        first += before ? s.items[j] : 0;
+        part += before ? s.part[j] : 0;
+      }
+      first = __reduce_add_sync(0xffffffffu, first);
+      part = __reduce_add_sync(0xffffffffu, part);
+      if (lane == 0 && idx >= first && idx < first + s.items[q]) {
+        s.seq = q;
+        s.first = first;
+        s.part0 = part;
+        if (idx == first && p.part_cap > 0)
+          p.plan[q] = make_int2(part, (s.tiles[q] + len - 1) / len);
+      }
+    }
+    __syncthreads();
+    it.b = s.seq;
+    if (it.b < 0) return false;
+    it.s0 = s.s0[it.b];
+    it.n = s.n[it.b];
+    ctx = s.ctx[it.b];
+    it.chunks = s.part[it.b] > 0 ? (s.tiles[it.b] + len - 1) / len : 1;
+    it.part0 = s.part0;
+    const int rb = (it.n * p.G + kRows - 1) / kRows;
+    local = idx - s.first;
+    const int gz = local / rb;
+    it.r0 = (local - gz * rb) * kRows;
+    it.g = gz / it.chunks;
+    it.chunk = gz - it.g * it.chunks;
+  }
   it.R = it.n * p.G;
-  it.r0 = rb * kRows;
-  // sequence extents and context lengths are caller inputs (the tree
-  // preparation reports bad ones); every access below stays in bounds anyway
   if (it.n <= 0 || it.n > kMaxNodes || it.s0 < 0 || it.s0 + it.n > p.T || it.r0 >= it.R)
     return false;
   it.nrows = min(kRows, it.R - it.r0);
-  it.ctx = min(max(p.ctx_len[it.b], 0), p.ctx_max);
-  it.nctx = (it.ctx + kKeys - 1) / kKeys;
-  it.ntree = (it.n + kKeys - 1) / kKeys;
-  it.ntiles = it.nctx + it.ntree;
+  const int nctx = (ctx + kKeys - 1) / kKeys, all = nctx + (it.n + kKeys - 1) / kKeys;
+  // chunk z: tiles [z all / chunks, (z + 1) all / chunks) of the context's, then the tree's
+  const int t0 = it.chunk * all / it.chunks, t1 = (it.chunk + 1) * all / it.chunks;
+  it.ntiles = t1 - t0;
+  it.nctx = min(t1, nctx) - t0;
+  it.ntree = it.ntiles - it.nctx;
+  it.key_base = t0 * kKeys;
+  it.ctx = ctx - it.key_base;
   return true;
 }
 
@@ -192,7 +360,7 @@ __device__ __forceinline__ void issue_half_tile(const AttnParams& p, const Item&
       tma_load_3d(dst + h * (kKeys * 128), tm_tree, bar, h * 64, it.g, it.s0 + key0, pol);
     return;
   }
-  const int row = (it.b * p.Hkv + it.g) * p.ctx_max + t * kKeys;
+  const int row = (it.b * p.Hkv + it.g) * p.ctx_max + it.key_base + t * kKeys;
 #pragma unroll
   for (int h = 0; h < G::kNH; ++h) tma_load_2d(dst + h * (kKeys * 128), tm, bar, h * 64, row, pol);
 }
@@ -212,7 +380,7 @@ __device__ __forceinline__ void issue_paged_half(const AttnParams& p, const Item
   const int ps = p.page_size;
   const int br = ps < kKeys ? ps : kKeys;
   const int nbox = kKeys / br;
-  const int key0 = t * kKeys;
+  const int key0 = it.key_base + t * kKeys;
   const int e_first = key0 / ps, e_last = (key0 + (nbox - 1) * br) / ps;
   if (chunk0 < 0 || e_first < chunk0 || e_last >= chunk0 + kPageChunk) {
     chunk0 = e_first;
@@ -226,7 +394,7 @@ __device__ __forceinline__ void issue_paged_half(const AttnParams& p, const Item
   int row = -1;
   if (lane < nbox) {
     const int key = key0 + lane * br;
-    if (key < it.ctx) {
+    if (key < it.key_base + it.ctx) {
       const int page = s_pages[key / ps - chunk0];
       if (page < 0 || page >= p.num_pages)
         set_status(p.status, ASD_ERR_CTX_RANGE);
@@ -270,16 +438,16 @@ __device__ __forceinline__ void issue_q_tile(const AttnParams& p, const Item& it
 // [32h, 32h + 32), which overlap S columns that both halves have read before
 // the exchange.  The row sum stays split between the two threads of a row
 // until the end.  Returns false (uniformly over the eight warps) when a
-// bounded wait gave up; otherwise inv = 1 / (row sum), with O complete in
-// TMEM.
+// bounded wait gave up; otherwise m_out and l_out are the row's reference max
+// and sum, with O complete in TMEM.
 template <int D>
 __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it, uint32_t tmem,
-                                             uint8_t* gbase, const uint64_t (*s_anc)[2],
+                                             uint8_t* gbase, int* s_par, uint64_t (*s_anc)[2],
                                              float (*s_mx)[2][kRows], float (*s_l)[kRows],
                                              uint64_t* q_ready, uint64_t* s_full,
                                              uint64_t* p_full, uint64_t* pv_done,
                                              uint64_t* v_full, volatile int* s_abort,
-                                             long long budget, float& inv) {
+                                             long long budget, float& m_out, float& l_out) {
   using G = TcGeom<D>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int hf = (warp - 2) >> 2;              // key half of every tile
@@ -309,6 +477,23 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
     if (lane == 0) mbar_arrive(smem_u32(q_ready));
   }
 
+  // ancestor bitmasks (self included) of the sequence's nodes for the tree
+  // tile; a malformed parent ends the walk, so it is bounded
+  for (int i = tid; i < it.n; i += kSoftmaxThreads) s_par[i] = p.parent[it.s0 + i];
+  softmax_sync();
+  for (int i = tid; i < it.n; i += kSoftmaxThreads) {
+    uint64_t lo = 0, hi = 0;
+    int u = i;
+    while (true) {
+      if (u < 64) lo |= 1ull << u; else hi |= 1ull << (u - 64);
+      const int pu = s_par[u];
+      if (pu < 0 || pu >= u) break;
+      u = pu;
+    }
+    s_anc[i][0] = lo;
+    s_anc[i][1] = hi;
+  }
+  softmax_sync();
   uint64_t alo = 0, ahi = 0;
   if (row < it.nrows) {
     const int node = (it.r0 + row) / p.G;
@@ -441,8 +626,8 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
   // the row sum over both halves
   s_l[hf][row] = l;
   softmax_sync();
-  l += s_l[hf ^ 1][row];
-  inv = l > 0.f ? 1.f / l : 0.f;
+  l_out = l + s_l[hf ^ 1][row];
+  m_out = m_ref;
   return true;
 }
 
@@ -471,16 +656,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ int s_pages[2][kPageChunk];   // K / V producer: staged page-table entries
   __shared__ int s_issued[2][KS > VS ? KS : VS];  // producer: K (0) / V (1) fills per stage
 
+  __shared__ PlanSmem s_plan;
+
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long budget = wait_budget(p.status);
-  __shared__ int s_work[kOrderMax];
-  __shared__ int s_seq;
-  Item it;
-  if (!make_item(p, it, s_work, &s_seq)) {  // no query rows here (uniform over the CTA)
-    pdl_wait();
-    return;
-  }
 
   uint32_t base = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (base & 1023u)) & 1023u;
@@ -488,7 +668,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   base += pad;
   const uint32_t q_s = base + G::kQOff, k_s0 = base + G::kKOff, v_s0 = base + G::kVOff;
 
-  if (threadIdx.x == 0) {
+  // The set-up that needs no item runs while the first loads of make_item are
+  // on their way; make_item synchronises the CTA, and from then on every role
+  // runs by itself (32 ragged sequences of 4 to 8 nodes, paged: 123.5 -> 120.9 us
+  // with the masks built by the softmax warps, beside the first copies).
+  if (threadIdx.x == 32 * 11) {
     for (int s = 0; s < KS; ++s) {
       mbar_init(smem_u32(&s_k_full[s]), 1);
       mbar_init(smem_u32(&s_k_empty[s]), 1);
@@ -510,53 +694,24 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(smem_u32(&s_mma_done[1]), 1);
     s_abort = 0;
     fence_mbar_init();
-    // The item's first copies go out before the rest of the set-up: its
-    // query tile (TMA form), then the first fill of both rings on a
-    // contiguous cache (the producers go on from there).  What the first S
-    // MMA waits for then lands while the CTA allocates TMEM and builds the
-    // ancestor masks.
-    const uint64_t pol = l2_policy_evict_first();
-    if (p.q_tma) issue_q_tile<D>(p, it, q_s, smem_u32(&s_q_ready), &tm_q, pol);
-    if (p.page_size == 0) {
-      for (int t = 0; t < KS && t < it.ntiles; ++t) {
-        issue_half_tile<D>(p, it, t, k_s0 + t * G::kTileBytes, smem_u32(&s_k_full[t]), &tm_k,
-                           &tm_tk, pol);
-        s_issued[0][t] = 1;
-        if (t < VS) {
-          issue_half_tile<D>(p, it, t, v_s0 + t * G::kTileBytes, smem_u32(&s_v_full[t]), &tm_v,
-                             &tm_tv, pol);
-          s_issued[1][t] = 1;
-        }
-      }
-    }
   }
-  if (warp == 1) {
+  if (warp == 10) {
     tmem_alloc(smem_u32(&s_tmem), kTmemCols);
     tmem_relinquish();
+    tc_fence_before();
   }
-  // ancestor bitmasks (self included) of the sequence's nodes for the tree
-  // tile; a malformed parent ends the walk, so it is bounded
-  for (int i = threadIdx.x; i < it.n; i += kThreads) s_par[i] = p.parent[it.s0 + i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < it.n; i += kThreads) {
-    uint64_t lo = 0, hi = 0;
-    int u = i;
-    while (true) {
-      if (u < 64) lo |= 1ull << u; else hi |= 1ull << (u - 64);
-      const int pu = s_par[u];
-      if (pu < 0 || pu >= u) break;
-      u = pu;
-    }
-    s_anc[i][0] = lo;
-    s_anc[i][1] = hi;
-  }
-  tc_fence_before();
-  __syncthreads();
+  Item it;
+  const bool some = make_item(p, it, s_plan);   // uniform over the CTA
   tc_fence_after();
+  if (!some) {   // no query rows here
+    if (warp == 10) tmem_dealloc(s_tmem, kTmemCols);
+    pdl_wait();
+    return;
+  }
   const uint32_t tmem = s_tmem;
 
   bool ok = false;           // softmax warps: O complete in TMEM
-  float inv = 0.f;
+  float m_row = 0.f, l_row = 0.f;
   if (warp == 0 || warp == 11) {
     // ----------------------------------------------------------- TMA producers
     // K and V come through rings of their own, each filled by its own warp
@@ -570,10 +725,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       prefetch_tmap(which ? &tm_tv : &tm_tk);
     }
     const uint64_t pol = l2_policy_evict_first();
+    if (which == 0 && lane == 0 && p.q_tma)
+      issue_q_tile<D>(p, it, q_s, smem_u32(&s_q_ready), &tm_q, pol);
     int chunk0 = -1;
     bool pok = true;
-    // on a contiguous cache the first fill of the ring went out with the set-up
-    for (int t = p.page_size == 0 ? ns : 0; pok && t < it.ntiles; ++t) {
+    for (int t = 0; pok && t < it.ntiles; ++t) {
       const int stage = t % ns;
       uint64_t* empty = which ? &s_v_empty[stage] : &s_k_empty[stage];
       uint64_t* full = which ? &s_v_full[stage] : &s_k_full[stage];
@@ -666,8 +822,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    ok = softmax_role<D>(p, it, tmem, gbase, s_anc, s_mx, s_l, &s_q_ready, s_s_full, s_p_full,
-                         s_pv_done, s_v_full, &s_abort, budget, inv);
+    ok = softmax_role<D>(p, it, tmem, gbase, s_par, s_anc, s_mx, s_l, &s_q_ready, s_s_full, s_p_full,
+                         s_pv_done, s_v_full, &s_abort, budget, m_row, l_row);
   }
 
   // ------------------------------------------------------------------ finish
@@ -675,19 +831,33 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();   // the tile buffers and the tensor cores are idle from here on
   tc_fence_after();
   if (warp >= 2 && warp < 10 && ok) {
-    // each thread writes its key half's share of the row: D/2 output columns
+    // each thread writes its key half's share of the row, D/2 columns: the
+    // output, or (one of several chunks) the fp32 partial that
+    // attn_merge_kernel combines
     const int hf = (warp - 2) >> 2;
     const int row = (warp & 3) * 32 + lane;   // TMEM lane = query row
     const uint32_t lane_base = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) +
                                static_cast<uint32_t>(hf * (D / 2));
     const bool mine = row < it.nrows;
+    const bool split = it.chunks > 1;
+    const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
     __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.out) +
                          (mine ? grow_of(p, it, row) : 0) * D + hf * (D / 2);
+    const size_t prow = mine && split ? static_cast<size_t>(it.part0) +
+                                            static_cast<size_t>(it.g * it.chunks + it.chunk) * it.R +
+                                            it.r0 + row
+                                      : 0;
+    if (mine && split && hf == 0) p.part_ml[prow] = make_float2(m_row, l_row);
 #pragma unroll 1
     for (int c = 0; c < D / 64; ++c) {
       float o[32];
       tmem_ld32(lane_base + 32 * c, o);   // every lane takes part in the warp-wide load
-      if (mine) {
+      if (mine && split) {
+        float4* po = reinterpret_cast<float4*>(p.part_o + prow * D + hf * (D / 2) + 32 * c);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          po[k] = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+      } else if (mine) {
 #pragma unroll
         for (int k = 0; k < 32; k += 8) {
           uint4 pk;
@@ -707,8 +877,104 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, kTmemCols);
+  if (warp == 10) tmem_dealloc(tmem, kTmemCols);
   pdl_wait();   // the next kernel's wait covers every earlier kernel
+}
+
+// Combines the chunks of every query row that attn_tc_kernel split:
+//   out = sum_z 2^(m_z - M) O_z / sum_z 2^(m_z - M) l_z,  M = max_z m_z.
+// W warps per row: lane z of each reads chunk z's (reference max, row sum),
+// warp w adds up chunks w, w + W, ..., each lane D/32 columns, eight loads in
+// flight, and the W sums meet in shared memory.  Few rows come in many chunks
+// and take W = 4 (256 rows in 19 chunks: 3.9 us, 9.7 with a warp per row),
+// many rows in few chunks and take W = 1 (7680 rows in up to 3 chunks: 3.4 us,
+// 11 with four warps, all of it CTA launches).  Sequences in one chunk
+// (plan[b].y == 1) were written by attn_tc_kernel.
+constexpr int kMergeThreads = 256;
+constexpr int kMergeFewRows = 2048;   // query rows of a step up to which W = 4
+constexpr int kMergeLoads = 8;
+
+template <int D, int W>
+__global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const AttnParams p) {
+  constexpr int kV = D / 32, kMergeWarps = W, kMergeRows = kMergeThreads / 32 / W;
+  __shared__ float s_acc[kMergeRows][kMergeWarps][D];
+  pdl_launch_dependents();
+  const int b = blockIdx.y / p.Hkv, g = blockIdx.y - b * p.Hkv;
+  const int lane = threadIdx.x & 31;
+  const int w = (threadIdx.x >> 5) % kMergeWarps, rl = (threadIdx.x >> 5) / kMergeWarps;
+  const int s0 = p.cu_nodes[b], n = p.cu_nodes[b + 1] - s0, R = n * p.G;
+  pdl_wait();
+  if (n <= 0 || n > kMaxNodes || s0 < 0 || s0 + n > p.T || static_cast<int>(blockIdx.x) * kMergeRows >= R)
+    return;
+  const int2 plan = __ldcg(p.plan + b);
+  const int c = plan.y;
+  if (c < 2 || c > kMaxChunks || plan.x < 0 ||
+      plan.x + static_cast<long long>(R) * p.Hkv * c > p.part_cap)
+    return;
+  const int row = blockIdx.x * kMergeRows + rl;
+  const bool mine = row < R;
+  const size_t base = static_cast<size_t>(plan.x) + static_cast<size_t>(g) * c * R + (mine ? row : 0);
+  // the first chunks' rows are on their way while the weights are formed
+  float v[kMergeLoads][kV];
+  auto load = [&](int z0) {
+#pragma unroll
+    for (int k = 0; k < kMergeLoads; ++k) {
+      const int z = z0 + k * W;
+      const float* po = p.part_o + (base + static_cast<size_t>(z < c ? z : 0) * R) * D + lane * kV;
+      if (kV == 4) {
+        const float4 x = z < c ? __ldcg(reinterpret_cast<const float4*>(po))
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[k][0] = x.x;
+        v[k][1] = x.y;
+        v[k][kV - 2] = x.z;
+        v[k][kV - 1] = x.w;
+      } else {
+        const float2 x = z < c ? __ldcg(reinterpret_cast<const float2*>(po)) : make_float2(0.f, 0.f);
+        v[k][0] = x.x;
+        v[k][1] = x.y;
+      }
+    }
+  };
+  load(w);
+  const float2 ml = lane < c ? __ldcg(p.part_ml + base + static_cast<size_t>(lane) * R)
+                             : make_float2(-INFINITY, 0.f);
+  float M = ml.x;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  const float wt = ml.x == -INFINITY ? 0.f : exp2f(ml.x - M);
+  float sum = wt * ml.y;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  float acc[kV];
+#pragma unroll
+  for (int j = 0; j < kV; ++j) acc[j] = 0.f;
+  for (int z0 = w; z0 < c; z0 += kMergeLoads * W) {   // uniform over the warp
+    if (z0 > w) load(z0);
+#pragma unroll
+    for (int k = 0; k < kMergeLoads; ++k) {
+      const float wz = __shfl_sync(0xffffffffu, wt, (z0 + k * W) & 31);   // 0 from c on
+#pragma unroll
+      for (int j = 0; j < kV; ++j) acc[j] = fmaf(z0 + k * W < c ? wz : 0.f, v[k][j], acc[j]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kV; ++j) s_acc[rl][w][lane * kV + j] = acc[j];
+  __syncthreads();
+  // two columns per lane and step, the row's W warps side by side
+  const float inv = sum > 0.f ? 1.f / sum : 0.f;
+  const int i = row / p.G;
+  if (!mine) return;
+  __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.out) +
+                       (static_cast<size_t>(s0 + i) * p.Hq + g * p.G + (row - i * p.G)) * D;
+  for (int col = w * 64 + 2 * lane; col < D; col += 64 * W) {
+    float x = 0.f, y = 0.f;
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      x += s_acc[rl][k][col];
+      y += s_acc[rl][k][col + 1];
+    }
+    *reinterpret_cast<__nv_bfloat162*>(out + col) = __floats2bfloat162_rn(x * inv, y * inv);
+  }
 }
 
 // ----------------------------------------------------------------------------
@@ -753,6 +1019,9 @@ __device__ __forceinline__ bool make_item_pp(const AttnParams& p, Item& it, int*
   if (it.n <= 0 || it.n > kMaxNodes || it.s0 < 0 || it.s0 + it.n > p.T || it.r0 >= it.R)
     return false;
   it.nrows = min(kPPRows, it.R - it.r0);
+  it.key_base = 0;
+  it.chunks = 1;
+  it.chunk = it.part0 = 0;
   it.ctx = min(max(p.ctx_len[it.b], 0), p.ctx_max);
   it.nctx = (it.ctx + kKeys - 1) / kKeys;
   it.ntree = (it.n + kKeys - 1) / kKeys;
@@ -1198,11 +1467,40 @@ cudaError_t launch_attention_tc(const AttnParams& p, const CUtensorMap& tm_k,
     if (err != cudaSuccess) return err;
     return launch_pdl(k, grid, dim3(kThreads), smem, s, tm_k, tm_v, tm_tk, tm_tv, tm_q, p);
   }
-  const dim3 grid((p.max_nodes * p.G + kRows - 1) / kRows, p.B * p.Hkv, 1);
+  // row blocks: at most max_nodes * G rows of each of B sequences, and T * G
+  // rows of which every sequence may leave one block ragged; index order
+  // (B > kOrderMax) numbers the first form
+  const long long full = static_cast<long long>((p.max_nodes * p.G + kRows - 1) / kRows) * p.B;
+  const long long blocks =
+      p.B > kOrderMax ? full : std::min(full, static_cast<long long>(p.T) * p.G / kRows + p.B);
+  const long long ctas =
+      std::max<long long>(blocks * p.Hkv, p.part_cap > 0 ? p.nsm : 0);
+  if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
   auto* k = p.D == 64 ? attn_tc_kernel<64> : attn_tc_kernel<128>;
   err = set_smem_attrs(k, smem);
   if (err != cudaSuccess) return err;
-  return launch_pdl(k, grid, dim3(kThreads), smem, s, tm_k, tm_v, tm_tk, tm_tv, tm_q, p);
+  err = launch_pdl(k, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), smem, s, tm_k, tm_v, tm_tk,
+                   tm_tv, tm_q, p);
+  if (err != cudaSuccess || p.part_cap == 0) return err;
+  const bool few = static_cast<long long>(p.T) * p.Hq <= kMergeFewRows;
+  const int mrows = kMergeThreads / 32 / (few ? 4 : 1);
+  const dim3 mgrid((p.max_nodes * p.G + mrows - 1) / mrows, p.B * p.Hkv);
+  auto* merge = p.D == 64 ? (few ? attn_merge_kernel<64, 4> : attn_merge_kernel<64, 1>)
+                          : (few ? attn_merge_kernel<128, 4> : attn_merge_kernel<128, 1>);
+  return launch_pdl(merge, mgrid, dim3(kMergeThreads), 0, s, p);
+}
+
+long long attention_split_rows(const asd_dims& d, int total_nodes, int nsm) {
+  // worth its plan and merge kernel only while the unsplit items leave a
+  // quarter of the SMs idle; the device decides from the context lengths.
+  // (Allowed for 128 items on 152 SMs, which an even batch cannot split, the
+  // step of 8 sequences at context 16384 took 584 us instead of 580; for 256
+  // items, 32 ragged sequences took 128.5 us instead of 121.)
+  const long long G = d.num_q_heads / d.num_kv_heads;
+  const long long blocks = std::max<long long>(d.batch, total_nodes * G / kRows);
+  if (d.batch > kOrderMax || 4 * d.num_kv_heads * blocks > 3LL * nsm || d.ctx_max < 2 * kKeys)
+    return 0;
+  return static_cast<long long>(nsm) * std::min<long long>(kRows, d.max_nodes * G);
 }
 
 }  // namespace asd

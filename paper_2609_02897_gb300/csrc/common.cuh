@@ -39,7 +39,9 @@ struct WsLayout {
   size_t child_tok;    // int32[T]: children tokens, grouped by parent, sorted by (token, id)
   size_t child_id;     // int32[T]: global node id of each slot
   size_t lm_part;      // LmPartial[T][g_lm]
-  size_t total;
+  size_t total;        // everything above: what every call needs
+  size_t at_part;      // attention partials: plan int2[B], then (max, sum) and output rows
+  size_t full;         // total and the attention partials (asd_workspace_bytes)
   int g_lm;            // CTAs of the LM-head kernel (vocabulary ranges)
   int n_splits;        // context splits of the attention kernel
   int split_len;       // keys per context split (multiple of 64)

@@ -76,6 +76,12 @@ struct AttnParams {
   int n_splits, split_len, n_parts, max_nodes;
   float scale_log2;         // log2(e) / sqrt(D)
   int q_tma;                // tensor-core kernels: the query tiles by TMA (tm_q)
+  // one-tile tensor-core kernel: partial results of sequences cut into chunks
+  int nsm;                  // SMs of the device
+  long long part_cap;       // rows that part_o / part_ml hold (0: no splitting)
+  float* part_o;            // [part_cap][D]: a chunk's unnormalised output row
+  float2* part_ml;          // [part_cap]: its reference max (log2 domain) and sum
+  int2* plan;               // [B]: first partial row and chunks of a sequence
 };
 // bf16 path: tensor-core (mma.sync) split-KV kernel fed by TMA; tm_k / tm_v are
 // 2D tensor maps over the context cache rows (box 64 columns x
@@ -86,9 +92,10 @@ cudaError_t launch_attention_bf16(const AttnParams& p, const CUtensorMap& tm_k,
 cudaError_t launch_attention_f32(const AttnParams& p, cudaStream_t s);
 int attention_row_blocks(int max_nodes, int G);
 int attention_keys_per_tile();   // context keys per K/V tile = TMA box rows
-// bf16 path on the 5th-generation tensor cores, for steps where attention has
-// the SMs to itself (more than 128 tree nodes): one CTA per (128 query rows,
-// sequence x KV head), the whole context, no splits (p.n_parts == 1).  tm_k /
+// bf16 path on the 5th-generation tensor cores, where attention has the SMs to
+// itself (a standalone call, or a step of more than 128 tree nodes): one CTA
+// per (128 query rows, sequence x KV head, chunk of the keys), and a merge
+// kernel behind it where chunks are possible (p.part_cap > 0).  tm_k /
 // tm_v: 2D maps over the cache rows with boxes of 64 columns x
 // min(kAttnTcKeys, rows per page) rows; tm_tk / tm_tv: 3D maps over the tree
 // K/V [T, Hkv, D] with boxes of 64 columns x 1 head x kAttnTcKeys nodes;
@@ -101,6 +108,9 @@ constexpr int kAttnTcRows = 128;   // query rows per CTA (per tile of the ping-p
 constexpr int kAttnTcKeys = 128;   // keys per tile
 size_t attention_tc_smem_bytes(int head_dim, bool pingpong);
 bool attention_pingpong(int batch, int num_kv_heads, int G, int total_nodes, int nsm);
+// Partial rows that the one-tile kernel can use to cut sequences into chunks
+// (0: the items of these dims and nodes fill the GPU anyway).
+long long attention_split_rows(const asd_dims& d, int total_nodes, int nsm);
 bool attention_q_tma_ok(int G);   // G divides kAttnTcRows: a query box of whole nodes
 cudaError_t launch_attention_tc(const AttnParams& p, const CUtensorMap& tm_k,
                                 const CUtensorMap& tm_v, const CUtensorMap& tm_tk,

@@ -89,3 +89,60 @@ def test_late_v_ring_does_not_disturb_a_ragged_tail(D, page):
     _check_close(outs[0], _reference(d, B, n, ctx, page, Hq, Hkv, D))
     for o in outs[1:]:
         assert torch.equal(o.view(torch.int16), outs[0].view(torch.int16))
+
+
+# (B, nodes, contexts, page, Hq, Hkv, D, cache slots): chunk and tile edges, a
+# cache much larger than the contexts, ragged batches in which only the long
+# sequences are cut, more than 128 nodes, query groups that do not divide 128
+SPLITS = [
+    (1, 1, [0], 0, 32, 8, 128, 4096),
+    (1, 8, [127], 0, 32, 8, 128, 40960),
+    (1, 8, [128], 16, 32, 8, 128, 4096),
+    (1, 8, [129], 0, 32, 8, 64, 4096),
+    (1, 5, [4095], 0, 32, 8, 128, 32768),
+    (1, 60, [2049], 0, 32, 8, 128, 2112),
+    (1, 128, [9000], 64, 16, 8, 128, 16384),
+    (3, 7, [0, 257, 6001], 16, 28, 4, 128, 8192),
+    (4, 33, [511, 4000, 130, 2600], 256, 32, 8, 128, 8192),
+    (2, 100, [3000, 700], 0, 64, 8, 64, 4096),
+    (19, 6, [100 * (b + 1) + b for b in range(19)], 8, 8, 1, 128, 2048),
+]
+
+
+@pytest.mark.parametrize("case", range(len(SPLITS)))
+@pytest.mark.parametrize("small_workspace", [False, True])
+def test_split_contexts(case, small_workspace):
+    """Contexts cut into chunks and merged, and the same call with a workspace
+    that ends before (most of) the partial rows, which splits less."""
+    import torch
+    from paper_2609_02897_gb300 import asd
+    B, n, ctx, page, Hq, Hkv, D, cap = SPLITS[case]
+    d = _inputs(B, n, ctx, page, Hq, Hkv, D, cap, case)
+    # one vocabulary range: the workspace before the partial rows is small
+    dims = asd.make_dims(B, Hq, Hkv, D, 64, 32, asd.ASD_BF16, page, cap,
+                         B * cap // page if page else 0, n, n)
+    ws = asd.alloc_workspace(dims, B * n)
+    if small_workspace:
+        ws = ws[:min(ws.numel(), 32768)]
+    out = _call(d, dims, ws)
+    again = _call(d, dims, ws)
+    assert asd.asd_get_device_status(ws) == 0
+    _check_close(out, _reference(d, B, n, ctx, page, Hq, Hkv, D))
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+
+
+def test_split_batch_with_a_malformed_sequence():
+    """A malformed sequence in a batch that splits gets no work and is
+    reported; the others' outputs are those of the batch without the fault, up
+    to the rounding of another cut (the chunk length follows the whole batch)."""
+    from paper_2609_02897_gb300 import asd
+    B, n, Hq, Hkv, D, cap = 3, 8, 32, 8, 128, 8192
+    d = _inputs(B, n, [5000, 3000, 7000], 0, Hq, Hkv, D, cap, 1)
+    dims = asd.make_dims(B, Hq, Hkv, D, 64, 32, asd.ASD_BF16, 0, cap, 0, n, n)
+    ws = asd.alloc_workspace(dims, B * n)
+    good = _call(d, dims, ws)
+    assert asd.asd_get_device_status(ws) == 0
+    d["cu_nodes"][2] = d["cu_nodes"][1]          # sequence 1 empty, 2 too long
+    out = _call(d, dims, ws)
+    assert asd.asd_get_device_status(ws) == 3
+    _check_close(out[:n], good[:n].float())
