@@ -143,8 +143,8 @@ def lmhead_bytes(wl, rows=None, passes=1):
 
 
 def lazy_work(wl, row_max):
-    """Rows the lazy schedule computed (row_max not NaN) and the tree levels they
-    span (one W pass each)."""
+    """Rows the lazy schedule reached (row_max not NaN) and the tree levels they
+    span (a W pass settles one level or more)."""
     reach = ~np.isnan(row_max)
     depth = np.zeros(wl.T, np.int64)
     for b in range(wl.B):
@@ -785,14 +785,16 @@ def run_asd(args):
     tpk, tpk_kind = tensor_peak()
     lm_rows, lm_passes = wl.T, 1
     if lazy:
-        lm_rows, lm_passes = lazy_work(wl, out["row_max"])
+        # rows reached; the passes that settled their levels are not reported,
+        # so the floor counts one stream of W
+        lm_rows, lm_levels = lazy_work(wl, out["row_max"])
     lmb = lmhead_bytes(wl, lm_rows, lm_passes)
     sb = step_bytes(wl, mean_path, lmb)
     fl = step_flops(wl, lm_rows)
     t_bytes, t_flops = sb / (peak * 1e9), fl / (tpk * 1e12)
     lm_kernel = lm_kernel_name(step)
     if lazy:
-        lm_kernel = (f"lmhead_wide_kernel + lazy_level_kernel, {lm_passes} non-empty levels of "
+        lm_kernel = (f"lmhead_wide_kernel + lazy_pass_kernel, {lm_levels} levels of "
                      f"{wl.max_path} (LM-head stage total)")
     traffic = lmhead_traffic(CONFIG) if packed and not lazy else None
     line = {
@@ -804,7 +806,7 @@ def run_asd(args):
         "config": workload_config(wl),
         "lm_head_weight": ("packed once at load by asd_pack_lm_head (same bytes, streaming order)"
                            if packed else "[vocab, hidden] rows"),
-        "lm_head_schedule": (f"lazy levels: {lm_rows} of {wl.T} rows computed, {lm_passes} W passes"
+        "lm_head_schedule": (f"lazy levels: {lm_rows} of {wl.T} rows reached, {lm_levels} levels"
                              if lazy else "every row"),
         "hbm_gbs": sb / (ms * 1e-3) / 1e9, "hbm_frac_of_" + peak_kind: sb / (ms * 1e-3) / 1e9 / peak,
         # the whole step against the binding resource: the time its bytes take at

@@ -101,18 +101,20 @@ typedef enum asd_lm_layout {
  *   ASD_LM_EVERY_ROW    every node's row (default).
  *   ASD_LM_LAZY_LEVELS  only the rows the accepted-path walk can read: the
  *       roots and the nodes whose every ancestor (root excluded) was
- *       accepted, computed one tree level per pass over W (max_path passes,
- *       the later ones empty when the accepted region ends).  A verdict needs
+ *       accepted, computed in passes over W that settle one tree level or
+ *       more each (at most max_path passes; a pass of fewer than 256 rows is
+ *       filled up with rows of nodes below, which are dropped if their
+ *       ancestors turn out rejected).  A verdict needs
  *       the parent's row (Eq. 1), so this is what a walk from the root can
  *       reach; the committed path, bonus token, n_promoted and the cache are
  *       those of ASD_LM_EVERY_ROW, and every computed row and verdict is
  *       bit-identical to it.  Nodes not reached keep row_max = row_lse = NaN,
  *       row_argmax = -1, ratio = l_draft = NaN and accept = 0.  Pays when the
- *       levels cost fewer weight passes than the full tree costs in flops
+ *       passes cost less than the full tree's rows
  *       (many sequences, few accepted nodes).  bf16 only; every tree must be
  *       shallower than max_path (a reached node at depth max_path records
  *       ASD_ERR_SHAPE).  The workspace grows by 2 x (T rounded up to 128) x
- *       hidden x 2 bytes for the levels' hidden rows.  Not available in
+ *       hidden x 2 bytes for the passes' hidden rows.  Not available in
  *       asd_lmhead_margin_noalloc (ASD_ERR_SHAPE). */
 typedef enum asd_lm_schedule {
   ASD_LM_EVERY_ROW = 0,
@@ -306,7 +308,7 @@ int32_t asd_abi_version(void);
  * Which LM-head kernel a call with these dims, node count and weight pointer
  * runs (a diagnostic query; no counterpart in the paper; nothing is
  * launched): 1 the weight-streaming tensor-core kernel (up to 128 nodes),
- * 2 the wide kernel (more nodes, or a level of the lazy schedule), 3 the wide
+ * 2 the wide kernel (more nodes, or a pass of the lazy schedule), 3 the wide
  * kernel in clusters of two SMs that multicast W between them (two pairs of
  * 128-node tiles, or four and more, and an even range count), 4 the fp32 kernel,
  * 0 for invalid arguments.  The clustered form multicasts from the calling

@@ -168,7 +168,8 @@ WsLayout layout(const asd_dims& d, int T, int nsm) {
   L.lm_part = off;     off = align256(off + sizeof(LmPartial) * static_cast<size_t>(T) * L.g_lm);
   if (d.lm_head_schedule == ASD_LM_LAZY_LEVELS) {
     L.lz_cap = (T + 127) / 128 * 128;
-    L.lz_count = off;  off = align256(off + 4 * (static_cast<size_t>(d.max_path) + 1));
+    L.lz_count = off;  off = align256(off + 8 * (static_cast<size_t>(d.max_path) + 1));
+    L.lz_seq = off;    off = align256(off + sizeof(int2) * static_cast<size_t>(d.batch));
     L.lz_rows = off;   off = align256(off + 4 * 2 * static_cast<size_t>(T));
     L.lz_h = off;      off = align256(off + 2 * 2 * static_cast<size_t>(L.lz_cap) * d.hidden);
   }
@@ -413,10 +414,11 @@ asd_status run_lmhead(const Ctx& c, const void* hidden, const void* w, float* l_
 
 float ln_tau(float tau);
 
-// The lazy schedule (asd_lm_schedule): level 0 holds the roots; each level's
-// rows go through the wide LM head, then the level kernel merges them,
-// judges their children and lists the accepted ones for the next level.
-// Writes every output of the finalize stage for the rows it computes.
+// The lazy schedule (asd_lm_schedule): each pass's rows go through the wide LM
+// head, then the pass kernel merges them, judges their children and lists the
+// next pass.  max_path passes are enqueued, since a pass settles at least one
+// tree level; the ones after the last find no rows and return.  Writes every
+// output of the finalize stage for the rows that are reached.
 asd_status run_lmhead_lazy(const Ctx& c, const void* hidden, const void* w,
                            const int32_t* parent, const int32_t* tokens,
                            const int32_t* cu_nodes, float tau, float* row_max,
@@ -459,9 +461,6 @@ asd_status run_lmhead_lazy(const Ctx& c, const void* hidden, const void* w,
   z.tokens = tokens;
   z.cu_nodes = cu_nodes;
   z.seq_flags = ws_at<int>(c.ws, c.L.seq_flags);
-  z.child_start = p.child_start;
-  z.child_cnt = p.child_cnt;
-  z.child_id = p.child_id;
   z.hidden = hidden;
   z.part = p.part;
   z.row_max = row_max;
@@ -471,27 +470,29 @@ asd_status run_lmhead_lazy(const Ctx& c, const void* hidden, const void* w,
   z.ratio = ratio;
   z.accept = accept;
   z.count = count;
+  z.active = count + levels + 1;
+  z.seq_rows = ws_at<int2>(c.ws, c.L.lz_seq);
   z.status = p.status;
   z.B = d.batch;
   z.T = c.T;
   z.K = d.hidden;
   z.g_lm = c.L.g_lm;
-  z.last_level = levels - 1;
+  z.levels = levels;
   z.ln_tau = ln_tau(tau);
+  z.pass = -1;
   z.rows_next = rows[0];
   z.h_next = h[0];
-  if (launch_lazy_init(z, levels, c.st) != cudaSuccess) return ASD_ERR_CUDA;
-  const int nsm = device_sm_count();
-  for (int lv = 0; lv < levels; ++lv) {
-    p.hidden = h[lv & 1];
-    p.t_dev = count + lv;
-    p.row_node = rows[lv & 1];
-    if (launch_lmhead_bf16(p, maps[lv & 1], c.st) != cudaSuccess) return ASD_ERR_CUDA;
-    z.level = lv;
-    z.rows_cur = rows[lv & 1];
-    z.rows_next = rows[(lv + 1) & 1];
-    z.h_next = h[(lv + 1) & 1];
-    if (launch_lazy_level(z, nsm, c.st) != cudaSuccess) return ASD_ERR_CUDA;
+  if (launch_lazy_init(z, c.st) != cudaSuccess) return ASD_ERR_CUDA;
+  for (int k = 0; k < levels; ++k) {
+    p.hidden = h[k & 1];
+    p.t_dev = count + k;
+    p.row_node = rows[k & 1];
+    if (launch_lmhead_bf16(p, maps[k & 1], c.st) != cudaSuccess) return ASD_ERR_CUDA;
+    z.pass = k;
+    z.rows_cur = rows[k & 1];
+    z.rows_next = rows[(k + 1) & 1];
+    z.h_next = h[(k + 1) & 1];
+    if (launch_lazy_pass(z, c.st) != cudaSuccess) return ASD_ERR_CUDA;
   }
   return ASD_OK;
 }
@@ -550,7 +551,7 @@ int32_t asd_lm_head_variant(const asd_dims* dims, int32_t total_nodes, const voi
   p.g_lm = lm_ranges(dims->vocab, nsm);
   p.w_local = on_this_device(w_lm) ? 1 : 0;
   p.t_dev = nullptr;
-  if (dims->lm_head_schedule == ASD_LM_LAZY_LEVELS) return 2;   // one level per launch
+  if (dims->lm_head_schedule == ASD_LM_LAZY_LEVELS) return 2;   // a pass per launch
   return lmhead_bf16_variant(p);
 }
 

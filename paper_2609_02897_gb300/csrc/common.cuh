@@ -47,8 +47,9 @@ struct WsLayout {
   int split_len;       // keys per context split (multiple of 64)
   int n_parts;         // = n_splits (the tree keys ride with the last split)
   // lazy LM-head schedule only (0 otherwise)
-  size_t lz_count;     // int32[max_path + 1]: rows per level
-  size_t lz_rows;      // int32[2][T]: node ids of a level's rows (two levels in flight)
+  size_t lz_count;     // int32[2][max_path + 1]: rows, then active sequences per pass
+  size_t lz_seq;       // int2[B]: a sequence's first row and rows in the pass
+  size_t lz_rows;      // int32[2][T]: node ids of a pass's rows (two passes in flight)
   size_t lz_h;         // bf16[2][lz_cap][hidden]: their hidden rows
   int lz_cap;          // T rounded up to 128
   int attn_tc;         // tensor-core attention (attention has the SMs to itself): 1 one

@@ -446,12 +446,13 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   const long long budget = wait_budget(p.status);
   const int rank = CL == 2 ? static_cast<int>(cta_rank_in_cluster()) : 0;
   const uint16_t both = static_cast<uint16_t>((1u << CL) - 1u);
-  // hidden rows of this launch: T, or (one level of the lazy schedule) the
+  // hidden rows of this launch: T, or (one pass of the lazy schedule) the
   // count and the rows that the previous kernel wrote
   int nrow = p.T;
   if (p.t_dev) {
     pdl_wait();
     nrow = min(max(*p.t_dev, 0), p.T);
+    if (nrow == 0) return;   // no rows left (uniform over the grid; CL = 1)
   }
 
   const int ngroups = (p.V + kLmBoxRows - 1) / kLmBoxRows;

@@ -76,6 +76,24 @@ def test_lazy_many_rows_per_level(dev, B):
     print(wl.name, B, rep)
 
 
+@pytest.mark.parametrize("B,nodes", [(2, 128), (40, 23), (255, 5), (256, 4), (300, 6)])
+@pytest.mark.parametrize("tau", [1.0, 0.1])
+def test_lazy_rows_ahead(dev, B, nodes, tau):
+    """The rows that a pass computes ahead of their verdicts: everything (few
+    sequences), a few per sequence, one sequence's root each (B = 256 fills the
+    256 rows of a pass) and none; whatever was computed ahead and not reached
+    leaves the fills."""
+    from paper_2609_02897_gb300 import synth
+    rng = np.random.default_rng(B)
+    trees = [synth.random_topological_relabel(synth.tree_grown(rng, nodes, 4 + b % 5, 1 + b % 6), rng)
+             for b in range(7)]
+    wl = H.prepared(3, small=True, rep=B, tree_override=trees, overrides=dict(B=B))
+    eager, s0, _, _ = dev.run_verify(wl, tau)
+    lazy, s1, _, _ = dev.run_verify(wl, tau, schedule=1)
+    assert s0 == 0 and s1 == 0
+    _check(wl, eager, lazy)
+
+
 def test_lazy_lmhead_margin_call(dev):
     """asd_lmhead_margin under the lazy schedule writes what the verify step
     writes."""
@@ -102,7 +120,7 @@ def test_lazy_lmhead_margin_call(dev):
 
 
 def test_lazy_step_in_a_cuda_graph(dev):
-    """The lazy schedule (a memset and two kernels per level) captured once
+    """The lazy schedule (a memset and two kernels per pass) captured once
     and replayed gives the eager-launch results."""
     import torch
     from paper_2609_02897_gb300 import asd
