@@ -209,7 +209,15 @@ struct Ctx {
   cudaStream_t st;
   void* ws;
   size_t ws_bytes;
+  long long wait_cycles;
 };
+
+// Clears the status word of a call whose first kernel does not.
+asd_status clear_status(const Ctx& c) {
+  return cudaMemsetAsync(ws_at<int>(c.ws, c.L.status), 0, 2 * sizeof(int), c.st) == cudaSuccess
+             ? ASD_OK
+             : ASD_ERR_CUDA;
+}
 
 // Wait budget (SM clock cycles) that asd_debug_set_wait_cycles set for the
 // kernels of later calls; 0: the kernels' default.
@@ -231,14 +239,7 @@ asd_status begin_call(const asd_dims* dims, int32_t total_nodes, void* ws, size_
   c->st = static_cast<cudaStream_t>(stream);
   c->ws = ws;
   c->ws_bytes = ws_bytes;
-  if (cudaMemsetAsync(ws_at<int>(ws, c->L.status), 0, 16, c->st) != cudaSuccess)
-    return ASD_ERR_CUDA;
-  // a test's shorter wait budget rides in words 2-3 of the status block
-  static thread_local long long budget;
-  budget = g_wait_cycles.load();
-  if (budget != 0 && cudaMemcpyAsync(ws_at<int>(ws, c->L.status) + 2, &budget, sizeof(budget),
-                                     cudaMemcpyHostToDevice, c->st) != cudaSuccess)
-    return ASD_ERR_CUDA;
+  c->wait_cycles = g_wait_cycles.load();
   return ASD_OK;
 }
 
@@ -280,6 +281,7 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
   a.page_table = page_table;
   a.parent = parent;
   a.status = ws_at<int>(c.ws, c.L.status);
+  a.wait_cycles = c.wait_cycles;
   a.out = out;
   a.B = d.batch;
   a.T = c.T;
@@ -389,6 +391,7 @@ asd_status run_lmhead(const Ctx& c, const void* hidden, const void* w, float* l_
   p.part = ws_at<LmPartial>(c.ws, c.L.lm_part);
   p.l_draft = l_draft;
   p.status = ws_at<int>(c.ws, c.L.status);
+  p.wait_cycles = c.wait_cycles;
   p.T = c.T;
   p.K = d.hidden;
   p.V = d.vocab;
@@ -441,6 +444,7 @@ asd_status run_lmhead_lazy(const Ctx& c, const void* hidden, const void* w,
   p.part = ws_at<LmPartial>(c.ws, c.L.lm_part);
   p.l_draft = l_draft;
   p.status = ws_at<int>(c.ws, c.L.status);
+  p.wait_cycles = c.wait_cycles;
   p.T = c.T;
   p.K = d.hidden;
   p.V = d.vocab;
@@ -679,6 +683,8 @@ asd_status asd_accept_path(const asd_dims* dims, const int32_t* parent, const in
   Ctx c;
   asd_status st = begin_call(dims, total_nodes, workspace, workspace_bytes, stream, &c);
   if (st != ASD_OK) return st;
+  st = clear_status(c);
+  if (st != ASD_OK) return st;
   TailParams t = tail_params(c, kTailWalk);
   t.ratio = const_cast<float*>(ratio);
   t.parent = parent;
@@ -707,6 +713,8 @@ asd_status asd_kv_compact(const asd_dims* dims, const void* tree_k, const void* 
     return ASD_ERR_INVALID_ARG;
   Ctx c;
   asd_status st = begin_call(dims, total_nodes, workspace, workspace_bytes, stream, &c);
+  if (st != ASD_OK) return st;
+  st = clear_status(c);
   if (st != ASD_OK) return st;
   TailParams t = tail_params(c, kTailCompact);
   t.parent = nullptr;  // path entries are checked against the tree sizes only
@@ -891,9 +899,7 @@ extern "C" asd_status asd_lmhead_margin_noalloc(
   c.ws = noalloc_scratch();
   if (!c.ws) return ASD_ERR_CUDA;
   c.st = static_cast<cudaStream_t>(stream);
-  // the status word must start at zero; every other region is written before it is read
-  if (cudaMemsetAsync(ws_at<int>(c.ws, c.L.status), 0, 16, c.st) != cudaSuccess)
-    return ASD_ERR_CUDA;
+  c.wait_cycles = 0;
   if (launch_tree_prep(prep_params(c, parent, tokens, cu_nodes, nullptr, l_draft), c.st) !=
       cudaSuccess)
     return ASD_ERR_CUDA;

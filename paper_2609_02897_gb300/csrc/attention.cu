@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(128) attn_bf16_kernel(const __grid_constant__ 
   __shared__ uint64_t s_anc[kMaxNodes][2];
 
   pdl_launch_dependents();  // nothing downstream reads this kernel's output early
-  const long long budget = wait_budget(p.status);
+  const long long budget = wait_budget(p.wait_cycles);
 
   // This kernel does not depend on the tree preparation: it derives the
   // ancestor masks itself and keeps every access inside the caller's arrays

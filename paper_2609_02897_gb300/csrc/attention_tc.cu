@@ -660,7 +660,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long budget = wait_budget(p.status);
+  const long long budget = wait_budget(p.wait_cycles);
 
   uint32_t base = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (base & 1023u)) & 1023u;
@@ -1053,7 +1053,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long budget = wait_budget(p.status);
+  const long long budget = wait_budget(p.wait_cycles);
   __shared__ int s_work[kOrderMax];
   __shared__ int s_seq;
   Item it;

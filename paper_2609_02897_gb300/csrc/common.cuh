@@ -31,8 +31,7 @@ struct LmPartial {
 
 // Offsets (bytes) of the workspace regions; every region is 256-byte aligned.
 struct WsLayout {
-  size_t status;       // int32[4]: [0] first device error code; [1] a bounded wait gave
-                       // up; [2..3] int64 wait budget (0: the default), set for testing
+  size_t status;       // int32[2]: [0] first device error code; [1] a bounded wait gave up
   size_t seq_flags;    // int32[B]
   size_t child_start;  // int32[T]: global slot of the node's first child
   size_t child_cnt;    // int32[T]
@@ -59,7 +58,20 @@ struct WsLayout {
 
 // ---------------------------------------------------------------- device utils
 
+// Programmatic dependent launch: a kernel launched with programmatic stream
+// serialisation may start while its predecessor in the stream still runs;
+// pdl_wait() blocks until every predecessor grid has completed and its memory
+// is visible, pdl_launch_dependents() lets the next kernel start launching.
+// Both are no-ops for kernels launched without the attribute.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// The first error of a call, in its status word.  The call's first kernel
+// clears the word, so a later kernel that started early waits for it here.
 __device__ __forceinline__ void set_status(int* status, int code) {
+  pdl_wait();
   atomicCAS(status, 0, code);
 }
 
@@ -89,16 +101,6 @@ __device__ __forceinline__ void merge_part(float& m, float& s, int& a, float m2,
   if (m2 > m) a = a2;
   else if (m2 == m) a = min(a, a2);
   m = M;
-}
-
-// Programmatic dependent launch: a kernel launched with programmatic stream
-// serialisation may start while its predecessor in the stream still runs;
-// pdl_wait() blocks until every predecessor grid has completed and its memory
-// is visible, pdl_launch_dependents() lets the next kernel start launching.
-// Both are no-ops for kernels launched without the attribute.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_dependents() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -174,13 +176,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
   }
 }
 
-// The wait budget of the kernels of one call: words 2-3 of the workspace
-// status block hold it when the host set a shorter one for testing
-// (asd_debug_set_wait_cycles), zero otherwise.  Waits for copies and MMAs
-// already in flight always use the full kWaitCycles.
-__device__ __forceinline__ long long wait_budget(const int* status) {
-  const long long b = *reinterpret_cast<const volatile long long*>(status + 2);
-  return b > 0 ? b : kWaitCycles;
+// The wait budget of a call: the host's, where a test set a shorter one
+// (asd_debug_set_wait_cycles).  Waits for copies and MMAs already in flight
+// always use the full kWaitCycles.
+__device__ __forceinline__ long long wait_budget(long long set) {
+  return set > 0 ? set : kWaitCycles;
 }
 
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {

@@ -55,8 +55,10 @@ struct PrepParams {
   int32_t* child_id;
   float* l_draft;           // may be null; set to NaN
   int B, T, vocab, max_nodes, ctx_max;
+  int clear_status;         // set by launch_tree_prep: the kernel clears the status word
 };
-cudaError_t launch_tree_prep(const PrepParams& p, cudaStream_t s);
+// Also clears the status word (the call's first launch).
+cudaError_t launch_tree_prep(PrepParams p, cudaStream_t s);
 
 // ------------------------------------------------------------------ attention
 struct AttnParams {
@@ -70,6 +72,7 @@ struct AttnParams {
   const int32_t* page_table;  // [B, ctx_max / ps] or null
   const int32_t* parent;      // local parent ids (ancestor masks are derived in-kernel)
   int* status;
+  long long wait_cycles;    // bound of the kernel's waits (0: the default)
   void* out;                // [T, Hq, D]
   int B, T, Hq, Hkv, G, D;
   int ctx_max, page_size, pages_per_seq, num_pages;
@@ -128,6 +131,7 @@ struct LmParams {
   LmPartial* part;          // [T][g_lm]
   float* l_draft;           // [T]
   int* status;
+  long long wait_cycles;    // bound of the kernel's waits (0: the default)
   int T, K, V, g_lm;
   int a_rows;               // node rows per hidden-state TMA box: min(128, T rounded to 8);
                             // accumulator rows past it belong to no node

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(192, 1)
   // kernels: only the epilogue (children lists, l_draft) waits for them
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long budget = wait_budget(p.status);
+  const long long budget = wait_budget(p.wait_cycles);
 
   // this CTA's vocabulary range, in whole groups of kLmBoxRows rows
   const int ngroups = (p.V + kLmBoxRows - 1) / kLmBoxRows;
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
 
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long budget = wait_budget(p.status);
+  const long long budget = wait_budget(p.wait_cycles);
   const int rank = CL == 2 ? static_cast<int>(cta_rank_in_cluster()) : 0;
   const uint16_t both = static_cast<uint16_t>((1u << CL) - 1u);
   // hidden rows of this launch: T, or (one pass of the lazy schedule) the

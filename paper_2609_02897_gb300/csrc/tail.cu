@@ -45,8 +45,10 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) 
   __shared__ int s_maxd, s_len, s_skip;
 
   // Until pdl_wait() this kernel reads only caller inputs (cu_nodes, parent,
-  // tokens): no kernel of the call writes them, and every call starts behind
-  // a stream-ordered memset, so they are final even before the wait.
+  // tokens): no kernel of the call writes them, and the call's first kernel
+  // waits for the stream's earlier work (a call of this kernel alone starts
+  // behind a memset), so they are final even before the wait.
+  pdl_launch_dependents();
   const int b = blockIdx.x;
   const int i = threadIdx.x;
   const int warp = i >> 5, lane = i & 31;
