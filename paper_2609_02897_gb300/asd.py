@@ -155,13 +155,14 @@ def _ptr(t: Optional[torch.Tensor]):
         raise ValueError("libasd takes device tensors")
     if not t.is_contiguous():
         raise ValueError("libasd takes contiguous tensors")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        # the raw handle of torch.cuda.current_stream(), without the Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _check(code: int, where: str):
