@@ -214,9 +214,8 @@ struct Ctx {
 
 // Clears the status word of a call whose first kernel does not.
 asd_status clear_status(const Ctx& c) {
-  return cudaMemsetAsync(ws_at<int>(c.ws, c.L.status), 0, 2 * sizeof(int), c.st) == cudaSuccess
-             ? ASD_OK
-             : ASD_ERR_CUDA;
+  return launch_clear_status(ws_at<int>(c.ws, c.L.status), c.st) == cudaSuccess ? ASD_OK
+                                                                                : ASD_ERR_CUDA;
 }
 
 // Wait budget (SM clock cycles) that asd_debug_set_wait_cycles set for the

@@ -59,6 +59,7 @@ struct PrepParams {
 };
 // Also clears the status word (the call's first launch).
 cudaError_t launch_tree_prep(PrepParams p, cudaStream_t s);
+cudaError_t launch_clear_status(int* status, cudaStream_t s);
 
 // ------------------------------------------------------------------ attention
 struct AttnParams {

@@ -46,8 +46,8 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) 
 
   // Until pdl_wait() this kernel reads only caller inputs (cu_nodes, parent,
   // tokens): no kernel of the call writes them, and the call's first kernel
-  // waits for the stream's earlier work (a call of this kernel alone starts
-  // behind a memset), so they are final even before the wait.
+  // waits for the stream's earlier work (in a call of this kernel alone,
+  // the one that clears the status word), so they are final even before the wait.
   pdl_launch_dependents();
   const int b = blockIdx.x;
   const int i = threadIdx.x;
