@@ -1,80 +1,225 @@
 // LM head fused with the margin-rule statistics (Eq. 1) for fp32 inputs:
 // exact fp32 FMA on the CUDA cores (the tensor cores have no fp32-exact mode).
-// Same decomposition as the tensor-core kernel: one CTA per vocabulary range,
-// one thread per node row, logits consumed in 32-wide chunks by the shared
-// per-row epilogue, one (max, argmax, sum-exp) partial per node and range.
+//
+// One CTA per (vocabulary range, tile of NT nodes); the ranges are those of the
+// tensor-core kernel.  A CTA walks its range in chunks of 64 vocabulary rows and
+// 64 hidden elements at a time, W and hidden rows through a ring of cp.async
+// stages, each thread accumulating a VP x NP block of logits from 16-byte
+// shared-memory reads along the hidden dimension.  The logits of a chunk meet in
+// shared memory, where a warp per node row folds them into the row's running
+// (max, lowest argmax, sum-exp) and picks the drafted tokens' logits of the
+// node's children.  One partial per node and range.
+//
+// Bound: W traffic up to some 25 nodes, FMA issue beyond; on small shapes the
+// latency of the loads, hence all stages in flight at once.  Whole fp32 step of
+// 8 nodes, hidden 256, vocabulary 4096, this kernel 34.4 -> 8.8 us (profiled): one
+// node per thread and 32 columns, loads between two barriers before.
+#include <type_traits>
+
 #include "kernels.h"
-#include "lm_epilogue.cuh"
 
 namespace asd {
 namespace {
 
-constexpr int kRows = 128;   // node rows per CTA pass (one per thread)
-constexpr int kKc = 32;      // hidden elements staged per step
+constexpr int kThreads = 256;
+constexpr int kVt = 64;          // vocabulary rows of a chunk
+constexpr int kKc = 64;          // hidden elements of a stage
+constexpr int kLd = kKc + 4;     // padded row: 8 rows' 16-byte reads touch all 32 banks
 
-__global__ void __launch_bounds__(kRows) lmhead_f32_kernel(const LmParams p) {
-  __shared__ float s_w[32][kKc + 1];
-  __shared__ float s_h[kRows][kKc + 1];
-  pdl_wait();
+template <int NT>
+struct Geom {
+  static constexpr int kTn = NT < 16 ? NT : 16;      // thread groups along the nodes
+  static constexpr int kTv = kThreads / kTn;         // and along the vocabulary
+  static constexpr int kVp = kVt / kTv;              // a thread's vocabulary rows
+  static constexpr int kNp = NT / kTn;               // and nodes
+  static constexpr int kStages = NT <= 16 ? 4 : 3;   // two CTAs per SM
+  static constexpr int kStageFloats = (kVt + NT) * kLd;
+  static constexpr size_t kBytes = sizeof(float) * kStages * kStageFloats;
+};
+
+// `bytes` (4 or 16) of global memory -> shared memory, zeros unless `in`.
+template <int bytes>
+__device__ __forceinline__ void copy_async(float* dst, const float* src, bool in) {
+  const int n = in ? bytes : 0;
+  if (bytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n)
+                 : "memory");
+}
+
+template <int NT>
+__global__ void __launch_bounds__(kThreads, 2) lmhead_f32_kernel(const LmParams p) {
+  using G = Geom<NT>;
+  extern __shared__ __align__(16) float smem[];
+  __shared__ float s_x[NT][kVt + 1];                 // logits of a chunk
+  __shared__ float s_m[NT], s_s[NT];                 // running statistics of a row
+  __shared__ int s_a[NT];
   pdl_launch_dependents();
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tn = tid / G::kTv, tv = tid % G::kTv;
   const float* hid = static_cast<const float*>(p.hidden);
   const float* w = static_cast<const float*>(p.w);
 
-  const int ngroups = (p.V + 31) / 32;
-  const int gs = static_cast<int>(static_cast<long long>(blockIdx.x) * ngroups / p.g_lm);
-  const int ge = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * ngroups / p.g_lm);
-  const int vs = gs * 32;
-  const int ve = min(p.V, ge * 32);
+  const int ngroups = (p.V + kLmBoxRows - 1) / kLmBoxRows;
+  const int tile = blockIdx.x / p.g_lm, range = blockIdx.x - tile * p.g_lm;
+  const int vs = lm_range_begin(range, p.g_lm, ngroups) * kLmBoxRows;
+  const int ve = min(p.V, lm_range_begin(range + 1, p.g_lm, ngroups) * kLmBoxRows);
+  const int node0 = tile * NT;
+  const int nk = (p.K + kKc - 1) / kKc;
+  const int total = (ve - vs + kVt - 1) / kVt * nk;
 
-  for (int nt = 0; nt * kRows < p.T; ++nt) {
-    const int node = nt * kRows + tid;
-    const bool active = node < p.T;
-    RowState st;
-    row_state_init(st, active, node, vs, p.child_start, p.child_cnt, p.child_tok, p.T);
-    for (int v0 = vs; v0 < ve; v0 += 32) {
-      const int nv = min(32, ve - v0);
-      float acc[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j] = 0.f;
-      for (int k0 = 0; k0 < p.K; k0 += kKc) {
-        for (int idx = tid; idx < 32 * kKc; idx += kRows) {
-          const int j = idx / kKc, kk = idx % kKc;
-          s_w[j][kk] = (j < nv && k0 + kk < p.K) ? w[static_cast<size_t>(v0 + j) * p.K + k0 + kk]
-                                                 : 0.f;
-        }
-        for (int idx = tid; idx < kRows * kKc; idx += kRows) {
-          const int r = idx / kKc, kk = idx % kKc;
-          const int nd = nt * kRows + r;
-          s_h[r][kk] = (nd < p.T && k0 + kk < p.K) ? hid[static_cast<size_t>(nd) * p.K + k0 + kk]
-                                                   : 0.f;
-        }
-        __syncthreads();
+  if (tid < NT) {
+    s_m[tid] = -INFINITY;
+    s_s[tid] = 0.f;
+    s_a[tid] = -1;
+  }
+
+  // stage `it`: 64 hidden elements of the chunk's W rows, then of the nodes' rows
+  auto load = [&](int it) {
+    float* st = smem + (it % G::kStages) * G::kStageFloats;
+    const int v0 = vs + it / nk * kVt, k0 = it % nk * kKc;
+    auto rows = [&](auto step) {   // 4 or 1 elements per copy
+      constexpr int kE = decltype(step)::value;
 #pragma unroll 4
-        for (int kk = 0; kk < kKc; ++kk) {
-          const float h = s_h[tid][kk];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) acc[j] = fmaf(h, s_w[j][kk], acc[j]);
-        }
-        __syncthreads();
+      for (int i = tid; i < (kVt + NT) * (kKc / kE); i += kThreads) {
+        const int r = i / (kKc / kE), k = k0 + i % (kKc / kE) * kE;
+        const bool is_w = r < kVt;
+        const int row = is_w ? v0 + r : node0 + r - kVt;
+        const bool in = k < p.K && row < (is_w ? ve : p.T);
+        const float* src = (is_w ? w : hid) + (in ? static_cast<size_t>(row) * p.K + k : 0);
+        copy_async<4 * kE>(st + r * kLd + (k - k0), src, in);
       }
-      if (active) row_chunk(st, acc, v0, nv, p.child_tok, p.child_id, p.l_draft, p.T);
+    };
+    if (p.K % 4 == 0)   // rows start 16-byte aligned
+      rows(std::integral_constant<int, 4>());
+    else
+      rows(std::integral_constant<int, 1>());
+  };
+
+#pragma unroll
+  for (int s = 0; s < G::kStages - 1; ++s) {
+    if (s < total) load(s);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  float acc[G::kVp][G::kNp];
+  bool waited = false;
+  for (int it = 0; it < total; ++it) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(G::kStages - 2) : "memory");
+    __syncthreads();   // stage `it` has landed, everyone is done with the one before
+    if (it + G::kStages - 1 < total) load(it + G::kStages - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (it % nk == 0) {
+#pragma unroll
+      for (int a = 0; a < G::kVp; ++a)
+#pragma unroll
+        for (int b = 0; b < G::kNp; ++b) acc[a][b] = 0.f;
     }
-    if (active) {
-      LmPartial part;
-      part.m = st.m;
-      part.s = st.s;
-      part.a = st.a;
-      part.pad = 0;
-      p.part[static_cast<size_t>(node) * p.g_lm + blockIdx.x] = part;
+    const float* st = smem + (it % G::kStages) * G::kStageFloats;
+    const float* sw = st + tv * kLd;
+    const float* sh = st + (kVt + tn) * kLd;
+#pragma unroll 4
+    for (int k = 0; k < kKc; k += 4) {
+      float4 x[G::kVp], y[G::kNp];
+#pragma unroll
+      for (int a = 0; a < G::kVp; ++a)
+        x[a] = *reinterpret_cast<const float4*>(sw + a * G::kTv * kLd + k);
+#pragma unroll
+      for (int b = 0; b < G::kNp; ++b)
+        y[b] = *reinterpret_cast<const float4*>(sh + b * G::kTn * kLd + k);
+#pragma unroll
+      for (int a = 0; a < G::kVp; ++a)
+#pragma unroll
+        for (int b = 0; b < G::kNp; ++b) {
+          acc[a][b] = fmaf(x[a].x, y[b].x, acc[a][b]);
+          acc[a][b] = fmaf(x[a].y, y[b].y, acc[a][b]);
+          acc[a][b] = fmaf(x[a].z, y[b].z, acc[a][b]);
+          acc[a][b] = fmaf(x[a].w, y[b].w, acc[a][b]);
+        }
+    }
+    if (it % nk != nk - 1) continue;
+
+    // the chunk's logits are complete
+    const int v0 = vs + it / nk * kVt, nv = min(kVt, ve - v0);
+#pragma unroll
+    for (int a = 0; a < G::kVp; ++a)
+#pragma unroll
+      for (int b = 0; b < G::kNp; ++b) s_x[tn + b * G::kTn][tv + a * G::kTv] = acc[a][b];
+    if (!waited) {   // the children lists come from the tree preparation
+      pdl_wait();
+      waited = true;
+    }
+    __syncthreads();
+    for (int r = warp; r < NT; r += kThreads / 32) {
+      const int node = node0 + r;
+      if (node >= p.T) break;
+      const float x0 = lane < nv ? s_x[r][lane] : -INFINITY;
+      const float x1 = lane + 32 < nv ? s_x[r][lane + 32] : -INFINITY;
+      float cm = fmaxf(x0, x1);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, o));
+      float m = s_m[r], sum = s_s[r];
+      __syncwarp();
+      if (cm > m) {   // uniform over the warp
+        const unsigned lo = __ballot_sync(0xffffffffu, x0 == cm);
+        const unsigned hi = __ballot_sync(0xffffffffu, x1 == cm);
+        if (lane == 0) s_a[r] = v0 + (lo ? __ffs(lo) - 1 : 31 + __ffs(hi));
+        sum *= exp2f((m - cm) * kLog2e);
+        m = cm;
+      }
+      const float nm = -m * kLog2e;
+      float e0, e1;
+      asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(fmaf(x0, kLog2e, nm)));
+      asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(fmaf(x1, kLog2e, nm)));
+      e0 += e1;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) e0 += __shfl_xor_sync(0xffffffffu, e0, o);
+      if (lane == 0) {
+        s_m[r] = m;
+        s_s[r] = sum + e0;
+      }
+      int cs = p.child_start[node], cnt = p.child_cnt[node];
+      if (cs < 0 || cnt < 0 || cnt > p.T || cs > p.T - cnt) cnt = 0;  // malformed tree: no children
+      for (int c = lane; c < cnt; c += 32) {
+        const int j = p.child_tok[cs + c] - v0;
+        const int cid = p.child_id[cs + c];
+        if (j >= 0 && j < nv && static_cast<unsigned>(cid) < static_cast<unsigned>(p.T))
+          p.l_draft[cid] = s_x[r][j];
+      }
     }
   }
+  pdl_wait();
+  __syncthreads();
+  if (tid < NT && node0 + tid < p.T) {
+    LmPartial part;
+    part.m = s_m[tid];
+    part.s = s_s[tid];
+    part.a = s_a[tid];
+    part.pad = 0;
+    p.part[static_cast<size_t>(node0 + tid) * p.g_lm + range] = part;
+  }
+}
+
+template <int NT>
+cudaError_t launch(const LmParams& p, cudaStream_t s) {
+  const cudaError_t err = cudaFuncSetAttribute(lmhead_f32_kernel<NT>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               static_cast<int>(Geom<NT>::kBytes));
+  if (err != cudaSuccess) return err;
+  return launch_pdl(lmhead_f32_kernel<NT>, dim3(p.g_lm * ((p.T + NT - 1) / NT)), dim3(kThreads),
+                    Geom<NT>::kBytes, s, p);
 }
 
 }  // namespace
 
 cudaError_t launch_lmhead_f32(const LmParams& p, cudaStream_t s) {
-  return launch_pdl(lmhead_f32_kernel, dim3(p.g_lm), dim3(kRows), 0, s, p);
+  // the smallest tile that holds the nodes, up to 64: wider tiles read W less
+  // often and feed more FMAs per shared-memory read
+  if (p.T <= 8) return launch<8>(p, s);
+  if (p.T <= 16) return launch<16>(p, s);
+  if (p.T <= 32) return launch<32>(p, s);
+  return launch<64>(p, s);
 }
 
 }  // namespace asd
