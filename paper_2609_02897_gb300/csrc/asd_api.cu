@@ -139,25 +139,16 @@ WsLayout layout(const asd_dims& d, int T, int nsm) {
   L.g_lm = lm_ranges(d.vocab, nsm);
   // context splits: at most one attention CTA per SM (in a verify step each
   // shares its SM with an LM-head CTA), at most kMaxAttnParts (the splits of a
-  // row block form one thread-block cluster); the last non-empty split of a
-  // sequence also takes its tree keys
+  // row block form one thread-block cluster); each sequence is cut evenly by
+  // its own length, and its last non-empty split also takes its tree keys
   const int rblocks = attention_row_blocks(d.max_nodes, G);
   const long long base = static_cast<long long>(rblocks) * d.batch * d.num_kv_heads;
-  const int max_splits = std::max(1, std::min(kMaxAttnParts, (d.ctx_max + 63) / 64));
-  long long ns = nsm / base;
-  ns = std::max(1LL, std::min(ns, static_cast<long long>(max_splits)));
-  const int per = static_cast<int>((std::max(d.ctx_max, 1) + ns - 1) / ns);
-  L.split_len = ((per + 63) / 64) * 64;
-  L.n_splits = std::max(1, (d.ctx_max + L.split_len - 1) / L.split_len);
-  L.n_parts = L.n_splits;
+  const long long max_splits = std::min(kMaxAttnParts, (d.ctx_max + 63) / 64);
+  L.n_parts = static_cast<int>(std::max(1LL, std::min(nsm / base, max_splits)));
   // more than one 128-node tile: the LM head (wide kernel) leaves no room on
   // its SMs, attention runs after it on the tensor-core kernel, unsplit
   L.attn_tc = (d.dtype == ASD_BF16 && T > kAttnTcRows) ? 1 : 0;
   if (L.attn_tc && attention_pingpong(d.batch, d.num_kv_heads, G, T, nsm)) L.attn_tc = 2;
-  if (L.attn_tc) {
-    L.n_splits = L.n_parts = 1;
-    L.split_len = std::max(d.ctx_max, 1);
-  }
   size_t off = 0;
   L.status = off;      off = align256(off + 16);
   L.seq_flags = off;   off = align256(off + 4 * static_cast<size_t>(d.batch));
@@ -292,8 +283,6 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
   a.page_size = d.page_size;
   a.pages_per_seq = d.page_size ? d.ctx_max / d.page_size : 0;
   a.num_pages = d.num_pages;
-  a.n_splits = c.L.n_splits;
-  a.split_len = c.L.split_len;
   a.n_parts = c.L.n_parts;
   a.max_nodes = d.max_nodes;
   a.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(d.head_dim)));

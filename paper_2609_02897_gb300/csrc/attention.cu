@@ -8,7 +8,7 @@
 // query rows of a (sequence, KV head) pair are its N nodes times the G query
 // heads that share the KV head (grouped-query attention), packed node-major:
 // row r -> node r / G, head g*G + r % G.  Split z covers context keys
-// [z*L, (z+1)*L) (flash-decoding split-KV); the CTA of the sequence's last
+// [z*L, (z+1)*L), L from the sequence's own length (flash-decoding split-KV); the CTA of the sequence's last
 // non-empty split also covers the tree keys, where a node only sees its
 // ancestors (bitmasks derived in-kernel from the parent array).  The splits of one
 // (row block, sequence x KV head) form a thread-block cluster: each CTA keeps
@@ -101,14 +101,17 @@ struct RowMap {
   }
 };
 
-// Key range of one CTA: context keys [kbeg, kend) and, for the sequence's
-// last non-empty split (split 0 when the context is empty), the tree keys.
+// Key range of one CTA: split z of n_parts equal runs of the sequence's own
+// context (whole key tiles; the host knows the cache's capacity only), and for
+// the last non-empty split (split 0 when the context is empty) the tree keys.
 struct KeyRange {
   int kbeg, kend, nctx, ntree;
-  __device__ KeyRange(int z, int split_len, int ctx, int n) {
-    kbeg = z * split_len;
+  __device__ KeyRange(int z, int n_parts, int ctx, int n) {
+    const int tiles = (ctx + kKeysPerTile - 1) / kKeysPerTile;
+    const int split_len = max((tiles + n_parts - 1) / n_parts, 1) * kKeysPerTile;
+    kbeg = min(z * split_len, ctx);
     kend = min(kbeg + split_len, ctx);
-    nctx = kend > kbeg ? (kend - kbeg + kKeysPerTile - 1) / kKeysPerTile : 0;
+    nctx = (kend - kbeg + kKeysPerTile - 1) / kKeysPerTile;
     const int last = ctx > 0 ? (ctx - 1) / split_len : 0;
     ntree = (z == last) ? (n + kKeysPerTile - 1) / kKeysPerTile : 0;
   }
@@ -252,7 +255,7 @@ __global__ void __launch_bounds__(128) attn_bf16_kernel(const __grid_constant__ 
     return;
   }
   const int nrows = min(kRowsPerCta, R - r0);
-  const KeyRange kr(z, p.split_len, min(p.ctx_len[b], p.ctx_max), n);
+  const KeyRange kr(z, p.n_parts, min(max(p.ctx_len[b], 0), p.ctx_max), n);
   const RowMap rm{s0, p.G, p.Hq, g, r0};
 
   uint32_t base = smem_u32(smem_raw);
@@ -538,20 +541,44 @@ __global__ void __launch_bounds__(128) attn_bf16_kernel(const __grid_constant__ 
 }
 
 // ----------------------------------------------------------- fp32 SIMT path
-// One warp per query row, 32 keys at a time: lane j scores key j of the chunk
-// over the whole head dimension (its K row loads in flight with the other
-// lanes'), the warp folds the chunk into the running softmax, and each lane
-// accumulates P V for D/32 output columns.  Exact fp32 math for the fp32
-// workloads (no reduced-precision tensor path).
+// Exact fp32 math on the CUDA cores.  The CTA's up to 64 query rows sit in
+// shared memory; its keys (the split's context keys, then the tree's) come 32 at
+// a time, K and V rows through a two-stage cp.async ring, and serve all rows:
+// scores by 16 x 16 threads (row, key), the online softmax by a warp per row
+// with a lane per key, P V by threads that own 4 columns of up to 64 rows.  With
+// a warp per row walking K and V in global memory, a load at a time per key, the
+// tiny fp32 workload's kernel took 42.6 us (profiled; now 15.6), nearly all of it
+// load latency.
+constexpr int kF32Threads = 256;
+
 template <int D>
-__global__ void __launch_bounds__(128) attn_f32_kernel(const AttnParams p) {
-  constexpr int kPer = D / 32;
-  extern __shared__ __align__(16) uint8_t smem_raw[];
-  __shared__ float s_lse[kRowsPerCta];
+struct F32Geom {
+  static constexpr int kLd = D + 4;   // padded row: 16-byte reads of 8 rows touch all banks
+  static constexpr int kTile = kKeysPerTile * kLd;
+  static constexpr int kQ = 0;
+  static constexpr int kK = kRowsPerCta * kLd;
+  static constexpr int kV = kK + 2 * kTile;
+  static constexpr int kP = kV + 2 * kTile;
+  static constexpr size_t kBytes = sizeof(float) * (kP + kRowsPerCta * (kKeysPerTile + 1));
+  static_assert(4 * kTile >= kRowsPerCta * D, "the K/V ring holds the output rows at the end");
+};
+
+// 16 bytes of global memory -> shared memory, zeros unless `in`.
+__device__ __forceinline__ void copy16_async(float* dst, const float* src, bool in) {
+  const int n = in ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n)
+               : "memory");
+}
+
+template <int D>
+__global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const AttnParams p) {
+  using G = F32Geom<D>;
+  constexpr int kLd = G::kLd, kPLd = kKeysPerTile + 1;
+  extern __shared__ __align__(16) float smem_f[];
+  __shared__ float s_lse[kRowsPerCta], s_m[kRowsPerCta], s_l[kRowsPerCta], s_al[kRowsPerCta];
+  __shared__ int s_seen[2][kKeysPerTile];   // the stage's key takes part: 1 context, 2 + j node j
   __shared__ int s_par[kMaxNodes];
   __shared__ uint64_t s_anc[kMaxNodes][2];
-  __shared__ __align__(16) float s_q[4][D];          // each warp's current query row
-  float* s_o = reinterpret_cast<float*>(smem_raw);   // [64][D] split output rows
   pdl_launch_dependents();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rb = blockIdx.x, bg = blockIdx.y, z = blockIdx.z;
@@ -565,7 +592,7 @@ __global__ void __launch_bounds__(128) attn_f32_kernel(const AttnParams p) {
     return;
   }
   const int nrows = min(kRowsPerCta, R - r0);
-  const KeyRange kr(z, p.split_len, min(p.ctx_len[b], p.ctx_max), n);
+  const KeyRange kr(z, p.n_parts, min(max(p.ctx_len[b], 0), p.ctx_max), n);
   const RowMap rm{s0, p.G, p.Hq, g, r0};
   const float* qp = static_cast<const float*>(p.q);
   const float* kc = static_cast<const float*>(p.k_cache);
@@ -574,104 +601,172 @@ __global__ void __launch_bounds__(128) attn_f32_kernel(const AttnParams p) {
   const float* tv = static_cast<const float*>(p.tree_v);
   const float c = p.scale_log2;
   const int ps = p.page_size;
-  const int nctx_keys = max(0, kr.kend - kr.kbeg);
-  const int ntree_keys = kr.ntree > 0 ? n : 0;
-  if (ntree_keys) tree_ancestors(p.parent, s0, n, s_par, s_anc);
+  const int nctx_keys = kr.kend - kr.kbeg;
+  const int nkeys = nctx_keys + (kr.ntree > 0 ? n : 0);
+  const int ntiles = (nkeys + kKeysPerTile - 1) / kKeysPerTile;
 
-  // element offset of key t's K / V row for this (sequence, KV head), or -1
-  // when the key does not take part (not an ancestor, or a bad page)
-  auto key_off = [&](int t, uint64_t alo, uint64_t ahi) -> long long {
-    if (t >= nctx_keys) {
-      const int key = t - nctx_keys;
-      if (!anc_bit(alo, ahi, key)) return -1;
-      return (static_cast<long long>(s0 + key) * p.Hkv + g) * D;
-    }
-    const int key = kr.kbeg + t;
-    if (ps == 0) return ((static_cast<long long>(b) * p.Hkv + g) * p.ctx_max + key) * D;
-    const int page = p.page_table[static_cast<size_t>(b) * p.pages_per_seq + key / ps];
-    if (page < 0 || page >= p.num_pages) {
-      set_status(p.status, ASD_ERR_CTX_RANGE);
-      return -1;
-    }
-    return ((static_cast<long long>(page) * p.Hkv + g) * ps + key % ps) * D;
-  };
-  const int nkeys = nctx_keys + ntree_keys;
-  float* s_qw = s_q[warp];
-
-  for (int r = warp; r < nrows; r += 4) {
-    const size_t gr = rm.grow(r);
-    if (nkeys == 0) {
-      // empty split: weight-zero log-sum-exp and a finite (zero) row
-      if (lane == 0) s_lse[r] = -INFINITY;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) s_o[r * D + lane + 32 * k] = 0.f;
-      continue;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) s_qw[lane + 32 * k] = qp[gr * D + lane + 32 * k];
-    __syncwarp();
-    uint64_t alo = 0, ahi = 0;
-    if (ntree_keys) {
-      const int node = (r0 + r) / p.G;
-      alo = s_anc[node][0];
-      ahi = s_anc[node][1];
-    }
-    float ov[kPer];
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) ov[k] = 0.f;
-    float m = -INFINITY, l = 0.f;
-    // 32 keys at a time: lane j scores key t0 + j over the whole head
-    // dimension, then the warp folds the chunk into the running softmax and
-    // every lane adds p_j V_j to its D/32 output columns
-    for (int t0 = 0; t0 < nkeys; t0 += 32) {
-      const int t = t0 + lane;
-      const long long off = t < nkeys ? key_off(t, alo, ahi) : -1;
-      float dot = -INFINITY;
-      if (off >= 0) {
-        const float4* kr4 = reinterpret_cast<const float4*>((t >= nctx_keys ? tk : kc) + off);
-        const float4* q4 = reinterpret_cast<const float4*>(s_qw);
-        float acc = 0.f;
-#pragma unroll 8
-        for (int d = 0; d < D / 4; ++d) {
-          const float4 kk = kr4[d], qq = q4[d];
-          acc = fmaf(qq.x, kk.x, acc);
-          acc = fmaf(qq.y, kk.y, acc);
-          acc = fmaf(qq.z, kk.z, acc);
-          acc = fmaf(qq.w, kk.w, acc);
+  // K and V rows of keys [32 t, 32 t + 32) of the split; a key past the end or
+  // on a bad page reads as zeros and takes no part
+  auto load = [&](int t) {
+    const int stage = t & 1;
+    for (int i = tid; i < kKeysPerTile * (D / 4); i += kF32Threads) {
+      const int j = i / (D / 4), ch = i - j * (D / 4);
+      const int u = t * kKeysPerTile + j;
+      long long off = -1;
+      int seen = 0;
+      if (u >= nctx_keys && u < nkeys) {
+        const int node = u - nctx_keys;
+        off = (static_cast<long long>(s0 + node) * p.Hkv + g) * D;
+        seen = 2 + node;
+      } else if (u < nctx_keys) {
+        const int key = kr.kbeg + u;
+        if (ps == 0) {
+          off = ((static_cast<long long>(b) * p.Hkv + g) * p.ctx_max + key) * D;
+        } else {
+          const int page = p.page_table[static_cast<size_t>(b) * p.pages_per_seq + key / ps];
+          if (page < 0 || page >= p.num_pages)
+            set_status(p.status, ASD_ERR_CTX_RANGE);
+          else
+            off = ((static_cast<long long>(page) * p.Hkv + g) * ps + key % ps) * D;
         }
-        dot = acc;
+        seen = off >= 0 ? 1 : 0;
       }
-      float cm = dot;
+      const bool tree = u >= nctx_keys, in = off >= 0;
+      const long long at = in ? off + 4 * ch : 0;
+      copy16_async(smem_f + G::kK + stage * G::kTile + j * kLd + 4 * ch, (tree ? tk : kc) + at, in);
+      copy16_async(smem_f + G::kV + stage * G::kTile + j * kLd + 4 * ch, (tree ? tv : vc) + at, in);
+      if (ch == 0) s_seen[stage][j] = seen;
+    }
+  };
+
+  for (int i = tid; i < nrows * (D / 4); i += kF32Threads) {
+    const int r = i / (D / 4), ch = i - r * (D / 4);
+    copy16_async(smem_f + G::kQ + r * kLd + 4 * ch, qp + rm.grow(r) * D + 4 * ch, true);
+  }
+  if (ntiles > 0) load(0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (int r = tid; r < kRowsPerCta; r += kF32Threads) {
+    s_m[r] = -INFINITY;
+    s_l[r] = 0.f;
+  }
+  if (kr.ntree > 0) tree_ancestors(p.parent, s0, n, s_par, s_anc);
+
+  // P V: the thread's 4 columns and rows pr, pr + kPr, ...
+  constexpr int kPc = D / 4, kPr = kF32Threads / kPc, kRows = kRowsPerCta / kPr;
+  const int pc = tid % kPc, pr = tid / kPc;
+  float4 o[kRows];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, o));
-      if (cm == -INFINITY) continue;          // nothing visible in this chunk (uniform)
+  for (int i = 0; i < kRows; ++i) o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int sr = tid >> 4, sk = tid & 15;    // scores: rows sr + 16 i, keys sk, sk + 16
+  float* sP = smem_f + G::kP;
+
+  for (int t = 0; t < ntiles; ++t) {
+    const int stage = t & 1;
+    if (t + 1 < ntiles) load(t + 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    const float* sK = smem_f + G::kK + stage * G::kTile;
+    const float* sV = smem_f + G::kV + stage * G::kTile;
+    // scores, masked
+    float acc[4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0.f;
+#pragma unroll 4
+    for (int d = 0; d < D; d += 4) {
+      const float4 k0 = *reinterpret_cast<const float4*>(sK + sk * kLd + d);
+      const float4 k1 = *reinterpret_cast<const float4*>(sK + (sk + 16) * kLd + d);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (16 * i >= nrows) break;           // uniform over the CTA
+        // rows past nrows read what is there; their scores are not used
+        const float4 q = *reinterpret_cast<const float4*>(smem_f + G::kQ + (sr + 16 * i) * kLd + d);
+        acc[i][0] = fmaf(q.x, k0.x, acc[i][0]);
+        acc[i][0] = fmaf(q.y, k0.y, acc[i][0]);
+        acc[i][0] = fmaf(q.z, k0.z, acc[i][0]);
+        acc[i][0] = fmaf(q.w, k0.w, acc[i][0]);
+        acc[i][1] = fmaf(q.x, k1.x, acc[i][1]);
+        acc[i][1] = fmaf(q.y, k1.y, acc[i][1]);
+        acc[i][1] = fmaf(q.z, k1.z, acc[i][1]);
+        acc[i][1] = fmaf(q.w, k1.w, acc[i][1]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = sr + 16 * i;
+      if (r >= nrows) break;
+      const int node = (r0 + r) / p.G;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int seen = s_seen[stage][sk + 16 * e];
+        const bool vis = seen == 1 || (seen >= 2 && anc_bit(s_anc[node][0], s_anc[node][1], seen - 2));
+        sP[r * kPLd + sk + 16 * e] = vis ? acc[i][e] : -INFINITY;
+      }
+    }
+    __syncthreads();
+    // online softmax, a warp per row, lane = key
+    for (int r = warp; r < nrows; r += kF32Threads / 32) {
+      const float x = sP[r * kPLd + lane];
+      float cm = x;
+#pragma unroll
+      for (int k = 16; k > 0; k >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, k));
+      const float m = s_m[r], l = s_l[r];
       const float mn = fmaxf(m, cm);
       const float al = m == -INFINITY ? 0.f : exp2f((m - mn) * c);
-      const float pe = dot == -INFINITY ? 0.f : exp2f((dot - mn) * c);
-      float ps_ = pe;
+      const float pe = x == -INFINITY ? 0.f : exp2f((x - mn) * c);
+      float sum = pe;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) ps_ += __shfl_xor_sync(0xffffffffu, ps_, o);
-      l = l * al + ps_;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) ov[k] *= al;
-      const int nj = min(32, nkeys - t0);
-#pragma unroll 4
-      for (int j = 0; j < nj; ++j) {
-        const float pj = __shfl_sync(0xffffffffu, pe, j);
-        const long long oj = __shfl_sync(0xffffffffu, off, j);
-        if (pj == 0.f || oj < 0) continue;    // uniform over the warp
-        const float* vr = (t0 + j >= nctx_keys ? tv : vc) + oj;
-#pragma unroll
-        for (int k = 0; k < kPer; ++k) ov[k] = fmaf(pj, vr[lane + 32 * k], ov[k]);
+      for (int k = 16; k > 0; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
+      sP[r * kPLd + lane] = pe;
+      __syncwarp();
+      if (lane == 0) {
+        s_m[r] = mn;
+        s_l[r] = l * al + sum;
+        s_al[r] = al;
       }
-      m = mn;
     }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
+    __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) s_o[r * D + lane + 32 * k] = ov[k] * inv;
-    if (lane == 0) s_lse[r] = (m == -INFINITY) ? -INFINITY : m * c + log2f(l);
+    for (int i = 0; i < kRows; ++i) {
+      if (pr + kPr * i >= nrows) break;
+      const float al = s_al[pr + kPr * i];
+      o[i].x *= al;
+      o[i].y *= al;
+      o[i].z *= al;
+      o[i].w *= al;
+    }
+#pragma unroll 4
+    for (int j = 0; j < kKeysPerTile; ++j) {
+      const float4 v = *reinterpret_cast<const float4*>(sV + j * kLd + 4 * pc);
+#pragma unroll
+      for (int i = 0; i < kRows; ++i) {
+        if (pr + kPr * i >= nrows) break;
+        const float w = sP[(pr + kPr * i) * kPLd + j];
+        if (w != 0.f) {   // a masked key's V may hold anything
+          o[i].x = fmaf(w, v.x, o[i].x);
+          o[i].y = fmaf(w, v.y, o[i].y);
+          o[i].z = fmaf(w, v.z, o[i].z);
+          o[i].w = fmaf(w, v.w, o[i].w);
+        }
+      }
+    }
+    __syncthreads();   // the stage and P are free
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // the split's rows, normalised, over the K/V ring; empty splits leave zero
+  // rows of zero weight
+  float* s_o = smem_f + G::kK;
+#pragma unroll
+  for (int i = 0; i < kRows; ++i) {
+    const int r = pr + kPr * i;
+    if (r >= nrows) break;
+    const float l = s_l[r], inv = l > 0.f ? 1.f / l : 0.f;
+    *reinterpret_cast<float4*>(s_o + r * D + 4 * pc) =
+        make_float4(o[i].x * inv, o[i].y * inv, o[i].z * inv, o[i].w * inv);
+  }
+  for (int r = tid; r < nrows; r += kF32Threads)
+    s_lse[r] = s_m[r] == -INFINITY ? -INFINITY : s_m[r] * c + log2f(s_l[r]);
   cluster_merge<float, D>(p, rm, nrows, smem_u32(s_o), smem_u32(s_lse));
   pdl_wait();
 }
@@ -696,11 +791,11 @@ static dim3 attn_grid(const AttnParams& p) {
 
 // The n_parts splits of one (row block, sequence x KV head) form a cluster.
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_attn(void (*kernel)(KArgs...), const AttnParams& p, size_t smem,
-                               cudaStream_t s, Args&&... args) {
+static cudaError_t launch_attn(void (*kernel)(KArgs...), const AttnParams& p, int threads,
+                               size_t smem, cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = attn_grid(p);
-  cfg.blockDim = dim3(128);
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
@@ -721,17 +816,19 @@ cudaError_t launch_attention_bf16(const AttnParams& p, const CUtensorMap& tm_k,
   if (p.D == 128) {
     cudaError_t err = set_smem_attrs(attn_bf16_kernel<128>, smem);
     if (err != cudaSuccess) return err;
-    return launch_attn(attn_bf16_kernel<128>, p, smem, s, tm_k, tm_v, p);
+    return launch_attn(attn_bf16_kernel<128>, p, 128, smem, s, tm_k, tm_v, p);
   }
   cudaError_t err = set_smem_attrs(attn_bf16_kernel<64>, smem);
   if (err != cudaSuccess) return err;
-  return launch_attn(attn_bf16_kernel<64>, p, smem, s, tm_k, tm_v, p);
+  return launch_attn(attn_bf16_kernel<64>, p, 128, smem, s, tm_k, tm_v, p);
 }
 
 cudaError_t launch_attention_f32(const AttnParams& p, cudaStream_t s) {
-  const size_t smem = static_cast<size_t>(kRowsPerCta) * p.D * sizeof(float);
-  if (p.D == 128) return launch_attn(attn_f32_kernel<128>, p, smem, s, p);
-  return launch_attn(attn_f32_kernel<64>, p, smem, s, p);
+  const size_t smem = p.D == 128 ? F32Geom<128>::kBytes : F32Geom<64>::kBytes;
+  auto* k = p.D == 128 ? attn_f32_kernel<128> : attn_f32_kernel<64>;
+  const cudaError_t err = set_smem_attrs(k, smem);
+  if (err != cudaSuccess) return err;
+  return launch_attn(k, p, kF32Threads, smem, s, p);
 }
 
 }  // namespace asd

@@ -42,9 +42,8 @@ struct WsLayout {
   size_t at_part;      // attention partials: plan int2[B], then (max, sum) and output rows
   size_t full;         // total and the attention partials (asd_workspace_bytes)
   int g_lm;            // CTAs of the LM-head kernel (vocabulary ranges)
-  int n_splits;        // context splits of the attention kernel
-  int split_len;       // keys per context split (multiple of 64)
-  int n_parts;         // = n_splits (the tree keys ride with the last split)
+  int n_parts;         // context splits of the mma.sync and fp32 attention kernels (the
+                       // tree keys ride with the last one)
   // lazy LM-head schedule only (0 otherwise)
   size_t lz_count;     // int32[2][max_path + 1]: rows, then active sequences per pass
   size_t lz_seq;       // int2[B]: a sequence's first row and rows in the pass

@@ -77,7 +77,7 @@ struct AttnParams {
   void* out;                // [T, Hq, D]
   int B, T, Hq, Hkv, G, D;
   int ctx_max, page_size, pages_per_seq, num_pages;
-  int n_splits, split_len, n_parts, max_nodes;
+  int n_parts, max_nodes;
   float scale_log2;         // log2(e) / sqrt(D)
   int q_tma;                // tensor-core kernels: the query tiles by TMA (tm_q)
   // one-tile tensor-core kernel: partial results of sequences cut into chunks
