@@ -324,8 +324,10 @@ int32_t asd_lm_head_variant(const asd_dims* dims, int32_t total_nodes, const voi
  * kernel with one 128-row query tile per CTA, 3 the tensor-core kernel with two
  * query tiles per CTA in ping-pong (when its 256-row items fill at least two
  * waves of CTAs), 4 the fp32 kernel, 0 for invalid arguments.
- * asd_tree_attention by itself has no LM head to share the SMs with and runs
- * form 2 where a step runs form 1 (same semantics, other roundings).  Form 2
+ * Where the answer is 1, a step whose contexts turn out longer than the LM head
+ * hides runs form 2 behind it instead (the device decides from ctx_len), and
+ * asd_tree_attention by itself, without an LM head to share the SMs with,
+ * always runs form 2 (same semantics, other roundings).  Form 2
  * may cut long contexts into chunks, whose length follows the batch's context
  * lengths.
  */

@@ -286,71 +286,73 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
   a.n_parts = c.L.n_parts;
   a.max_nodes = d.max_nodes;
   a.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(d.head_dim)));
-  cudaError_t err;
+  a.nsm = device_sm_count();
+  a.co_tiles = -1;
+  if (d.dtype != ASD_BF16)
+    return launch_attention_f32(a, c.st) == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
   // up to 128 nodes the mma.sync kernel runs beside the LM head of a verify
-  // step; with the SMs to itself the tensor-core kernel is the faster one at
-  // every size
-  const int tc = c.L.attn_tc ? c.L.attn_tc : (d.dtype == ASD_BF16 && !in_step ? 1 : 0);
-  if (tc) {
-    CUtensorMap tk, tv, ttk, ttv, tq;
-    uint64_t rows;
-    uint32_t box_rows;
-    if (d.page_size == 0) {
-      rows = static_cast<uint64_t>(d.batch) * d.num_kv_heads * static_cast<uint64_t>(d.ctx_max);
-      box_rows = static_cast<uint32_t>(kAttnTcKeys);
-    } else {
-      rows = static_cast<uint64_t>(d.num_pages) * d.num_kv_heads * d.page_size;
-      box_rows = static_cast<uint32_t>(std::min(d.page_size, kAttnTcKeys));
-    }
-    if (rows == 0) rows = 1;  // no context at all: the map is never used
-    if (!make_tmap_bf16(&tk, k_cache, d.head_dim, rows, box_rows) ||
-        !make_tmap_bf16(&tv, v_cache, d.head_dim, rows, box_rows) ||
-        !make_tree_tmap_bf16(&ttk, tree_k, d.head_dim, d.num_kv_heads, c.T, kAttnTcKeys) ||
-        !make_tree_tmap_bf16(&ttv, tree_v, d.head_dim, d.num_kv_heads, c.T, kAttnTcKeys))
-      return ASD_ERR_CUDA;
-    // the tensor-core kernels load the query tiles by TMA where G divides
-    // their 128 rows (otherwise the softmax warps stage them; tq goes unused)
-    tq = ttk;
-    if (attention_q_tma_ok(a.G)) {
-      if (!make_q_tmap_bf16(&tq, q, d.head_dim, d.num_q_heads, c.T, a.G)) return ASD_ERR_CUDA;
-      a.q_tma = 1;
-    }
-    a.nsm = device_sm_count();
-    if (tc == 1) {
-      // a standalone call has no use for the LM head's partials either
-      const size_t at = in_step ? c.L.at_part : c.L.lm_part;
-      const size_t rows_at = at + align256(sizeof(int2) * static_cast<size_t>(d.batch));
-      const size_t row_bytes = sizeof(float2) + 4 * static_cast<size_t>(d.head_dim);
-      const size_t end = std::min(c.ws_bytes, c.L.full);
-      if (end > rows_at) {
-        a.part_cap = std::min<long long>(attention_split_rows(d, c.T, a.nsm),
-                                         static_cast<long long>((end - rows_at) / row_bytes) & ~63LL);
-        a.plan = ws_at<int2>(c.ws, at);
-        a.part_ml = ws_at<float2>(c.ws, rows_at);
-        a.part_o = ws_at<float>(c.ws, rows_at + sizeof(float2) * static_cast<size_t>(a.part_cap));
-      }
-    }
-    err = launch_attention_tc(a, tk, tv, ttk, ttv, tq, tc == 2, c.st);
-  } else if (d.dtype == ASD_BF16) {
-    CUtensorMap tk, tv;
-    uint64_t rows;
-    uint32_t box_rows;
-    if (d.page_size == 0) {
-      rows = static_cast<uint64_t>(d.batch) * d.num_kv_heads * static_cast<uint64_t>(d.ctx_max);
-      box_rows = static_cast<uint32_t>(attention_keys_per_tile());
-    } else {
-      rows = static_cast<uint64_t>(d.num_pages) * d.num_kv_heads * d.page_size;
-      box_rows = static_cast<uint32_t>(std::min(d.page_size, attention_keys_per_tile()));
-    }
-    if (rows == 0) rows = 1;  // no context at all: the map is never used
-    if (!make_tmap_bf16(&tk, k_cache, d.head_dim, rows, box_rows) ||
-        !make_tmap_bf16(&tv, v_cache, d.head_dim, rows, box_rows))
-      return ASD_ERR_CUDA;
-    err = launch_attention_bf16(a, tk, tv, c.st);
-  } else {
-    err = launch_attention_f32(a, c.st);
+  // step, unless the contexts may be longer than the LM head hides: then both
+  // kernels are launched and the context lengths decide which one works.
+  // With the SMs to itself the tensor-core kernel is the faster one at every
+  // size.
+  const bool beside = in_step && !c.L.attn_tc;
+  bool tc = !beside;
+  if (beside && attention_co_tiles_max(d, c.L.n_parts, a.nsm) > attention_co_tiles_limit(d)) {
+    a.co_tiles = attention_co_tiles_limit(d);
+    tc = true;
   }
-  return err == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
+  // maps over the context cache's rows with boxes of `keys` rows at most
+  auto cache_maps = [&](int keys, CUtensorMap* tk, CUtensorMap* tv) {
+    uint64_t rows;
+    int box;
+    if (d.page_size == 0) {
+      rows = static_cast<uint64_t>(d.batch) * d.num_kv_heads * static_cast<uint64_t>(d.ctx_max);
+      box = keys;
+    } else {
+      rows = static_cast<uint64_t>(d.num_pages) * d.num_kv_heads * d.page_size;
+      box = std::min(d.page_size, keys);
+    }
+    if (rows == 0) rows = 1;  // no context at all: the map is never used
+    return make_tmap_bf16(tk, k_cache, d.head_dim, rows, static_cast<uint32_t>(box)) &&
+           make_tmap_bf16(tv, v_cache, d.head_dim, rows, static_cast<uint32_t>(box));
+  };
+  CUtensorMap tk, tv;
+  if (beside) {
+    if (!cache_maps(attention_keys_per_tile(), &tk, &tv) ||
+        launch_attention_bf16(a, tk, tv, c.st) != cudaSuccess)
+      return ASD_ERR_CUDA;
+  }
+  if (!tc) return ASD_OK;
+  CUtensorMap ttk, ttv, tq;
+  if (!cache_maps(kAttnTcKeys, &tk, &tv) ||
+      !make_tree_tmap_bf16(&ttk, tree_k, d.head_dim, d.num_kv_heads, c.T, kAttnTcKeys) ||
+      !make_tree_tmap_bf16(&ttv, tree_v, d.head_dim, d.num_kv_heads, c.T, kAttnTcKeys))
+    return ASD_ERR_CUDA;
+  // the tensor-core kernels load the query tiles by TMA where G divides
+  // their 128 rows (otherwise the softmax warps stage them; tq goes unused)
+  tq = ttk;
+  if (attention_q_tma_ok(a.G)) {
+    if (!make_q_tmap_bf16(&tq, q, d.head_dim, d.num_q_heads, c.T, a.G)) return ASD_ERR_CUDA;
+    a.q_tma = 1;
+  }
+  const bool pingpong = c.L.attn_tc == 2;
+  if (!pingpong) {
+    // a standalone call has no use for the LM head's partials either
+    const size_t at = in_step ? c.L.at_part : c.L.lm_part;
+    const size_t rows_at = at + align256(sizeof(int2) * static_cast<size_t>(d.batch));
+    const size_t row_bytes = sizeof(float2) + 4 * static_cast<size_t>(d.head_dim);
+    const size_t end = std::min(c.ws_bytes, c.L.full);
+    if (end > rows_at) {
+      a.part_cap = std::min<long long>(attention_split_rows(d, c.T, a.nsm),
+                                       static_cast<long long>((end - rows_at) / row_bytes)) &
+                   ~63LL;   // part_o stays aligned behind part_ml
+      a.plan = ws_at<int2>(c.ws, at);
+      a.part_ml = ws_at<float2>(c.ws, rows_at);
+      a.part_o = ws_at<float>(c.ws, rows_at + sizeof(float2) * static_cast<size_t>(a.part_cap));
+    }
+  }
+  return launch_attention_tc(a, tk, tv, ttk, ttv, tq, pingpong, c.st) == cudaSuccess ? ASD_OK
+                                                                                    : ASD_ERR_CUDA;
 }
 
 // True when `w` is device memory of the current device (the only memory the
@@ -744,7 +746,7 @@ asd_status asd_verify_step(const asd_dims* dims, const asd_verify_args* a, void*
   // The LM head goes first and takes one CTA per SM; the attention kernel
   // starts right behind it (it reads no output of the LM head).  Up to 128
   // nodes its CTAs share the SMs with the LM head's while the weights stream
-  // in; beyond that the wide LM head fills the SMs' shared memory and the
+  // in, unless the contexts are longer than that hides; beyond that the wide LM head fills the SMs' shared memory and the
   // tensor-core attention runs after it.  The lazy schedule also finalises
   // the rows it computes, so the tail only walks.
   const bool lazy = c.d.lm_head_schedule == ASD_LM_LAZY_LEVELS;

@@ -16,13 +16,15 @@
 // after a cluster barrier every CTA merges a slice of the rows by reading its
 // peers' partials through distributed shared memory.  No partial leaves the
 // cluster.
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace asd {
 namespace {
 
-constexpr int kRowsPerCta = 64;   // 4 warps x 16 query rows
-constexpr int kKeysPerTile = 32;  // keys per K/V tile (TMA box rows)
+constexpr int kRowsPerCta = kCoRows;   // 4 warps x 16 query rows
+constexpr int kKeysPerTile = kCoKeys;  // keys per K/V tile (TMA box rows)
 constexpr int kAttnStages = 2;
 // With D = 128 a CTA takes 1 KB + 16 KB (Q) + 32 KB (K/V ring) of dynamic
 // shared memory, small enough to share an SM with an LM-head CTA.
@@ -243,6 +245,10 @@ __global__ void __launch_bounds__(128) attn_bf16_kernel(const __grid_constant__ 
   // ancestor masks itself and keeps every access inside the caller's arrays
   // whatever the inputs hold (the preparation kernel reports malformed ones;
   // the outputs of such a sequence are then unspecified).
+  if (p.co_tiles >= 0 && !attention_beside_lm_head(p)) {   // the tensor-core kernel's step
+    pdl_wait();
+    return;
+  }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rb = blockIdx.x, bg = blockIdx.y, z = blockIdx.z;
   const int b = bg / p.Hkv, g = bg - b * p.Hkv;
@@ -783,6 +789,30 @@ int attention_keys_per_tile() { return kKeysPerTile; }
 
 int attention_row_blocks(int max_nodes, int G) {
   return (max_nodes * G + kRowsPerCta - 1) / kRowsPerCta;
+}
+
+long long attention_co_tiles_max(const asd_dims& d, int n_parts, int nsm) {
+  const int G = d.num_q_heads / d.num_kv_heads;
+  const long long tree = (d.max_nodes + kKeysPerTile - 1) / kKeysPerTile;
+  const long long tiles = (static_cast<long long>(d.ctx_max) + kKeysPerTile - 1) / kKeysPerTile;
+  const long long items = static_cast<long long>(attention_row_blocks(d.max_nodes, G)) * d.num_kv_heads;
+  return std::max((tiles + n_parts - 1) / n_parts + tree,
+                  d.batch * ((items * (tiles + tree) + nsm - 1) / nsm));
+}
+
+int attention_co_tiles_limit(const asd_dims& d) {
+  // A tile takes the kernel about 1.2 us at D = 128 (0.9 at 64), the LM head
+  // streams W at about 6.4 TB/s, and the tensor-core kernel needs about a
+  // quarter of this one's time: it wins from 4/3 of the LM head's time on, and
+  // beside a short LM head from about the time that its own launches take.
+  // Steps of a Llama-3.1-8B-shaped LM head (limit 182 tiles), always this kernel
+  // before and the rule now: 60 nodes at context 24576 276 -> 218 us, 65536
+  // 628 -> 254; 8 x 8 nodes at 16384 349 -> 266, 32768 631 -> 339; under the
+  // limit (60 nodes at 16384: 205) the same.  Deciding on the device costs a
+  // step of short contexts in a roomy cache 1.5 to 5 us.
+  const double lm_us = 2.0 * d.vocab * static_cast<double>(d.hidden) / 6.4e6;
+  const double tile_us = d.head_dim == 128 ? 1.2 : 0.9;
+  return static_cast<int>(std::max(16.0, std::min(4.0 / 3.0 * lm_us / tile_us, 1e6)));
 }
 
 static dim3 attn_grid(const AttnParams& p) {

@@ -659,6 +659,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ PlanSmem s_plan;
 
   pdl_launch_dependents();
+  if (p.co_tiles >= 0 && attention_beside_lm_head(p)) {   // the mma.sync kernel's step
+    pdl_wait();
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long budget = wait_budget(p.wait_cycles);
 
@@ -904,6 +908,7 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const AttnPar
   const int w = (threadIdx.x >> 5) % kMergeWarps, rl = (threadIdx.x >> 5) / kMergeWarps;
   const int s0 = p.cu_nodes[b], n = p.cu_nodes[b + 1] - s0, R = n * p.G;
   pdl_wait();
+  if (p.co_tiles >= 0 && attention_beside_lm_head(p)) return;   // nothing was cut
   if (n <= 0 || n > kMaxNodes || s0 < 0 || s0 + n > p.T || static_cast<int>(blockIdx.x) * kMergeRows >= R)
     return;
   const int2 plan = __ldcg(p.plan + b);

@@ -80,13 +80,40 @@ struct AttnParams {
   int n_parts, max_nodes;
   float scale_log2;         // log2(e) / sqrt(D)
   int q_tma;                // tensor-core kernels: the query tiles by TMA (tm_q)
-  // one-tile tensor-core kernel: partial results of sequences cut into chunks
   int nsm;                  // SMs of the device
+  // steps of up to 128 nodes whose cache could hold more keys than the LM head
+  // hides: the 32-key tiles up to which the mma.sync kernel beside the LM head
+  // takes the step, beyond which the tensor-core kernel does after it (both
+  // are launched and decide alike, attention_beside_lm_head); -1: no choice
+  int co_tiles;
+  // one-tile tensor-core kernel: partial results of sequences cut into chunks
   long long part_cap;       // rows that part_o / part_ml hold (0: no splitting)
   float* part_o;            // [part_cap][D]: a chunk's unnormalised output row
   float2* part_ml;          // [part_cap]: its reference max (log2 domain) and sum
   int2* plan;               // [B]: first partial row and chunks of a sequence
 };
+// Whether this step's attention runs beside the LM head (p.co_tiles): the key
+// tiles of its longest split, or an even share of all of them per SM, against
+// the limit.  Every lane of a warp calls it; the answer is uniform over the
+// grid.  B <= 128 here.
+constexpr int kCoKeys = 32, kCoRows = 64;   // keys per tile, query rows per CTA
+__device__ __forceinline__ bool attention_beside_lm_head(const AttnParams& p) {
+  int longest = 0, total = 0;
+  for (int q = threadIdx.x & 31; q < p.B; q += 32) {
+    const int n = min(max(p.cu_nodes[q + 1] - p.cu_nodes[q], 0), kMaxNodes);
+    const int ctx = min(max(p.ctx_len[q], 0), p.ctx_max);
+    const int tree = (n + kCoKeys - 1) / kCoKeys;
+    const int tiles = (ctx + kCoKeys - 1) / kCoKeys;
+    longest = max(longest, (tiles + p.n_parts - 1) / p.n_parts + tree);
+    // a share per SM (rounded up per sequence): far from overflow
+    const long long work = static_cast<long long>((n * p.G + kCoRows - 1) / kCoRows) * p.Hkv *
+                           (tiles + tree);
+    total += static_cast<int>(min((work + p.nsm - 1) / p.nsm, 1LL << 20));
+  }
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  total = __reduce_add_sync(0xffffffffu, total);
+  return max(longest, total) <= p.co_tiles;
+}
 // bf16 path: tensor-core (mma.sync) split-KV kernel fed by TMA; tm_k / tm_v are
 // 2D tensor maps over the context cache rows (box 64 columns x
 // min(attention_keys_per_tile(), rows per page) rows).
@@ -95,6 +122,10 @@ cudaError_t launch_attention_bf16(const AttnParams& p, const CUtensorMap& tm_k,
                                   const CUtensorMap& tm_v, cudaStream_t s);
 cudaError_t launch_attention_f32(const AttnParams& p, cudaStream_t s);
 int attention_row_blocks(int max_nodes, int G);
+// Key tiles of the busiest SM of the kernel beside the LM head, for contexts of
+// the cache's capacity, and up to how many of them it is the faster choice.
+long long attention_co_tiles_max(const asd_dims& d, int n_parts, int nsm);
+int attention_co_tiles_limit(const asd_dims& d);
 int attention_keys_per_tile();   // context keys per K/V tile = TMA box rows
 // bf16 path on the 5th-generation tensor cores, where attention has the SMs to
 // itself (a standalone call, or a step of more than 128 tree nodes): one CTA

@@ -146,3 +146,30 @@ def test_split_batch_with_a_malformed_sequence():
     out = _call(d, dims, ws)
     assert asd.asd_get_device_status(ws) == 3
     _check_close(out[:n], good[:n].float())
+
+
+# contexts short enough for the kernel beside the LM head and too long for it,
+# in the same cache of 24576 slots (small LM head: the limit is 16 key tiles of
+# 32 keys on the busiest SM)
+@pytest.mark.parametrize("ctx", [[0, 5], [300, 1500], [20000, 40], [24000, 23999], [1, 24500]])
+@pytest.mark.parametrize("D,page,nodes", [(128, 0, 40), (64, 16, 9)])
+@pytest.mark.parametrize("lazy", [False, True])
+def test_small_steps_choose_their_attention_by_context(ctx, D, page, nodes, lazy):
+    import torch
+    from paper_2609_02897_gb300 import asd
+    B, Hq, Hkv, cap, hidden, vocab = 2, 16, 4, 24576, 64, 200
+    d = _inputs(B, nodes, ctx, page, Hq, Hkv, D, cap, 7)
+    g = torch.Generator(device="cuda").manual_seed(9)
+    d["hidden"] = torch.randn(B * nodes, hidden, generator=g, device="cuda").to(torch.bfloat16)
+    d["w_lm"] = torch.randn(vocab, hidden, generator=g, device="cuda").to(torch.bfloat16)
+    d["tokens"] = torch.randint(0, vocab, (B * nodes,), generator=g, device="cuda").int()
+    dims = asd.make_dims(B, Hq, Hkv, D, hidden, vocab, asd.ASD_BF16, page, cap,
+                         B * cap // page if page else 0, nodes, 8,
+                         lm_head_schedule=1 if lazy else 0)
+    step = asd.VerifyStep(dims, B * nodes).bind(tau=0.5, **d)
+    ref = _reference(d, B, nodes, ctx, page, Hq, Hkv, D)
+    for _ in range(2):
+        step.out["attn_out"].fill_(float("nan"))
+        out = step.run()["attn_out"]
+        assert step.device_status() == 0
+        _check_close(out, ref)
