@@ -163,7 +163,7 @@ __device__ __forceinline__ int sequence_of_rank(const AttnParams& p, int r, int*
 }
 
 constexpr int kMaxChunks = 32;   // chunks per sequence: one lane of the merging warp each
-constexpr float kMergeOverhead = 3.f;   // cost of the merge in key tiles of ~1 us
+constexpr int kMergeOverhead = 3;   // cost of the merge in key tiles of ~1 us
 
 // Shared-memory scratch of make_item, one entry per sequence.
 struct PlanSmem {
@@ -172,12 +172,14 @@ struct PlanSmem {
   int items[kOrderMax];    // query row blocks x KV heads, then CTAs
   int key[kOrderMax];      // key tiles of the longest chunk
   int part[kOrderMax];     // partial rows (0: one chunk)
-  float cost[kMaxChunks];  // of cutting the longest sequence into 1, 2, ... chunks
+  int chunks[kOrderMax];
+  int cut_ctas[kMaxChunks];   // CTAs and partial rows when the longest sequence is
+  int cut_part[kMaxChunks];   // cut into 1, 2, ... chunks
   int seq, first, part0;   // the sequence of this CTA, its first CTA and partial row
 };
 
-// ceil(t / len) for 0 <= t from inv ~ 1 / len, for quotients up to kMaxChunks
-// (the estimate is then off by one at most).
+// ceil(t / len) and a / b for quotients up to about 2^12, from an approximate
+// reciprocal (the estimate is then off by one at most).
 __device__ __forceinline__ int ceil_div_est(int t, int len, float inv) {
   int c = static_cast<int>(static_cast<float>(t) * inv);
   c -= (c - 1) * len >= t ? 1 : 0;
@@ -185,15 +187,24 @@ __device__ __forceinline__ int ceil_div_est(int t, int len, float inv) {
   c += c * len < t ? 1 : 0;
   return c;
 }
+__device__ __forceinline__ int div_est(int a, int b) {
+  int q = static_cast<int>(static_cast<float>(a) * __frcp_rn(static_cast<float>(b)));
+  q -= q * b > a ? 1 : 0;
+  q += (q + 1) * b <= a ? 1 : 0;
+  return q;
+}
 
-// Key tiles per chunk.  Warp w weighs cutting the longest sequence into w + 1,
-// w + 1 + warps, ... chunks (and the others into chunks no longer than its),
-// its lanes summing over the sequences.  The chunks run at once, one CTA per
-// SM (a second wave would pay a CTA's overhead again), so a step takes its
-// longest chunk: the shortest length that fits, unless the merge costs more
-// than the cut saves.  Every thread of the CTA calls it (it synchronises the
-// CTA) and returns the same length.
+// Key tiles per chunk.  Lane k weighs cutting the longest sequence into k + 1
+// chunks (and the others into chunks no longer than its), each warp adding up
+// some of the sequences.  The chunks run at once, one CTA per SM (a second wave
+// would pay a CTA's overhead again), so a step takes its longest chunk: the
+// shortest length that fits, unless the merge costs more than the cut saves.
+// Every thread of the CTA calls it (it synchronises the CTA) and returns the
+// same length; s.cut_* are zero on entry.  It stands between the start of every
+// CTA and its first copy: 1.0 us (1.9 with three candidates per warp, a lane per
+// sequence).
 __device__ __forceinline__ int chunk_length(const AttnParams& p, PlanSmem& s) {
+  static_assert(kMaxChunks == 32, "a lane per candidate");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int longest = 1, items = 0;
   for (int q = lane; q < p.B; q += 32) {
@@ -203,31 +214,27 @@ __device__ __forceinline__ int chunk_length(const AttnParams& p, PlanSmem& s) {
   longest = __reduce_max_sync(0xffffffffu, longest);
   items = __reduce_add_sync(0xffffffffu, items);
   if (items == 0 || items > p.nsm) return longest;   // uniform over the CTA
-  for (int k = warp; k < kMaxChunks; k += kThreads / 32) {
-    const int len = (longest + k) / (k + 1);
-    const float inv = 1.f / static_cast<float>(len);
-    int ctas = 0, part = 0;
-    for (int q = lane; q < p.B; q += 32) {
-      const int c = ceil_div_est(s.tiles[q], len, inv);
-      ctas += s.items[q] * c;
-      part += c > 1 ? s.n[q] * p.Hq * c : 0;
-    }
-    ctas = __reduce_add_sync(0xffffffffu, ctas);
-    part = __reduce_add_sync(0xffffffffu, part);
-    // one chunk each (k = 0) is always possible
-    if (lane == 0)
-      s.cost[k] = k > 0 && (part > p.part_cap || ctas > p.nsm)
-                      ? INFINITY
-                      : static_cast<float>(len) + (part > 0 ? kMergeOverhead : 0.f);
+  const int len = (longest + lane) / (lane + 1);
+  const float inv = __frcp_rn(static_cast<float>(len));
+  int ctas = 0, part = 0;
+  for (int q = warp; q < p.B; q += kThreads / 32) {
+    const int c = ceil_div_est(s.tiles[q], len, inv);
+    ctas += s.items[q] * c;
+    part += c > 1 ? s.n[q] * p.Hq * c : 0;
+  }
+  if (warp < p.B) {
+    atomicAdd(&s.cut_ctas[lane], ctas);
+    atomicAdd(&s.cut_part[lane], part);
   }
   __syncthreads();
-  static_assert(kMaxChunks == 32, "a lane per candidate");
-  const float cost = s.cost[lane];
-  float best = cost;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-  const int k = __ffs(__ballot_sync(0xffffffffu, cost == best)) - 1;
-  return (longest + k) / (k + 1);
+  ctas = s.cut_ctas[lane];
+  part = s.cut_part[lane];
+  // one chunk each (lane 0) is always possible
+  const unsigned cost = lane > 0 && (part > p.part_cap || ctas > p.nsm)
+                            ? 0xffffffffu
+                            : static_cast<unsigned>(len + (part > 0 ? kMergeOverhead : 0));
+  const unsigned best = __reduce_min_sync(0xffffffffu, cost);
+  return __shfl_sync(0xffffffffu, len, __ffs(__ballot_sync(0xffffffffu, cost == best)) - 1);
 }
 
 // The chunk of CTA blockIdx.x: sequences in decreasing order of their chunks'
@@ -236,7 +243,7 @@ __device__ __forceinline__ int chunk_length(const AttnParams& p, PlanSmem& s) {
 // none.  Every thread of the CTA calls it (it synchronises the CTA).
 __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSmem& s) {
   const int idx = blockIdx.x;
-  int local, ctx;
+  int local, ctx, longest;   // longest: key tiles of the sequence's longest chunk
   if (p.B > kOrderMax) {   // index order, unsplit
     const int rbmax = (p.max_nodes * p.G + kRows - 1) / kRows;
     it.b = idx / (rbmax * p.Hkv);
@@ -253,11 +260,13 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
     it.s0 = p.cu_nodes[it.b];
     it.n = p.cu_nodes[it.b + 1] - it.s0;
     ctx = min(max(p.ctx_len[it.b], 0), p.ctx_max);
+    longest = 0x3fffffff;
     __syncthreads();
   } else {
     // sequence extents and context lengths are caller inputs (the tree
     // preparation reports bad ones): a malformed sequence gets no CTA
     if (threadIdx.x == 0) s.seq = -1;
+    if (threadIdx.x < kMaxChunks) s.cut_ctas[threadIdx.x] = s.cut_part[threadIdx.x] = 0;
     for (int q = threadIdx.x; q < p.B; q += blockDim.x) {
       const int s0 = p.cu_nodes[q], n = p.cu_nodes[q + 1] - s0;
       const int c = min(max(p.ctx_len[q], 0), p.ctx_max);
@@ -269,14 +278,16 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
       s.items[q] = okq ? (n * p.G + kRows - 1) / kRows * p.Hkv : 0;
       s.key[q] = s.tiles[q];
       s.part[q] = 0;
+      s.chunks[q] = 1;
     }
     __syncthreads();
-    int len = 0x3fffffff;
     if (p.part_cap > 0) {
-      len = chunk_length(p, s);
+      const int len = chunk_length(p, s);
       __syncthreads();   // every warp has read s.items
+      const float inv = __frcp_rn(static_cast<float>(len));
       for (int q = threadIdx.x; q < p.B; q += blockDim.x) {
-        const int t = s.tiles[q], c = (t + len - 1) / len;
+        const int t = s.tiles[q], c = ceil_div_est(t, len, inv);
+        s.chunks[q] = c;
         if (c > 1) {
           s.items[q] *= c;
           s.key[q] = (t + c - 1) / c;
@@ -303,7 +314,7 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
         s.first = first;
         s.part0 = part;
         if (idx == first && p.part_cap > 0)
-          p.plan[q] = make_int2(part, (s.tiles[q] + len - 1) / len);
+          p.plan[q] = make_int2(part, s.chunks[q]);
       }
     }
     __syncthreads();
@@ -312,22 +323,27 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
     it.s0 = s.s0[it.b];
     it.n = s.n[it.b];
     ctx = s.ctx[it.b];
-    it.chunks = s.part[it.b] > 0 ? (s.tiles[it.b] + len - 1) / len : 1;
+    it.chunks = s.chunks[it.b];
     it.part0 = s.part0;
     const int rb = (it.n * p.G + kRows - 1) / kRows;
     local = idx - s.first;
-    const int gz = local / rb;
+    const int gz = div_est(local, rb);
     it.r0 = (local - gz * rb) * kRows;
-    it.g = gz / it.chunks;
+    it.g = div_est(gz, it.chunks);
     it.chunk = gz - it.g * it.chunks;
+    longest = s.key[it.b];
   }
   it.R = it.n * p.G;
   if (it.n <= 0 || it.n > kMaxNodes || it.s0 < 0 || it.s0 + it.n > p.T || it.r0 >= it.R)
     return false;
   it.nrows = min(kRows, it.R - it.r0);
   const int nctx = (ctx + kKeys - 1) / kKeys, all = nctx + (it.n + kKeys - 1) / kKeys;
-  // chunk z: tiles [z all / chunks, (z + 1) all / chunks) of the context's, then the tree's
-  const int t0 = it.chunk * all / it.chunks, t1 = (it.chunk + 1) * all / it.chunks;
+  // of the context's tiles, then the tree's, the first chunks take one more
+  // than the others where they do not divide
+  const int few = it.chunks == 1 ? all : (longest * it.chunks == all ? longest : longest - 1);
+  const int more = all - few * it.chunks;
+  const int t0 = it.chunk * few + min(it.chunk, more);
+  const int t1 = t0 + few + (it.chunk < more ? 1 : 0);
   it.ntiles = t1 - t0;
   it.nctx = min(t1, nctx) - t0;
   it.ntree = it.ntiles - it.nctx;
@@ -835,46 +851,68 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();   // the tile buffers and the tensor cores are idle from here on
   tc_fence_after();
   if (warp >= 2 && warp < 10 && ok) {
-    // each thread writes its key half's share of the row, D/2 columns: the
-    // output, or (one of several chunks) the fp32 partial that
-    // attn_merge_kernel combines
+    // Each thread holds its key half's share of a row, D/2 columns: the output,
+    // or (one of several chunks) the fp32 partial that attn_merge_kernel
+    // combines.
     const int hf = (warp - 2) >> 2;
-    const int row = (warp & 3) * 32 + lane;   // TMEM lane = query row
-    const uint32_t lane_base = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) +
+    const int row0 = (warp & 3) * 32, row = row0 + lane;   // TMEM lane = query row
+    const uint32_t lane_base = tmem + (static_cast<uint32_t>(row0) << 16) +
                                static_cast<uint32_t>(hf * (D / 2));
     const bool mine = row < it.nrows;
-    const bool split = it.chunks > 1;
-    const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
-    __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.out) +
-                         (mine ? grow_of(p, it, row) : 0) * D + hf * (D / 2);
-    const size_t prow = mine && split ? static_cast<size_t>(it.part0) +
-                                            static_cast<size_t>(it.g * it.chunks + it.chunk) * it.R +
-                                            it.r0 + row
-                                      : 0;
-    if (mine && split && hf == 0) p.part_ml[prow] = make_float2(m_row, l_row);
+    if (it.chunks == 1) {
+      const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
+      __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.out) +
+                           (mine ? grow_of(p, it, row) : 0) * D + hf * (D / 2);
 #pragma unroll 1
-    for (int c = 0; c < D / 64; ++c) {
-      float o[32];
-      tmem_ld32(lane_base + 32 * c, o);   // every lane takes part in the warp-wide load
-      if (mine && split) {
-        float4* po = reinterpret_cast<float4*>(p.part_o + prow * D + hf * (D / 2) + 32 * c);
+      for (int c = 0; c < D / 64; ++c) {
+        float o[32];
+        tmem_ld32(lane_base + 32 * c, o);   // every lane takes part in the warp-wide load
+        if (mine) {
+#pragma unroll
+          for (int k = 0; k < 32; k += 8) {
+            uint4 pk;
+            __nv_bfloat162 h0 = __floats2bfloat162_rn(o[k] * inv, o[k + 1] * inv);
+            __nv_bfloat162 h1 = __floats2bfloat162_rn(o[k + 2] * inv, o[k + 3] * inv);
+            __nv_bfloat162 h2 = __floats2bfloat162_rn(o[k + 4] * inv, o[k + 5] * inv);
+            __nv_bfloat162 h3 = __floats2bfloat162_rn(o[k + 6] * inv, o[k + 7] * inv);
+            pk.x = *reinterpret_cast<uint32_t*>(&h0);
+            pk.y = *reinterpret_cast<uint32_t*>(&h1);
+            pk.z = *reinterpret_cast<uint32_t*>(&h2);
+            pk.w = *reinterpret_cast<uint32_t*>(&h3);
+            *reinterpret_cast<uint4*>(out + 32 * c + k) = pk;
+          }
+        }
+      }
+    } else if (row0 < it.nrows) {
+      // Written by the lanes that hold them, the partials' 16-byte stores would
+      // touch 32 rows each; turned through shared memory (the tile buffers are
+      // free), eight lanes write 128 consecutive bytes: 2.6 -> 1.6 us for a
+      // CTA's 128 rows of 128 columns.  (The bf16 output, half the bytes, is
+      // faster as it is: 0.6 us against 1.4 for 32 rows.)
+      const size_t prow = static_cast<size_t>(it.part0) +
+                          static_cast<size_t>(it.g * it.chunks + it.chunk) * it.R + it.r0 + row0;
+      if (mine && hf == 0) p.part_ml[prow + lane] = make_float2(m_row, l_row);
+      constexpr int kStLd = 36;   // padded row of 32 columns
+      float* stg = reinterpret_cast<float*>(gbase) + (warp - 2) * 32 * kStLd;
+#pragma unroll 1
+      for (int c = 0; c < D / 64; ++c) {
+        float o[32];
+        tmem_ld32(lane_base + 32 * c, o);
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          po[k] = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
-      } else if (mine) {
+          *reinterpret_cast<float4*>(stg + lane * kStLd + 4 * k) =
+              make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+        __syncwarp();
+        const int col = 4 * (lane & 7);
+        float* po = p.part_o + prow * D + hf * (D / 2) + 32 * c + col;
 #pragma unroll
-        for (int k = 0; k < 32; k += 8) {
-          uint4 pk;
-          __nv_bfloat162 h0 = __floats2bfloat162_rn(o[k] * inv, o[k + 1] * inv);
-          __nv_bfloat162 h1 = __floats2bfloat162_rn(o[k + 2] * inv, o[k + 3] * inv);
-          __nv_bfloat162 h2 = __floats2bfloat162_rn(o[k + 4] * inv, o[k + 5] * inv);
-          __nv_bfloat162 h3 = __floats2bfloat162_rn(o[k + 6] * inv, o[k + 7] * inv);
-          pk.x = *reinterpret_cast<uint32_t*>(&h0);
-          pk.y = *reinterpret_cast<uint32_t*>(&h1);
-          pk.z = *reinterpret_cast<uint32_t*>(&h2);
-          pk.w = *reinterpret_cast<uint32_t*>(&h3);
-          *reinterpret_cast<uint4*>(out + 32 * c + k) = pk;
+        for (int i = 0; i < 8; ++i) {
+          const int r = 4 * i + (lane >> 3);
+          if (row0 + r < it.nrows)
+            *reinterpret_cast<float4*>(po + static_cast<size_t>(r) * D) =
+                *reinterpret_cast<const float4*>(stg + r * kStLd + col);
         }
+        __syncwarp();
       }
     }
   }
