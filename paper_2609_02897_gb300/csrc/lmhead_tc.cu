@@ -325,15 +325,15 @@ __global__ void __launch_bounds__(192, 1)
 // the epilogue has drained it.
 //
 // CL = 2: the CTAs come in clusters of two that own two adjacent vocabulary
-// ranges together and take alternate node pairs.  Each CTA copies one of the
-// two 128-row halves of every W stage and multicasts it to both, so every SM
-// pulls 48 KB per stage instead of 64 and W crosses HBM once per four node
-// tiles.  A stage is refilled only after both CTAs' MMAs have read it (each
-// CTA's commit arrives on both CTAs' empty barriers); both CTAs run the same
-// sequence of stages, a CTA without a node pair in the last round still
-// copying its half.  Every thread keeps one running state per vocabulary
-// range and writes one partial per range, so the statistics are those of
-// CTAs that own one range each, bit for bit.
+// ranges together and share out the node tiles, four in a round (wide_slot).
+// Each CTA copies one of the two 128-row halves of every W stage and multicasts
+// it to both, so every SM pulls 48 KB per stage instead of 64 and W crosses HBM
+// once per four node tiles.  A stage is refilled only after both CTAs' MMAs have
+// read it (each CTA's commit arrives on both CTAs' empty barriers); both CTAs
+// run the same sequence of stages, a CTA without a node tile for a stage still
+// copying its half.  Every thread keeps one running state per vocabulary range
+// and writes one partial per range, so the statistics are those of CTAs that
+// own one range each, bit for bit.
 //
 // Warp roles (352 threads): warp 0 TMA producer, warp 1 TMEM allocator and
 // MMA issuer for node tile 0 of every pair, warp 10 MMA issuer for node tile
@@ -427,6 +427,64 @@ struct WideVocab {
   }
 };
 
+// How the node tiles are shared out in rounds.  CL = 1: two tiles in a round.
+// CL = 2: four tiles in a round, two per CTA; of what is left at the end
+//   three  go one to each CTA, the third computed on range 0 by the one and on
+//          range 1 by the other: three tiles' MMAs where two pairs, one of them
+//          half empty, took four (the stages' round trip bounds a round more
+//          than its MMAs do: 384 nodes 330 -> 326 us at W 128256 x 4096, 102 ->
+//          97 at 32000 x 4096);
+//   two    go one to each CTA, not both to one (1280 nodes 991 -> 940 us and
+//          279 -> 257);
+//   one    goes to the first CTA.
+template <int CL>
+struct WideRounds {
+  int nnt, rounds;
+  __device__ __forceinline__ explicit WideRounds(int tiles)
+      : nnt(tiles), rounds((tiles + 2 * CL - 1) / (2 * CL)) {}
+  // Node tile of slot j (0, 1) of the CTA of rank `rank` in round `it`, or -1;
+  // only: the one range it is computed for, or -1 (all of the CTA's).
+  __device__ __forceinline__ int slot(int it, int j, int rank, int& only) const {
+    only = -1;
+    const int first = 2 * CL * it, left = nnt - first;
+    if (CL == 1) return j < left ? first + j : -1;
+    if (left >= 4) return first + 2 * rank + j;
+    if (j == 0) return rank < left ? first + rank : -1;
+    if (left < 3) return -1;
+    only = rank;
+    return first + 2;
+  }
+};
+
+// The accumulators (256 TMEM columns each) of a CTA's two slots, tracked alike
+// by the MMA issuers and the epilogue.  Where a round has both slots, slot j's
+// tiles go to accumulator j, whose issuer and epilogue group then see every
+// phase of its barriers.  A round with slot 0 alone alternates between the two,
+// so that one tile's drain overlaps the next tile's MMAs; its threads then wait
+// for phases of the other slot's barriers, which is sound while the two issuers
+// are within one tile of each other (a tile of at least kWideStages + 1 stages).
+struct WideAcc {
+  int cnt0 = 0, cnt1 = 0, flip = 0;   // uses so far of either accumulator
+  bool may_flip;
+  __device__ __forceinline__ explicit WideAcc(int nkb) : may_flip(nkb > 3) {}
+  // accumulator of slot j, `use`: how often it was used before
+  __device__ __forceinline__ int of(int j, bool two, int& use) const {
+    const int acc = j == 1 ? 1 : (two ? 0 : flip);
+    use = acc ? cnt1 : cnt0;
+    return acc;
+  }
+  __device__ __forceinline__ void next(bool two, bool has0, bool has1) {
+    if (two) {
+      cnt0 += has0 ? 1 : 0;
+      cnt1 += has1 ? 1 : 0;
+    } else if (has0) {
+      if (flip) ++cnt1;
+      else ++cnt0;
+      if (may_flip) flip ^= 1;
+    }
+  }
+};
+
 template <int CL>
 __global__ void __launch_bounds__(kWideThreads, 1)
     lmhead_wide_kernel(const __grid_constant__ LmMaps maps, const LmParams p) {
@@ -466,8 +524,8 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   voc.nt1 = (voc.ge1 - voc.gs1 + kTileGroups - 1) / kTileGroups;
   voc.ntiles = voc.nt0 + voc.nt1;
   const int nnt = (nrow + kM - 1) / kM;                  // node tiles
-  const int nng = (nnt + kWideG - 1) / kWideG;           // node-tile pairs
-  const int nit = (nng + CL - 1) / CL;                   // rounds: pair i*CL + rank in round i
+  const WideRounds<CL> rounds(nnt);
+  const int nit = rounds.rounds;
   const int nkb = (p.K + kKB - 1) / kKB;
 
   uint32_t base = smem_u32(smem_raw);
@@ -507,6 +565,10 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   // 256-row vocabulary tiles (pairs of packed tiles); none when a packed
   // weight does not match (both CTAs of a cluster read the same header)
   const int nvt = s_pack_bad ? 0 : (voc.ntiles + 1) / 2;
+  // whether 256-row tile vt holds rows of range `only` (-1: any range)
+  auto covers = [&](int vt, int only) -> bool {
+    return only < 0 || (only == 0 ? 2 * vt < voc.nt0 : 2 * vt + 1 >= voc.nt0);
+  };
   // a wait that gives up stops this CTA and its peer
   auto abort_cta = [&]() {
     note_timeout(p.status);
@@ -531,9 +593,13 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     uint32_t ph = 0;
     bool ok = true;
     for (int it = 0; it < nit && ok; ++it) {
-      const int pi = it * CL + rank;                       // this CTA's node pair
-      const int gn = pi < nng ? min(kWideG, nnt - pi * kWideG) : 0;
+      int only[kWideG], tile[kWideG];                      // this CTA's node tiles
+#pragma unroll
+      for (int j = 0; j < kWideG; ++j) tile[j] = rounds.slot(it, j, rank, only[j]);
       for (int vt = 0; vt < nvt && ok; ++vt) {
+        bool has[kWideG];
+#pragma unroll
+        for (int j = 0; j < kWideG; ++j) has[j] = tile[j] >= 0 && covers(vt, only[j]);
         int q[2], g0[2], ng[2], v0[2], rows[2];
         int wbytes = 0;
 #pragma unroll
@@ -556,10 +622,12 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             const uint32_t a_s = base + stage * kWideSlot;
             const uint32_t b_s = a_s + kWideG * kWideA;
             // every W byte of the stage lands here (half of it from the peer)
-            mbar_expect_tx(full, static_cast<uint32_t>(gn * kWideA + wbytes));
-            for (int j = 0; j < gn; ++j)
-              tma_load_2d(a_s + j * kWideA, &maps.h, full, kb * kKB, (pi * kWideG + j) * kM,
-                          pol_h);
+            mbar_expect_tx(full, static_cast<uint32_t>(((has[0] ? 1 : 0) + (has[1] ? 1 : 0)) * kWideA +
+                                                       wbytes));
+#pragma unroll
+            for (int j = 0; j < kWideG; ++j)
+              if (has[j])
+                tma_load_2d(a_s + j * kWideA, &maps.h, full, kb * kKB, tile[j] * kM, pol_h);
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
               if (ng[hf] == 0 || (CL == 2 && hf != rank)) continue;   // the peer's half
@@ -611,26 +679,27 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     // ------------------------------------------------------------ MMA issuers
     // Two issuing threads, one per node tile of the pair (warp 1: tile 0,
     // warp 10: tile 1), so that the one's barrier waits overlap the other's
-    // MMAs.  Both read every stage and both release it.  Accumulator use u
-    // (counted over the kernel) goes to TMEM buffer u % 2; its empty barrier
-    // completes once per lap.
+    // MMAs.  Both read every stage and both release it.
     const int j = warp == 1 ? 0 : 1;
     int stage = 0;
     uint32_t ph = 0;
-    int used = 0;
+    WideAcc accs(nkb);
     bool ok = true;
     for (int it = 0; it < nit && ok; ++it) {
-      const int pi = it * CL + rank;
-      const int gn = pi < nng ? min(kWideG, nnt - pi * kWideG) : 0;
+      int only0, only1;
+      const int tile0 = rounds.slot(it, 0, rank, only0);
+      const int tile1 = rounds.slot(it, 1, rank, only1);
       for (int vt = 0; vt < nvt && ok; ++vt) {
+        const bool has0 = tile0 >= 0 && covers(vt, only0), has1 = tile1 >= 0 && covers(vt, only1);
+        const bool mine = j == 0 ? has0 : has1;
         // N covers the low half's rows, or all 128 of them and the high half's
         int q, g0, ng, v0, rows_lo, rows_hi = 0;
         voc.tile(2 * vt, p.V, q, g0, ng, v0, rows_lo);
         if (2 * vt + 1 < voc.ntiles) voc.tile(2 * vt + 1, p.V, q, g0, ng, v0, rows_hi);
         const int ncols = rows_hi > 0 ? kLmTileN + rows_hi : rows_lo;
         const uint32_t idesc = idesc_bf16(kM, (ncols + 15) & ~15);
-        const int u = used + j;
-        const int acc = u % kWideG;
+        int use;
+        const int acc = accs.of(j, tile1 >= 0, use);
         for (int kb = 0; kb < nkb && ok; ++kb) {
           ok = __shfl_sync(0xffffffffu, mbar_wait(smem_u32(&s_full[stage]), ph, budget), 0);
           if (!ok || s_abort) {
@@ -640,13 +709,12 @@ __global__ void __launch_bounds__(kWideThreads, 1)
           tc_fence_after();
           const uint32_t a_s = base + stage * kWideSlot;
           const uint32_t b_s = a_s + kWideG * kWideA;
-          if (j < gn) {
+          if (mine) {
             if (kb == 0) {
               // the epilogue must have drained this buffer's previous tile
               ok = __shfl_sync(
                   0xffffffffu,
-                  mbar_wait(smem_u32(&s_tempty[acc]), ((static_cast<uint32_t>(u / kWideG)) & 1u) ^ 1u,
-                            budget),
+                  mbar_wait(smem_u32(&s_tempty[acc]), (static_cast<uint32_t>(use) & 1u) ^ 1u, budget),
                   0);
               if (!ok || s_abort) {
                 ok = false;
@@ -678,7 +746,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             ph ^= 1u;
           }
         }
-        used += gn;
+        accs.next(tile1 >= 0, has0, has1);
       }
     }
     if (!ok && lane == 0) abort_cta();
@@ -691,34 +759,36 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     __syncwarp();
   } else {
     // ----------------------------------------------------------------- epilogue
-    // Two groups of four warps: group g drains the accumulator of node tile
-    // j = g of the current pair, so both accumulators of a vocabulary tile
+    // Two groups of four warps: group g drains the accumulators of the CTA's
+    // node tile slot g, so both accumulators of a vocabulary tile
     // drain at once.  Thread `row` of a group owns TMEM lane `row`: row `row`
     // of its node tile, one running state per vocabulary range.
     const int q4 = warp & 3;
     const int row = q4 * 32 + lane;
     const int g = (warp - 2) >> 2;
     pdl_wait();
-    int used = 0;
+    WideAcc accs(nkb);
     bool ok = true;
     for (int it = 0; it < nit && ok; ++it) {
-      const int pi = it * CL + rank;
-      const int gn = pi < nng ? min(kWideG, nnt - pi * kWideG) : 0;
-      const int r = (pi * kWideG + g) * kM + row;
-      const int node = (g < gn && r < nrow && p.row_node) ? p.row_node[r] : r;
-      const bool act = g < gn && r < nrow && node >= 0 && node < p.T;
+      int only0, only1;
+      const int tile0 = rounds.slot(it, 0, rank, only0);
+      const int tile1 = rounds.slot(it, 1, rank, only1);
+      const int tile = g == 0 ? tile0 : tile1, only = g == 0 ? only0 : only1;
+      const int r = tile * kM + row;
+      const int node = (tile >= 0 && r < nrow && p.row_node) ? p.row_node[r] : r;
+      const bool act = tile >= 0 && r < nrow && node >= 0 && node < p.T;
       RowState st[CL];
 #pragma unroll
       for (int qq = 0; qq < CL; ++qq)
         row_state_init(st[qq], act, node, (qq ? voc.gs1 : voc.gs0) * kLmBoxRows, p.child_start,
                        p.child_cnt, p.child_tok, p.T);
       for (int vt = 0; vt < nvt && ok; ++vt) {
-        if (g < gn) {
-          const int u = used + g;
-          const int acc = u % kWideG;
+        const bool has0 = tile0 >= 0 && covers(vt, only0), has1 = tile1 >= 0 && covers(vt, only1);
+        if (g == 0 ? has0 : has1) {
+          int use;
+          const int acc = accs.of(g, tile1 >= 0, use);
           ok = __shfl_sync(0xffffffffu,
-                           mbar_wait(smem_u32(&s_tfull[acc]), (static_cast<uint32_t>(u / kWideG)) & 1u,
-                                     budget),
+                           mbar_wait(smem_u32(&s_tfull[acc]), static_cast<uint32_t>(use) & 1u, budget),
                            0);
           if (!ok || s_abort) {
             ok = false;
@@ -733,6 +803,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             if (2 * vt + hf >= voc.ntiles) break;
             int q, g0, ng, v0, rows;
             voc.tile(2 * vt + hf, p.V, q, g0, ng, v0, rows);
+            if (CL == 2 && only >= 0 && q != only) continue;   // the other CTA's
             for (int c = 0; c < rows; c += 64) {
               float x[64];
               tmem_ld64(taddr + hf * kLmTileN + c, x);
@@ -757,11 +828,12 @@ __global__ void __launch_bounds__(kWideThreads, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive(smem_u32(&s_tempty[acc]));
         }
-        used += gn;
+        accs.next(tile1 >= 0, has0, has1);
       }
-      if (ok && g < gn && r < nrow) {   // partials by row, one per range
+      if (ok && tile >= 0 && r < nrow) {   // partials by row, one per range
 #pragma unroll
         for (int qq = 0; qq < CL; ++qq) {
+          if (only >= 0 && qq != only) continue;
           LmPartial part;
           part.m = st[qq].m;
           part.s = st[qq].s;
@@ -911,15 +983,15 @@ int lmhead_bf16_variant(const LmParams& p) {
   // several node tiles, or a row count known on the device only: the wide
   // kernel (full 128-row node boxes).  Clusters of two halve the W traffic
   // (each W stage is read once per cluster) and move their CTAs in lock step
-  // through the rounds of node pairs, so they pay unless that lock step leaves
-  // one CTA idle for a large share of the work: with three pairs the CTA
-  // without a pair in the second round idles for half of it (measured with
-  // two MMA-issuing threads: two pairs 430 -> 393 us on the Qwen3-8B B8
-  // workload, four and more pairs 10 % faster).  The ranges must pair up, and
-  // the W multicast reads this GPU's own memory only: a weight elsewhere
-  // (host or another device) runs unclustered.
-  const int pairs = (p.T + kWideG * kM - 1) / (kWideG * kM);
-  return (p.g_lm % 2 == 0 && !p.t_dev && (pairs == 2 || pairs >= 4) && p.w_local) ? 3 : 2;
+  // through the rounds of node tiles.  The ranges must pair up, and the W
+  // multicast reads this GPU's own memory only: a weight elsewhere (host or
+  // another device) runs unclustered.
+  const int tiles = (p.T + kM - 1) / kM;
+  if (p.g_lm % 2 != 0 || p.t_dev || !p.w_local) return 2;
+  // W of 128256 x 4096, a cluster's round against unclustered ones: four tiles
+  // 337 us (393), three 326 (366), two 257 (199: a CTA then has only half a
+  // stage of W in flight), so clusters for three, four and from seven tiles on.
+  return tiles == 3 || tiles == 4 || tiles >= 7 ? 3 : 2;
 }
 
 cudaError_t launch_lmhead_bf16(const LmParams& p, const LmMaps& maps, cudaStream_t s) {
