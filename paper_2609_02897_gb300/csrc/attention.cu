@@ -17,6 +17,7 @@
 // peers' partials through distributed shared memory.  No partial leaves the
 // cluster.
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -553,8 +554,9 @@ __global__ void __launch_bounds__(128) attn_bf16_kernel(const __grid_constant__ 
 // scores by 16 x 16 threads (row, key), the online softmax by a warp per row
 // with a lane per key, P V by threads that own 4 columns of up to 64 rows.  With
 // a warp per row walking K and V in global memory, a load at a time per key, the
-// tiny fp32 workload's kernel took 42.6 us (profiled; now 15.6), nearly all of it
-// load latency.
+// tiny fp32 workload's kernel took 42.6 us (profiled), nearly all of it load
+// latency; with row tests inside the tile loops a tile still took 4 us, now 2.
+// Tiny fp32 step, on the GPU: 73 -> 18 us with the fp32 LM head, which it overlaps.
 constexpr int kF32Threads = 256;
 
 template <int D>
@@ -611,37 +613,35 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const AttnParams 
   const int nkeys = nctx_keys + (kr.ntree > 0 ? n : 0);
   const int ntiles = (nkeys + kKeysPerTile - 1) / kKeysPerTile;
 
-  // K and V rows of keys [32 t, 32 t + 32) of the split; a key past the end or
-  // on a bad page reads as zeros and takes no part
+  // K and V rows of keys [32 t, 32 t + 32) of the split, D/4 threads side by
+  // side on a row; a key past the end or on a bad page reads as zeros and takes
+  // no part
+  const int ps_shift = 31 - __clz(max(ps, 1));   // pages are a power of two
   auto load = [&](int t) {
     const int stage = t & 1;
-    for (int i = tid; i < kKeysPerTile * (D / 4); i += kF32Threads) {
-      const int j = i / (D / 4), ch = i - j * (D / 4);
+#pragma unroll
+    for (int i = 0; i < kKeysPerTile * (D / 4) / kF32Threads; ++i) {
+      const int j = tid / (D / 4) + i * (kF32Threads / (D / 4)), ch = tid % (D / 4);
       const int u = t * kKeysPerTile + j;
-      long long off = -1;
-      int seen = 0;
-      if (u >= nctx_keys && u < nkeys) {
-        const int node = u - nctx_keys;
-        off = (static_cast<long long>(s0 + node) * p.Hkv + g) * D;
-        seen = 2 + node;
-      } else if (u < nctx_keys) {
+      const bool tree = u >= nctx_keys;
+      long long row = -1;   // K / V row of the key
+      if (tree) {
+        if (u < nkeys) row = static_cast<long long>(s0 + u - nctx_keys) * p.Hkv + g;
+      } else if (ps == 0) {
+        row = (static_cast<long long>(b) * p.Hkv + g) * p.ctx_max + kr.kbeg + u;
+      } else {
         const int key = kr.kbeg + u;
-        if (ps == 0) {
-          off = ((static_cast<long long>(b) * p.Hkv + g) * p.ctx_max + key) * D;
-        } else {
-          const int page = p.page_table[static_cast<size_t>(b) * p.pages_per_seq + key / ps];
-          if (page < 0 || page >= p.num_pages)
-            set_status(p.status, ASD_ERR_CTX_RANGE);
-          else
-            off = ((static_cast<long long>(page) * p.Hkv + g) * ps + key % ps) * D;
-        }
-        seen = off >= 0 ? 1 : 0;
+        const int page = p.page_table[static_cast<size_t>(b) * p.pages_per_seq + (key >> ps_shift)];
+        if (page < 0 || page >= p.num_pages)
+          set_status(p.status, ASD_ERR_CTX_RANGE);
+        else
+          row = ((static_cast<long long>(page) * p.Hkv + g) << ps_shift) + (key & (ps - 1));
       }
-      const bool tree = u >= nctx_keys, in = off >= 0;
-      const long long at = in ? off + 4 * ch : 0;
+      const bool in = row >= 0;
+      const long long at = in ? row * D + 4 * ch : 0;
       copy16_async(smem_f + G::kK + stage * G::kTile + j * kLd + 4 * ch, (tree ? tk : kc) + at, in);
       copy16_async(smem_f + G::kV + stage * G::kTile + j * kLd + 4 * ch, (tree ? tv : vc) + at, in);
-      if (ch == 0) s_seen[stage][j] = seen;
+      if (ch == 0) s_seen[stage][j] = in ? (tree ? 2 + u - nctx_keys : 1) : 0;
     }
   };
 
@@ -666,48 +666,49 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const AttnParams 
   const int sr = tid >> 4, sk = tid & 15;    // scores: rows sr + 16 i, keys sk, sk + 16
   float* sP = smem_f + G::kP;
 
-  for (int t = 0; t < ntiles; ++t) {
+  // One key tile for the first 16 NR rows: no tests on the rows inside the
+  // loops, whose loads then run ahead of the arithmetic (a row past nrows works
+  // on whatever is there and is dropped).
+  auto tile = [&](int t, auto nr) {
+    constexpr int NR = decltype(nr)::value, kO = 16 * NR / kPr;
     const int stage = t & 1;
-    if (t + 1 < ntiles) load(t + 1);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();
     const float* sK = smem_f + G::kK + stage * G::kTile;
     const float* sV = smem_f + G::kV + stage * G::kTile;
     // scores, masked
-    float acc[4][2];
+    float acc[NR][2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0.f;
+    for (int i = 0; i < NR; ++i) acc[i][0] = acc[i][1] = 0.f;
 #pragma unroll 4
     for (int d = 0; d < D; d += 4) {
       const float4 k0 = *reinterpret_cast<const float4*>(sK + sk * kLd + d);
       const float4 k1 = *reinterpret_cast<const float4*>(sK + (sk + 16) * kLd + d);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (16 * i >= nrows) break;           // uniform over the CTA
-        // rows past nrows read what is there; their scores are not used
+      for (int i = 0; i < NR; ++i) {
         const float4 q = *reinterpret_cast<const float4*>(smem_f + G::kQ + (sr + 16 * i) * kLd + d);
         acc[i][0] = fmaf(q.x, k0.x, acc[i][0]);
-        acc[i][0] = fmaf(q.y, k0.y, acc[i][0]);
-        acc[i][0] = fmaf(q.z, k0.z, acc[i][0]);
-        acc[i][0] = fmaf(q.w, k0.w, acc[i][0]);
         acc[i][1] = fmaf(q.x, k1.x, acc[i][1]);
+        acc[i][0] = fmaf(q.y, k0.y, acc[i][0]);
         acc[i][1] = fmaf(q.y, k1.y, acc[i][1]);
+        acc[i][0] = fmaf(q.z, k0.z, acc[i][0]);
         acc[i][1] = fmaf(q.z, k1.z, acc[i][1]);
+        acc[i][0] = fmaf(q.w, k0.w, acc[i][0]);
         acc[i][1] = fmaf(q.w, k1.w, acc[i][1]);
       }
     }
+    const int seen0 = s_seen[stage][sk], seen1 = s_seen[stage][sk + 16];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < NR; ++i) {
       const int r = sr + 16 * i;
-      if (r >= nrows) break;
-      const int node = (r0 + r) / p.G;
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int seen = s_seen[stage][sk + 16 * e];
-        const bool vis = seen == 1 || (seen >= 2 && anc_bit(s_anc[node][0], s_anc[node][1], seen - 2));
-        sP[r * kPLd + sk + 16 * e] = vis ? acc[i][e] : -INFINITY;
+      uint64_t lo = 0, hi = 0;
+      if ((seen0 | seen1) > 1) {   // a tree key
+        const int node = (r0 + min(r, nrows - 1)) / p.G;
+        lo = s_anc[node][0];
+        hi = s_anc[node][1];
       }
+      const bool v0 = seen0 == 1 || (seen0 >= 2 && anc_bit(lo, hi, seen0 - 2));
+      const bool v1 = seen1 == 1 || (seen1 >= 2 && anc_bit(lo, hi, seen1 - 2));
+      sP[r * kPLd + sk] = v0 ? acc[i][0] : -INFINITY;
+      sP[r * kPLd + sk + 16] = v1 ? acc[i][1] : -INFINITY;
     }
     __syncthreads();
     // online softmax, a warp per row, lane = key
@@ -733,30 +734,40 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const AttnParams 
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kRows; ++i) {
-      if (pr + kPr * i >= nrows) break;
+    for (int i = 0; i < kO; ++i) {
       const float al = s_al[pr + kPr * i];
       o[i].x *= al;
       o[i].y *= al;
       o[i].z *= al;
       o[i].w *= al;
     }
-#pragma unroll 4
+#pragma unroll 8
     for (int j = 0; j < kKeysPerTile; ++j) {
       const float4 v = *reinterpret_cast<const float4*>(sV + j * kLd + 4 * pc);
 #pragma unroll
-      for (int i = 0; i < kRows; ++i) {
-        if (pr + kPr * i >= nrows) break;
+      for (int i = 0; i < kO; ++i) {
         const float w = sP[(pr + kPr * i) * kPLd + j];
-        if (w != 0.f) {   // a masked key's V may hold anything
-          o[i].x = fmaf(w, v.x, o[i].x);
-          o[i].y = fmaf(w, v.y, o[i].y);
-          o[i].z = fmaf(w, v.z, o[i].z);
-          o[i].w = fmaf(w, v.w, o[i].w);
-        }
+        const bool in = w != 0.f;   // a masked key's V may hold anything
+        o[i].x = in ? fmaf(w, v.x, o[i].x) : o[i].x;
+        o[i].y = in ? fmaf(w, v.y, o[i].y) : o[i].y;
+        o[i].z = in ? fmaf(w, v.z, o[i].z) : o[i].z;
+        o[i].w = in ? fmaf(w, v.w, o[i].w) : o[i].w;
       }
     }
     __syncthreads();   // the stage and P are free
+  };
+
+  for (int t = 0; t < ntiles; ++t) {
+    if (t + 1 < ntiles) load(t + 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    if (nrows <= 16)
+      tile(t, std::integral_constant<int, 1>());
+    else if (nrows <= 32)
+      tile(t, std::integral_constant<int, 2>());
+    else
+      tile(t, std::integral_constant<int, 4>());
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();

@@ -203,9 +203,7 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_f32_kernel(const LmParams 
 
 template <int NT>
 cudaError_t launch(const LmParams& p, cudaStream_t s) {
-  const cudaError_t err = cudaFuncSetAttribute(lmhead_f32_kernel<NT>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(Geom<NT>::kBytes));
+  const cudaError_t err = set_smem_attrs(lmhead_f32_kernel<NT>, Geom<NT>::kBytes);
   if (err != cudaSuccess) return err;
   return launch_pdl(lmhead_f32_kernel<NT>, dim3(p.g_lm * ((p.T + NT - 1) / NT)), dim3(kThreads),
                     Geom<NT>::kBytes, s, p);
