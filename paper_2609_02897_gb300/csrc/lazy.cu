@@ -21,9 +21,6 @@
 // same order, so every computed row and verdict is bit-identical to the
 // every-row schedule's.  Which sequence's rows come first within a pass depends
 // on atomic appends; no result depends on it.
-#include <algorithm>
-#include <climits>
-
 #include "kernels.h"
 
 namespace asd {
@@ -31,7 +28,6 @@ namespace {
 
 constexpr int kLazyThreads = 256;
 constexpr int kWarps = kLazyThreads / 32;
-constexpr int kMaxPartsPerLane = kMaxLmRanges / 32;
 // Rows of a pass that are computed ahead at most: two 128-row node tiles, which
 // the wide LM head takes over one stream of W.
 constexpr int kLazyRows = 256;
@@ -173,30 +169,15 @@ __global__ void __launch_bounds__(kLazyThreads) lazy_pass_kernel(const LazyParam
   if (!load_tree(p, b, s0, n, s)) return;
   if (i < n) s.acc[i] = 0;
 
-  // one warp per row: every lane loads its (up to 8) partials before merging
+  // one warp per row
   for (int k = warp; k < mine.y; k += kWarps) {
     const int r = mine.x + k;
     if (r < 0 || r >= p.T) break;
     const int node = p.rows_cur[r] - s0;
     if (node < 0 || node >= n) continue;
-    const float4* src = reinterpret_cast<const float4*>(p.part + static_cast<size_t>(r) * p.g_lm);
-    float4 q[kMaxPartsPerLane];
-#pragma unroll
-    for (int j = 0; j < kMaxPartsPerLane; ++j) {
-      const int g = lane + 32 * j;
-      q[j] = g < p.g_lm ? __ldcg(src + g) : make_float4(-INFINITY, 0.f, 0.f, 0.f);
-    }
-    float m = -INFINITY, sm = 0.f;
-    int a = INT_MAX;
-#pragma unroll
-    for (int j = 0; j < kMaxPartsPerLane; ++j) merge_part(m, sm, a, q[j].x, q[j].y, __float_as_int(q[j].z));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-      const float s2 = __shfl_xor_sync(0xffffffffu, sm, off);
-      const int a2 = __shfl_xor_sync(0xffffffffu, a, off);
-      merge_part(m, sm, a, m2, s2, a2);
-    }
+    float m, sm;
+    int a;
+    merge_row(p.part + static_cast<size_t>(r) * p.g_lm, p.g_lm, m, sm, a);
     if (lane == 0) {
       s.slot[node] = r;
       s.m[node] = m;

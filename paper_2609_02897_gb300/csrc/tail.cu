@@ -8,9 +8,8 @@
 //  walk      choose the committed path under one of four readings of the
 //            paper's first-mismatch rule (Sec. 3.2; TailParams::rule):
 //            0 the longest root-to-node path of accepted nodes, ties to the
-//              lexicographically smallest node sequence: heights of accepted
-//              subtrees bottom-up by depth, then from the root the
-//              lowest-index accepted child whose height is one less;
+//              lexicographically smallest node sequence: from the root the
+//              lowest-index child on any longest path;
 //            1 the same over paths with at most one promoted node (accepted,
 //              not a strict match): strict-only and one-promotion heights;
 //            2 greedy: a strict child if any (lowest index), else the accepted
@@ -26,7 +25,6 @@ namespace asd {
 namespace {
 
 constexpr int kTailThreads = 1024;     // 32 warps: one node's merge per warp
-constexpr int kMaxPartsPerLane = kMaxLmRanges / 32;
 
 __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) {
   __shared__ int s_par[kMaxNodes];
@@ -42,7 +40,7 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) 
   __shared__ int s_bc1[kMaxNodes];                   // rule 1: best child, promotion left
   __shared__ float s_ratio[kMaxNodes];               // rules 2, 3
   __shared__ unsigned long long s_bp[kMaxNodes];     // rules 2, 3: best promoted child key
-  __shared__ int s_maxd, s_len, s_skip;
+  __shared__ int s_maxd, s_deep, s_len, s_skip;
 
   // Until pdl_wait() this kernel reads only caller inputs (cu_nodes, parent,
   // tokens): no kernel of the call writes them, and the call's first kernel
@@ -80,6 +78,7 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) 
   }
   if (i == 0) {
     s_maxd = 0;
+    s_deep = 0;
     s_len = 0;
   }
   const int tree_bad = __syncthreads_or(!okn);
@@ -115,27 +114,12 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) 
   // ---------------------------------------------------------------- finalize
   if (p.mode & kTailFinalize) {
     if (!tree_bad) {
-      // one warp per node: every lane loads its (up to 8) partials before merging
+      // one warp per node
       for (int r = warp; r < n; r += kTailThreads / 32) {
         const size_t node = static_cast<size_t>(s + r);
-        const float4* src = reinterpret_cast<const float4*>(p.part + node * p.g_lm);
-        float4 q[kMaxPartsPerLane];
-#pragma unroll
-        for (int k = 0; k < kMaxPartsPerLane; ++k) {
-          const int g = lane + 32 * k;
-          q[k] = g < p.g_lm ? __ldcg(src + g) : make_float4(-INFINITY, 0.f, 0.f, 0.f);
-        }
-        float m = -INFINITY, sm = 0.f;
-        int a = INT_MAX;
-#pragma unroll
-        for (int k = 0; k < kMaxPartsPerLane; ++k) merge_part(m, sm, a, q[k].x, q[k].y, __float_as_int(q[k].z));
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-          const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-          const float s2 = __shfl_xor_sync(0xffffffffu, sm, off);
-          const int a2 = __shfl_xor_sync(0xffffffffu, a, off);
-          merge_part(m, sm, a, m2, s2, a2);
-        }
+        float m, sm;
+        int a;
+        merge_row(p.part + node * p.g_lm, p.g_lm, m, sm, a);
         if (lane == 0) {
           p.row_max[node] = m;
           p.row_argmax[node] = a;
@@ -176,20 +160,36 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) 
       // a node is strict when it drafts its parent row's top-1; root-level
       // quantities are per node below, the walk runs on thread 0
       const bool strict_i = i > 0 && i < n && s_acc[i] && s_tok[i] == s_arg[s_par[i]];
-      if (p.rule <= 1) {
-        // s_h: heights over accepted (rule 0) or strict-only (rule 1) children;
-        // s_h1: heights with at most one promotion below the node (rule 1)
+      if (p.rule == 0) {
+        // the longest accepted paths end at the deepest nodes whose ancestors
+        // were all accepted; marked up to the root, their nodes leave the walk
+        // the lowest-index marked child at every step (no barrier per level,
+        // as heights bottom-up would need)
+        bool reach = i < n;
+        for (int u = i; reach && u > 0; u = s_par[u]) reach = s_acc[u] != 0;
+        if (i < kMaxNodes) {
+          const int d = __reduce_max_sync(0xffffffffu, reach ? s_dep[i] : 0);
+          if (lane == 0) atomicMax(&s_deep, d);
+        }
+        __syncthreads();
+        if (reach && s_dep[i] == s_deep)
+          for (int u = i; u >= 0; u = s_par[u]) s_h[u] = 0;   // marked
+        __syncthreads();
+        if (i > 0 && i < n && s_h[i] == 0) atomicMin(&s_bc[s_par[i]], i);
+      } else if (p.rule == 1) {
+        // s_h: heights over strict-only children; s_h1: heights with at most
+        // one promotion below the node
         for (int dd = s_maxd; dd >= 1; --dd) {
           if (i < n && s_dep[i] == dd && s_acc[i]) {
-            if (p.rule == 0 || strict_i) atomicMax(&s_h[s_par[i]], s_h[i] + 1);
-            if (p.rule == 1) atomicMax(&s_h1[s_par[i]], (strict_i ? s_h1[i] : s_h[i]) + 1);
+            if (strict_i) atomicMax(&s_h[s_par[i]], s_h[i] + 1);
+            atomicMax(&s_h1[s_par[i]], (strict_i ? s_h1[i] : s_h[i]) + 1);
           }
           __syncthreads();
         }
         if (i > 0 && i < n && s_acc[i]) {
           const int u = s_par[i];
-          if ((p.rule == 0 || strict_i) && s_h[i] == s_h[u] - 1) atomicMin(&s_bc[u], i);
-          if (p.rule == 1 && (strict_i ? s_h1[i] : s_h[i]) == s_h1[u] - 1) atomicMin(&s_bc1[u], i);
+          if (strict_i && s_h[i] == s_h[u] - 1) atomicMin(&s_bc[u], i);
+          if ((strict_i ? s_h1[i] : s_h[i]) == s_h1[u] - 1) atomicMin(&s_bc1[u], i);
         }
       } else if (i > 0 && i < n && s_acc[i]) {
         const int u = s_par[i];
