@@ -134,34 +134,6 @@ struct Item {
 
 constexpr int kOrderMax = 256;   // batches ordered by work in-kernel (larger ones: index order)
 
-// The sequence of rank r when the B sequences are ordered by decreasing
-// attention work (their context and tree key tiles, ties by index): the
-// hardware dispatches CTAs in blockIdx order, so the longest items start
-// first and the short ones fill the last wave.  Every thread of the CTA calls
-// it (it synchronises the CTA); s_work holds kOrderMax ints.
-__device__ __forceinline__ int sequence_of_rank(const AttnParams& p, int r, int* s_work,
-                                                int* s_b) {
-  if (p.B > kOrderMax) return r;
-  if (threadIdx.x == 0) *s_b = r;
-  for (int q = threadIdx.x; q < p.B; q += blockDim.x) {
-    const int c = min(max(p.ctx_len[q], 0), p.ctx_max);
-    const int n = min(max(p.cu_nodes[q + 1] - p.cu_nodes[q], 0), kMaxNodes);
-    s_work[q] = (c + kKeys - 1) / kKeys + (n + kKeys - 1) / kKeys;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < p.B; q += blockDim.x) {
-    const int w = s_work[q];
-    int rank = 0;
-    for (int j = 0; j < p.B; ++j) {
-      const int v = s_work[j];
-      rank += (v > w || (v == w && j < q)) ? 1 : 0;
-    }
-    if (rank == r) *s_b = q;
-  }
-  __syncthreads();
-  return *s_b;
-}
-
 constexpr int kMaxChunks = 32;   // chunks per sequence: one lane of the merging warp each
 constexpr int kMergeOverhead = 3;   // cost of the merge in key tiles of ~1 us
 
@@ -169,8 +141,9 @@ constexpr int kMergeOverhead = 3;   // cost of the merge in key tiles of ~1 us
 struct PlanSmem {
   int s0[kOrderMax], n[kOrderMax], ctx[kOrderMax];   // first node, nodes, context length
   int tiles[kOrderMax];    // key tiles (0: no query rows)
-  int items[kOrderMax];    // query row blocks x KV heads, then CTAs
+  int items[kOrderMax];    // query row blocks x KV heads
   int key[kOrderMax];      // key tiles of the longest chunk
+  int2 order[kOrderMax];   // larger first: by key, then by index; the sequence's CTAs
   int part[kOrderMax];     // partial rows (0: one chunk)
   int chunks[kOrderMax];
   int cut_ctas[kMaxChunks];   // CTAs and partial rows when the longest sequence is
@@ -192,6 +165,12 @@ __device__ __forceinline__ int div_est(int a, int b) {
   q -= q * b > a ? 1 : 0;
   q += (q + 1) * b <= a ? 1 : 0;
   return q;
+}
+
+// Sort key of a sequence: the length of its chunks, then its index, ascending.
+__device__ __forceinline__ int order_key(int tiles, int q) {
+  static_assert(kOrderMax <= 512, "9 bits of index");
+  return (min(tiles, 1 << 21) << 9) | (511 - q);
 }
 
 // Key tiles per chunk.  Lane k weighs cutting the longest sequence into k + 1
@@ -239,13 +218,15 @@ __device__ __forceinline__ int chunk_length(const AttnParams& p, PlanSmem& s) {
 
 // The chunk of CTA blockIdx.x: sequences in decreasing order of their chunks'
 // length (ties by index), within one its KV heads, its chunks, its blocks of
-// query rows (which read the same keys) innermost.  False when the CTA has
-// none.  Every thread of the CTA calls it (it synchronises the CTA).
+// query rows (which read the same keys) innermost.  The hardware dispatches
+// CTAs in blockIdx order, so the longest run first and the short ones fill the
+// last wave.  False when the CTA has none.  Every thread of the CTA calls it (it synchronises the CTA).
+template <int ROWS>
 __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSmem& s) {
   const int idx = blockIdx.x;
   int local, ctx, longest;   // longest: key tiles of the sequence's longest chunk
   if (p.B > kOrderMax) {   // index order, unsplit
-    const int rbmax = (p.max_nodes * p.G + kRows - 1) / kRows;
+    const int rbmax = (p.max_nodes * p.G + ROWS - 1) / ROWS;
     it.b = idx / (rbmax * p.Hkv);
     if (it.b >= p.B) {
       __syncthreads();
@@ -253,7 +234,7 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
     }
     local = idx - it.b * rbmax * p.Hkv;
     it.g = local / rbmax;
-    it.r0 = (local - it.g * rbmax) * kRows;
+    it.r0 = (local - it.g * rbmax) * ROWS;
     it.chunks = 1;
     it.chunk = 0;
     it.part0 = 0;
@@ -275,47 +256,47 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
       s.n[q] = n;
       s.ctx[q] = c;
       s.tiles[q] = okq ? (c + kKeys - 1) / kKeys + (n + kKeys - 1) / kKeys : 0;
-      s.items[q] = okq ? (n * p.G + kRows - 1) / kRows * p.Hkv : 0;
+      s.items[q] = okq ? (n * p.G + ROWS - 1) / ROWS * p.Hkv : 0;
       s.key[q] = s.tiles[q];
       s.part[q] = 0;
       s.chunks[q] = 1;
+      s.order[q] = make_int2(order_key(s.tiles[q], q), s.items[q]);
     }
     __syncthreads();
     if (p.part_cap > 0) {
       const int len = chunk_length(p, s);
-      __syncthreads();   // every warp has read s.items
       const float inv = __frcp_rn(static_cast<float>(len));
       for (int q = threadIdx.x; q < p.B; q += blockDim.x) {
         const int t = s.tiles[q], c = ceil_div_est(t, len, inv);
         s.chunks[q] = c;
         if (c > 1) {
-          s.items[q] *= c;
           s.key[q] = (t + c - 1) / c;
           s.part[q] = s.n[q] * p.Hq * c;
+          s.order[q] = make_int2(order_key(s.key[q], q), s.items[q] * c);
         }
       }
       __syncthreads();
     }
-    // a warp per sequence, its lanes summing the CTAs and partial rows before it
-    const int lane = threadIdx.x & 31;
-    for (int q = threadIdx.x >> 5; q < p.B; q += kThreads / 32) {
-      const int key = s.key[q];
+    // the CTAs (and partial rows) of the sequences before each one, a thread per
+    // sequence: on the way of every CTA's first copy (a warp per sequence, its
+    // lanes over the others, was slower: 64 sequences of 8 nodes at contexts 300
+    // to 1000, 3.4 waves of CTAs, 68.5 us against 61.2)
+    for (int q = threadIdx.x; q < p.B; q += blockDim.x) {
+      const int2 mine = s.order[q];
       int first = 0, part = 0;
-      for (int j = lane; j < p.B; j += 32) {
-        const int kj = s.key[j];
-        const bool before = kj > key || (kj == key && j < q);
-        first += before ? s.items[j] : 0;
-        part += before ? s.part[j] : 0;
+#pragma unroll 8
+      for (int j = 0; j < p.B; ++j) {
+        const int2 o = s.order[j];
+        first += o.x > mine.x ? o.y : 0;
       }
-      first = __reduce_add_sync(0xffffffffu, first);
-      part = __reduce_add_sync(0xffffffffu, part);
-      if (lane == 0 && idx >= first && idx < first + s.items[q]) {
-        s.seq = q;
-        s.first = first;
-        s.part0 = part;
-        if (idx == first && p.part_cap > 0)
-          p.plan[q] = make_int2(part, s.chunks[q]);
+      if (idx < first || idx >= first + mine.y) continue;
+      if (p.part_cap > 0) {
+        for (int j = 0; j < p.B; ++j) part += s.order[j].x > mine.x ? s.part[j] : 0;
+        if (idx == first) p.plan[q] = make_int2(part, s.chunks[q]);
       }
+      s.seq = q;
+      s.first = first;
+      s.part0 = part;
     }
     __syncthreads();
     it.b = s.seq;
@@ -325,10 +306,10 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
     ctx = s.ctx[it.b];
     it.chunks = s.chunks[it.b];
     it.part0 = s.part0;
-    const int rb = (it.n * p.G + kRows - 1) / kRows;
+    const int rb = (it.n * p.G + ROWS - 1) / ROWS;
     local = idx - s.first;
     const int gz = div_est(local, rb);
-    it.r0 = (local - gz * rb) * kRows;
+    it.r0 = (local - gz * rb) * ROWS;
     it.g = div_est(gz, it.chunks);
     it.chunk = gz - it.g * it.chunks;
     longest = s.key[it.b];
@@ -336,7 +317,7 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
   it.R = it.n * p.G;
   if (it.n <= 0 || it.n > kMaxNodes || it.s0 < 0 || it.s0 + it.n > p.T || it.r0 >= it.R)
     return false;
-  it.nrows = min(kRows, it.R - it.r0);
+  it.nrows = min(ROWS, it.R - it.r0);
   const int nctx = (ctx + kKeys - 1) / kKeys, all = nctx + (it.n + kKeys - 1) / kKeys;
   // of the context's tiles, then the tree's, the first chunks take one more
   // than the others where they do not divide
@@ -446,6 +427,28 @@ __device__ __forceinline__ void issue_q_tile(const AttnParams& p, const Item& it
                 pol);
 }
 
+// Ancestor bitmasks (self included) of the sequence's nodes for the tree tile,
+// by the eight softmax warps; a malformed parent ends the walk, so it is bounded.
+__device__ __forceinline__ void tree_masks(const AttnParams& p, const Item& it, int* s_par,
+                                           uint64_t (*s_anc)[2]) {
+  const int tid = threadIdx.x - 64;
+  for (int i = tid; i < it.n; i += kSoftmaxThreads) s_par[i] = p.parent[it.s0 + i];
+  softmax_sync();
+  for (int i = tid; i < it.n; i += kSoftmaxThreads) {
+    uint64_t lo = 0, hi = 0;
+    int u = i;
+    while (true) {
+      if (u < 64) lo |= 1ull << u; else hi |= 1ull << (u - 64);
+      const int pu = s_par[u];
+      if (pu < 0 || pu >= u) break;
+      u = pu;
+    }
+    s_anc[i][0] = lo;
+    s_anc[i][1] = hi;
+  }
+  softmax_sync();
+}
+
 // Softmax warps (eight): warp w handles TMEM lane quarter w % 4 (its 32 query
 // rows, one thread per row) and half h = (w - 2) / 4 of every tile's 128 keys.
 // Per tile: read its 64 S columns, mask, exchange the row's partial max with
@@ -493,23 +496,7 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
     if (lane == 0) mbar_arrive(smem_u32(q_ready));
   }
 
-  // ancestor bitmasks (self included) of the sequence's nodes for the tree
-  // tile; a malformed parent ends the walk, so it is bounded
-  for (int i = tid; i < it.n; i += kSoftmaxThreads) s_par[i] = p.parent[it.s0 + i];
-  softmax_sync();
-  for (int i = tid; i < it.n; i += kSoftmaxThreads) {
-    uint64_t lo = 0, hi = 0;
-    int u = i;
-    while (true) {
-      if (u < 64) lo |= 1ull << u; else hi |= 1ull << (u - 64);
-      const int pu = s_par[u];
-      if (pu < 0 || pu >= u) break;
-      u = pu;
-    }
-    s_anc[i][0] = lo;
-    s_anc[i][1] = hi;
-  }
-  softmax_sync();
+  tree_masks(p, it, s_par, s_anc);
   uint64_t alo = 0, ahi = 0;
   if (row < it.nrows) {
     const int node = (it.r0 + row) / p.G;
@@ -721,7 +708,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
   }
   Item it;
-  const bool some = make_item(p, it, s_plan);   // uniform over the CTA
+  const bool some = make_item<kRows>(p, it, s_plan);   // uniform over the CTA
   tc_fence_after();
   if (!some) {   // no query rows here
     if (warp == 10) tmem_dealloc(s_tmem, kTmemCols);
@@ -926,19 +913,19 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Combines the chunks of every query row that attn_tc_kernel split:
 //   out = sum_z 2^(m_z - M) O_z / sum_z 2^(m_z - M) l_z,  M = max_z m_z.
 // W warps per row: lane z of each reads chunk z's (reference max, row sum),
-// warp w adds up chunks w, w + W, ..., each lane D/32 columns, eight loads in
-// flight, and the W sums meet in shared memory.  Few rows come in many chunks
+// warp w adds up chunks w, w + W, ..., each lane D/32 columns, four or eight
+// loads in flight, and the W sums meet in shared memory.  Few rows come in many chunks
 // and take W = 4 (256 rows in 19 chunks: 3.9 us, 9.7 with a warp per row),
 // many rows in few chunks and take W = 1 (7680 rows in up to 3 chunks: 3.4 us,
 // 11 with four warps, all of it CTA launches).  Sequences in one chunk
 // (plan[b].y == 1) were written by attn_tc_kernel.
 constexpr int kMergeThreads = 256;
 constexpr int kMergeFewRows = 2048;   // query rows of a step up to which W = 4
-constexpr int kMergeLoads = 8;
 
 template <int D, int W>
 __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const AttnParams p) {
   constexpr int kV = D / 32, kMergeWarps = W, kMergeRows = kMergeThreads / 32 / W;
+  constexpr int kMergeLoads = W == 1 ? 4 : 8;   // of 3 and 19 chunks in the cases above
   __shared__ float s_acc[kMergeRows][kMergeWarps][D];
   pdl_launch_dependents();
   const int b = blockIdx.y / p.Hkv, g = blockIdx.y - b * p.Hkv;
@@ -957,9 +944,12 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const AttnPar
   const int row = blockIdx.x * kMergeRows + rl;
   const bool mine = row < R;
   const size_t base = static_cast<size_t>(plan.x) + static_cast<size_t>(g) * c * R + (mine ? row : 0);
-  // the first chunks' rows are on their way while the weights are formed
-  float v[kMergeLoads][kV];
-  auto load = [&](int z0) {
+  float wt = 0.f, sum = 0.f, acc[kV];
+#pragma unroll
+  for (int j = 0; j < kV; ++j) acc[j] = 0.f;
+#pragma unroll 1
+  for (int z0 = w; z0 < c; z0 += kMergeLoads * W) {   // uniform over the warp
+    float v[kMergeLoads][kV];
 #pragma unroll
     for (int k = 0; k < kMergeLoads; ++k) {
       const int z = z0 + k * W;
@@ -977,22 +967,17 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const AttnPar
         v[k][1] = x.y;
       }
     }
-  };
-  load(w);
-  const float2 ml = lane < c ? __ldcg(p.part_ml + base + static_cast<size_t>(lane) * R)
-                             : make_float2(-INFINITY, 0.f);
-  float M = ml.x;
+    if (z0 == w) {   // the weights, while the first chunks' rows are on their way
+      const float2 ml = lane < c ? __ldcg(p.part_ml + base + static_cast<size_t>(lane) * R)
+                                 : make_float2(-INFINITY, 0.f);
+      float M = ml.x;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-  const float wt = ml.x == -INFINITY ? 0.f : exp2f(ml.x - M);
-  float sum = wt * ml.y;
+      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+      wt = ml.x == -INFINITY ? 0.f : exp2f(ml.x - M);
+      sum = wt * ml.y;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  float acc[kV];
-#pragma unroll
-  for (int j = 0; j < kV; ++j) acc[j] = 0.f;
-  for (int z0 = w; z0 < c; z0 += kMergeLoads * W) {   // uniform over the warp
-    if (z0 > w) load(z0);
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    }
 #pragma unroll
     for (int k = 0; k < kMergeLoads; ++k) {
       const float wz = __shfl_sync(0xffffffffu, wt, (z0 + k * W) & 31);   // 0 from c on
@@ -1049,29 +1034,6 @@ struct PPGeom {
   static constexpr int kBytes = kVOff + kStages * kKVTile;
 };
 
-__device__ __forceinline__ bool make_item_pp(const AttnParams& p, Item& it, int* s_work,
-                                             int* s_b) {
-  const int rb = blockIdx.x, bg = blockIdx.y;
-  const int r = bg / p.Hkv;
-  it.b = sequence_of_rank(p, r, s_work, s_b);
-  it.g = bg - r * p.Hkv;
-  it.s0 = p.cu_nodes[it.b];
-  it.n = p.cu_nodes[it.b + 1] - it.s0;
-  it.R = it.n * p.G;
-  it.r0 = rb * kPPRows;
-  if (it.n <= 0 || it.n > kMaxNodes || it.s0 < 0 || it.s0 + it.n > p.T || it.r0 >= it.R)
-    return false;
-  it.nrows = min(kPPRows, it.R - it.r0);
-  it.key_base = 0;
-  it.chunks = 1;
-  it.chunk = it.part0 = 0;
-  it.ctx = min(max(p.ctx_len[it.b], 0), p.ctx_max);
-  it.nctx = (it.ctx + kKeys - 1) / kKeys;
-  it.ntree = (it.n + kKeys - 1) / kKeys;
-  it.ntiles = it.nctx + it.ntree;
-  return true;
-}
-
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_pp_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -1094,24 +1056,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ int s_pages[2][kPageChunk];   // K / V producer: staged page-table entries
   __shared__ int s_issued[2][S];   // producer: K (0) and V (1) fills issued per stage
 
+  __shared__ PlanSmem s_plan;
+
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long budget = wait_budget(p.wait_cycles);
-  __shared__ int s_work[kOrderMax];
-  __shared__ int s_seq;
-  Item it;
-  if (!make_item_pp(p, it, s_work, &s_seq)) {  // no query rows here (uniform over the CTA)
-    pdl_wait();
-    return;
-  }
-  const int nx = it.nrows > kRows ? 2 : 1;   // query tiles present
 
   uint32_t base = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (base & 1023u)) & 1023u;
   uint8_t* gbase = smem_raw + pad;
   base += pad;
 
-  if (threadIdx.x == 0) {
+  // as in the one-tile kernel: the set-up that needs no item under make_item's
+  // first loads, then every role by itself
+  if (threadIdx.x == 32 * 11) {
     for (int s = 0; s < S; ++s) {
       mbar_init(smem_u32(&s_k_full[s]), 1);
       mbar_init(smem_u32(&s_k_empty[s]), 1);
@@ -1124,45 +1082,27 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(smem_u32(&s_p_full[x]), 4);
       mbar_init(smem_u32(&s_pv_done[x]), 1);
     }
-    // the query tiles: one TMA per present tile (p.q_tma), issued before the
-    // rest of the set-up, or the eight softmax warps' stores
+    // the query tiles: TMA (p.q_tma) or the eight softmax warps' stores
     mbar_init(smem_u32(&s_q_ready), p.q_tma ? 1 : 8);
     mbar_init(smem_u32(&s_mma_done[0]), 1);
     mbar_init(smem_u32(&s_mma_done[1]), 1);
     s_abort = 0;
     fence_mbar_init();
-    if (p.q_tma) {
-      const uint64_t pol = l2_policy_evict_first();
-      const uint32_t bar = smem_u32(&s_q_ready);
-      mbar_expect_tx(bar, static_cast<uint32_t>(nx * G::kQTile));
-      for (int x = 0; x < nx; ++x)
-#pragma unroll
-        for (int h = 0; h < G::kNH; ++h)
-          tma_load_3d(base + G::kQOff + x * G::kQTile + h * (kRows * 128), &tm_q, bar, h * 64,
-                      it.g * p.G, it.s0 + (it.r0 + x * kRows) / p.G, pol);
-    }
   }
-  if (warp == 1) {
+  if (warp == 10) {
     tmem_alloc(smem_u32(&s_tmem), kTmemCols);
     tmem_relinquish();
+    tc_fence_before();
   }
-  for (int i = threadIdx.x; i < it.n; i += kThreads) s_par[i] = p.parent[it.s0 + i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < it.n; i += kThreads) {
-    uint64_t lo = 0, hi = 0;
-    int u = i;
-    while (true) {
-      if (u < 64) lo |= 1ull << u; else hi |= 1ull << (u - 64);
-      const int pu = s_par[u];
-      if (pu < 0 || pu >= u) break;
-      u = pu;
-    }
-    s_anc[i][0] = lo;
-    s_anc[i][1] = hi;
-  }
-  tc_fence_before();
-  __syncthreads();
+  Item it;
+  const bool some = make_item<kPPRows>(p, it, s_plan);   // uniform over the CTA
   tc_fence_after();
+  if (!some) {   // no query rows here
+    if (warp == 10) tmem_dealloc(s_tmem, kTmemCols);
+    pdl_wait();
+    return;
+  }
+  const int nx = it.nrows > kRows ? 2 : 1;   // query tiles present
   const uint32_t tmem = s_tmem;
 
   if (warp == 0 || warp == 11) {
@@ -1175,6 +1115,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       prefetch_tmap(which ? &tm_tv : &tm_tk);
     }
     const uint64_t pol = l2_policy_evict_first();
+    if (which == 0 && lane == 0 && p.q_tma) {
+      const uint32_t bar = smem_u32(&s_q_ready);
+      mbar_expect_tx(bar, static_cast<uint32_t>(nx * G::kQTile));
+      for (int x = 0; x < nx; ++x)
+#pragma unroll
+        for (int h = 0; h < G::kNH; ++h)
+          tma_load_3d(base + G::kQOff + x * G::kQTile + h * (kRows * 128), &tm_q, bar, h * 64,
+                      it.g * p.G, it.s0 + (it.r0 + x * kRows) / p.G, pol);
+    }
     int chunk0 = -1;
     bool pok = true;
     for (int t = 0; t < it.ntiles; ++t) {
@@ -1312,6 +1261,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&s_q_ready));
     }
+    tree_masks(p, it, s_par, s_anc);
     uint64_t alo = 0, ahi = 0;
     if (mine) {
       const int node = (it.r0 + rr) / p.G;
@@ -1473,7 +1423,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, kTmemCols);
+  if (warp == 10) tmem_dealloc(tmem, kTmemCols);
   pdl_wait();   // the next kernel's wait covers every earlier kernel
 }
 
@@ -1503,23 +1453,18 @@ cudaError_t launch_attention_tc(const AttnParams& p, const CUtensorMap& tm_k,
   const size_t smem = attention_tc_smem_bytes(p.D, pingpong);
   if (p.D != 64 && p.D != 128) return cudaErrorInvalidValue;
   cudaError_t err;
-  if (pingpong) {
-    const dim3 grid((p.max_nodes * p.G + kPPRows - 1) / kPPRows, p.B * p.Hkv, 1);
-    auto* k = p.D == 64 ? attn_pp_kernel<64> : attn_pp_kernel<128>;
-    err = set_smem_attrs(k, smem);
-    if (err != cudaSuccess) return err;
-    return launch_pdl(k, grid, dim3(kThreads), smem, s, tm_k, tm_v, tm_tk, tm_tv, tm_q, p);
-  }
   // row blocks: at most max_nodes * G rows of each of B sequences, and T * G
   // rows of which every sequence may leave one block ragged; index order
   // (B > kOrderMax) numbers the first form
-  const long long full = static_cast<long long>((p.max_nodes * p.G + kRows - 1) / kRows) * p.B;
+  const int rows = pingpong ? kPPRows : kRows;
+  const long long full = static_cast<long long>((p.max_nodes * p.G + rows - 1) / rows) * p.B;
   const long long blocks =
-      p.B > kOrderMax ? full : std::min(full, static_cast<long long>(p.T) * p.G / kRows + p.B);
+      p.B > kOrderMax ? full : std::min(full, static_cast<long long>(p.T) * p.G / rows + p.B);
   const long long ctas =
       std::max<long long>(blocks * p.Hkv, p.part_cap > 0 ? p.nsm : 0);
   if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
-  auto* k = p.D == 64 ? attn_tc_kernel<64> : attn_tc_kernel<128>;
+  auto* k = pingpong ? (p.D == 64 ? attn_pp_kernel<64> : attn_pp_kernel<128>)
+                     : (p.D == 64 ? attn_tc_kernel<64> : attn_tc_kernel<128>);
   err = set_smem_attrs(k, smem);
   if (err != cudaSuccess) return err;
   err = launch_pdl(k, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), smem, s, tm_k, tm_v, tm_tk,

@@ -335,6 +335,11 @@ __global__ void __launch_bounds__(192, 1)
 // and writes one partial per range, so the statistics are those of CTAs that
 // own one range each, bit for bit.
 //
+// What bounds it (W 128256 x 4096): at 512 nodes 337 us, of which the MMAs alone
+// 317, 85 ns per 128 x 256 x 16 product, the rate of the library's own bf16 GEMM
+// on this GPU (1.9 PFLOP/s), the rest the drains; the loads alone take 250.  From
+// 1024 nodes on (662 us) the power limit sets the pace.
+//
 // Warp roles (352 threads): warp 0 TMA producer, warp 1 TMEM allocator and
 // MMA issuer for node tile 0 of every pair, warp 10 MMA issuer for node tile
 // 1 (two issuing threads: a barrier wait costs its thread a few hundred
@@ -430,10 +435,10 @@ struct WideVocab {
 // How the node tiles are shared out in rounds.  CL = 1: two tiles in a round.
 // CL = 2: four tiles in a round, two per CTA; of what is left at the end
 //   three  go one to each CTA, the third computed on range 0 by the one and on
-//          range 1 by the other: three tiles' MMAs where two pairs, one of them
-//          half empty, took four (the stages' round trip bounds a round more
-//          than its MMAs do: 384 nodes 330 -> 326 us at W 128256 x 4096, 102 ->
-//          97 at 32000 x 4096);
+//          range 1 by the other (the CTAs run in lock step, so the one with two
+//          tiles sets a stage's pace and what this saves over two pairs is
+//          small: 384 nodes 330 -> 326 us at W 128256 x 4096, 102 -> 97 at
+//          32000 x 4096);
 //   two    go one to each CTA, not both to one (1280 nodes 991 -> 940 us and
 //          279 -> 257);
 //   one    goes to the first CTA.
