@@ -203,12 +203,6 @@ struct Ctx {
   long long wait_cycles;
 };
 
-// Clears the status word of a call whose first kernel does not.
-asd_status clear_status(const Ctx& c) {
-  return launch_clear_status(ws_at<int>(c.ws, c.L.status), c.st) == cudaSuccess ? ASD_OK
-                                                                                : ASD_ERR_CUDA;
-}
-
 // Wait budget (SM clock cycles) that asd_debug_set_wait_cycles set for the
 // kernels of later calls; 0: the kernels' default.
 std::atomic<long long> g_wait_cycles{0};
@@ -673,8 +667,6 @@ asd_status asd_accept_path(const asd_dims* dims, const int32_t* parent, const in
   Ctx c;
   asd_status st = begin_call(dims, total_nodes, workspace, workspace_bytes, stream, &c);
   if (st != ASD_OK) return st;
-  st = clear_status(c);
-  if (st != ASD_OK) return st;
   TailParams t = tail_params(c, kTailWalk);
   t.ratio = const_cast<float*>(ratio);
   t.parent = parent;
@@ -686,7 +678,7 @@ asd_status asd_accept_path(const asd_dims* dims, const int32_t* parent, const in
   t.path_len = path_len;
   t.bonus = bonus;
   t.n_promoted = n_promoted;
-  return launch_tail(t, c.st) == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
+  return launch_tail_alone(t, c.st) == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
 }
 
 asd_status asd_kv_compact(const asd_dims* dims, const void* tree_k, const void* tree_v,
@@ -704,8 +696,6 @@ asd_status asd_kv_compact(const asd_dims* dims, const void* tree_k, const void* 
   Ctx c;
   asd_status st = begin_call(dims, total_nodes, workspace, workspace_bytes, stream, &c);
   if (st != ASD_OK) return st;
-  st = clear_status(c);
-  if (st != ASD_OK) return st;
   TailParams t = tail_params(c, kTailCompact);
   t.parent = nullptr;  // path entries are checked against the tree sizes only
   t.cu_nodes = cu_nodes;
@@ -718,7 +708,7 @@ asd_status asd_kv_compact(const asd_dims* dims, const void* tree_k, const void* 
   t.ctx_len = ctx_len;
   t.page_table = page_table;
   t.ctx_len_out = ctx_len_out;
-  return launch_tail(t, c.st) == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
+  return launch_tail_alone(t, c.st) == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
 }
 
 asd_status asd_verify_step(const asd_dims* dims, const asd_verify_args* a, void* workspace,

@@ -253,10 +253,14 @@ struct TailParams {
   int32_t* ctx_len_out;
   int* status;
   int rule;                   // accepted-path reading (asd_accept_rule)
+  int clear_status;           // set by launch_tail_alone: the grid is one cluster, whose
+                              // first CTA clears the status word
   int B, T, Hkv, D, elem_bytes, max_nodes, max_path;
   int ctx_max, page_size, pages_per_seq, num_pages;
 };
 cudaError_t launch_tail(const TailParams& p, cudaStream_t s);
+// The same as a call's only work (walk or commit): it also clears the status word.
+cudaError_t launch_tail_alone(TailParams p, cudaStream_t s);
 
 // Lazy LM head: rows are computed for the roots and for nodes reached through
 // accepted nodes only, in passes over W (lazy.cu).

@@ -25,6 +25,7 @@ namespace asd {
 namespace {
 
 constexpr int kTailThreads = 1024;     // 32 warps: one node's merge per warp
+constexpr int kMaxTailCluster = 16;    // CTAs of a cluster (more than 8: not portable)
 
 __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) {
   __shared__ int s_par[kMaxNodes];
@@ -44,8 +45,15 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) 
 
   // Until pdl_wait() this kernel reads only caller inputs (cu_nodes, parent,
   // tokens): no kernel of the call writes them, and the call's first kernel
-  // waits for the stream's earlier work (in a call of this kernel alone,
-  // the one that clears the status word), so they are final even before the wait.
+  // waits for the stream's earlier work, so they are final even before the wait.
+  // As the call's only kernel it waits here, then its cluster's first CTA clears
+  // the status word before any CTA may set it.
+  if (p.clear_status) {
+    pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.status[0] = p.status[1] = 0;
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
+                 ::: "memory");
+  }
   pdl_launch_dependents();
   const int b = blockIdx.x;
   const int i = threadIdx.x;
@@ -314,6 +322,40 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) 
 
 cudaError_t launch_tail(const TailParams& p, cudaStream_t s) {
   return launch_pdl(tail_kernel, dim3(p.B), dim3(kTailThreads), 0, s, p);
+}
+
+cudaError_t launch_tail_alone(TailParams p, cudaStream_t s) {
+  // Up to 16 sequences as one cluster that clears the status word itself: the
+  // host's launch of a kernel for it is what such a call costs most (walk and
+  // commit of 16 sequences, two calls 15.7 -> 13.6 us).  More, or a device that does not
+  // take the cluster, keep the kernel.
+  if (p.B <= kMaxTailCluster) {
+    cudaError_t err = cudaSuccess;
+    if (p.B > 8)
+      err = cudaFuncSetAttribute(tail_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (err == cudaSuccess) {
+      p.clear_status = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(p.B);
+      cfg.blockDim = dim3(kTailThreads);
+      cfg.stream = s;
+      cudaLaunchAttribute attr[2];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = static_cast<unsigned>(p.B);
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[1].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 2;
+      err = cudaLaunchKernelEx(&cfg, tail_kernel, p);
+      if (err == cudaSuccess) return err;
+    }
+    cudaGetLastError();
+    p.clear_status = 0;
+  }
+  const cudaError_t err = launch_clear_status(p.status, s);
+  return err != cudaSuccess ? err : launch_tail(p, s);
 }
 
 }  // namespace asd
