@@ -428,10 +428,10 @@ __device__ __forceinline__ void issue_q_tile(const AttnParams& p, const Item& it
 }
 
 // Ancestor bitmasks (self included) of the sequence's nodes for the tree tile,
-// by the eight softmax warps; a malformed parent ends the walk, so it is bounded.
-__device__ __forceinline__ void tree_masks(const AttnParams& p, const Item& it, int* s_par,
+// by the eight softmax warps (tid: thread among them); a malformed parent ends
+// the walk, so it is bounded.
+__device__ __forceinline__ void tree_masks(const AttnParams& p, const Item& it, int tid, int* s_par,
                                            uint64_t (*s_anc)[2]) {
-  const int tid = threadIdx.x - 64;
   for (int i = tid; i < it.n; i += kSoftmaxThreads) s_par[i] = p.parent[it.s0 + i];
   softmax_sync();
   for (int i = tid; i < it.n; i += kSoftmaxThreads) {
@@ -449,16 +449,17 @@ __device__ __forceinline__ void tree_masks(const AttnParams& p, const Item& it, 
   softmax_sync();
 }
 
-// One thread's share of a softmax tile: P = exp2(x c - mu) of 64 scores as bf16
+// One thread's share of a softmax tile: P = exp2(x c - mu) of N scores as bf16
 // pairs, and their sum.  Two scores per multiply-add and per addition: the
 // softmax sets the pace at D = 64 and in the ping-pong form (8 x 64 nodes at
 // context 16384, one-tile form: D = 64 123.2 -> 116.3 us, D = 128 129.6 -> 124.4).
-__device__ __forceinline__ float exp2_tile(const float (&x)[64], float c, float mu,
-                                           uint32_t (&pk)[32]) {
+template <int N>
+__device__ __forceinline__ float exp2_tile(const float* x, float c, float mu,
+                                           uint32_t (&pk)[N / 2]) {
   const uint64_t c2 = pack_f32x2(c, c), nmu2 = pack_f32x2(-mu, -mu);
   uint64_t sum = 0ull;
 #pragma unroll
-  for (int k = 0; k < 64; k += 2) {
+  for (int k = 0; k < N; k += 2) {
     float y0, y1;
     unpack_f32x2(fma_f32x2(pack_f32x2(x[k], x[k + 1]), c2, nmu2), y0, y1);
     const float p0 = ex2_approx(y0), p1 = ex2_approx(y1);
@@ -518,7 +519,7 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
     if (lane == 0) mbar_arrive(smem_u32(q_ready));
   }
 
-  tree_masks(p, it, s_par, s_anc);
+  tree_masks(p, it, tid, s_par, s_anc);
   uint64_t alo = 0, ahi = 0;
   if (row < it.nrows) {
     const int node = (it.r0 + row) / p.G;
@@ -598,7 +599,7 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
     }
     const float mu = (m_ref == -INFINITY) ? 0.f : m_ref;
     uint32_t pk[32];
-    l += exp2_tile(x, c, mu, pk);
+    l += exp2_tile<64>(x, c, mu, pk);
     tmem_st32u(sb + 32 * hf, pk);
     if (valid < kKeys) {
       // ragged tile: V rows past the last valid key may hold anything; zero
@@ -1028,15 +1029,28 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const AttnPar
 // both: S_A = Q_A.K^T and S_B = Q_B.K^T, then O_A += P_A.V and O_B += P_B.V, so
 // the MMAs of one tile run while the other tile's softmax works, and a K/V
 // byte feeds twice the products.  Q stays in shared memory (both tiles, 128-byte
-// swizzled, by TMA or written by the softmax threads); TMEM holds O_A [0, D),
-// O_B [D, 2D) and S/P_A [256, 384), S/P_B [384, 512).  K and V come through
+// swizzled, by TMA or written by the softmax threads).  K and V come through
 // separate rings with their own barriers, so a K slot is refilled as soon as
 // both S MMAs have read it.  Warps: 0 K producer, 1 S-MMA issuer (lane 0),
-// 2-5 softmax of tile A, 6-9 softmax of tile B, 10 P.V-MMA issuer (lane 0),
-// 11 V producer; a softmax thread owns one row
-// of its tile and all 128 keys of every key tile, so no exchange between warps
-// is needed: per key tile it reads S twice (the row max, then the
-// exponentials) and writes P as bf16 pairs over the S columns already read.
+// 2 P.V-MMA issuer (lane 0), 3 V producer, 4-7 softmax of tile A, 8-11 softmax
+// of tile B; a softmax thread owns one row of its tile and all 128 keys of
+// every key tile, so no exchange between warps is needed.  It takes the row's
+// 128 scores into registers with one TMEM load, which frees the S columns: S of
+// the next tile does not wait for the softmax or for P.V.  P has columns of its
+// own (bf16 pairs, half as many), so TMEM holds O_A, O_B, one S buffer and P_A,
+// P_B at D = 128, an S buffer per query tile at D = 64.  The 128 scores need
+// more than 168 registers a thread, so the softmax warpgroups take what the
+// issuing one leaves (setmaxnreg).
+//
+// Measured against S and P sharing their columns, the scores read twice (before
+// -> now, 8 KV heads, G = 4): 64 x 128 nodes at context 2048 303.5 -> 274.5 us
+// (D = 128), 265.6 -> 225 us (D = 64); contexts 300-1000 180.7 -> 149 us; 62 x
+// 60 nodes at 17-137 66.8 -> 53.5 us.  What bounds it: a pair of key tiles takes
+// ~3,950 cycles, of which the MMAs alone ~3,200 (shared memory feeds the S ones);
+// the rest is S read -> next S.  No faster: two warps per row quarter, 64 keys
+// each and a pair barrier (299 us), P handed over by key halves (274.3, D = 64
+// 252), P.V held back while S MMAs are issued (282), waits that spin on test_wait
+// instead of try_wait (288).
 constexpr int kPPRows = 2 * kRows;   // query rows per CTA
 
 template <int D>
@@ -1049,7 +1063,33 @@ struct PPGeom {
   static constexpr int kKOff = 2 * kQTile;
   static constexpr int kVOff = kKOff + kStages * kKVTile;
   static constexpr int kBytes = kVOff + kStages * kKVTile;
+  // TMEM columns: O_A, O_B, then the S buffers (at D = 128 one for both query
+  // tiles), then P_A and P_B
+  static constexpr int kSBufs = D == 64 ? 2 : 1;
+  static __device__ __forceinline__ uint32_t s_col(int x) {
+    return 2 * D + (kSBufs == 2 ? kKeys * static_cast<uint32_t>(x) : 0u);
+  }
+  static __device__ __forceinline__ uint32_t p_col(int x) {
+    return 384u + kKeys / 2 * static_cast<uint32_t>(x);
+  }
 };
+
+// Registers per thread of the issuing warpgroup (warps 0-3) and of the two
+// softmax ones, out of the 168 each that the block is launched with (a split
+// whose sum is above that would wait forever).  88 / 208: D = 64 229 us, not 225.
+constexpr int kPPIssueRegs = 120, kPPSoftmaxRegs = 192;
+static_assert(128 * kPPIssueRegs + 256 * kPPSoftmaxRegs <= kThreads * 168,
+              "more registers than the block is launched with");
+
+template <int N>
+__device__ __forceinline__ void regs_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+
+template <int N>
+__device__ __forceinline__ void regs_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -1062,6 +1102,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t s_k_full[S], s_k_empty[S], s_v_full[S], s_v_empty[S];
   __shared__ __align__(8) uint64_t s_s_full[2];    // S of tile X computed (MMA -> softmax X)
+  __shared__ __align__(8) uint64_t s_s_read[2];    // S of tile X read (softmax X -> MMA)
   __shared__ __align__(8) uint64_t s_p_full[2];    // P of tile X written (softmax X -> MMA)
   __shared__ __align__(8) uint64_t s_pv_done[2];   // O_X += P_X V done (MMA -> softmax X)
   __shared__ __align__(8) uint64_t s_q_ready;
@@ -1086,7 +1127,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   // as in the one-tile kernel: the set-up that needs no item under make_item's
   // first loads, then every role by itself
-  if (threadIdx.x == 32 * 11) {
+  if (threadIdx.x == 32 * 3) {
     for (int s = 0; s < S; ++s) {
       mbar_init(smem_u32(&s_k_full[s]), 1);
       mbar_init(smem_u32(&s_k_empty[s]), 1);
@@ -1096,6 +1137,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int x = 0; x < 2; ++x) {
       mbar_init(smem_u32(&s_s_full[x]), 1);
+      mbar_init(smem_u32(&s_s_read[x]), 4);
       mbar_init(smem_u32(&s_p_full[x]), 4);
       mbar_init(smem_u32(&s_pv_done[x]), 1);
     }
@@ -1106,7 +1148,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     s_abort = 0;
     fence_mbar_init();
   }
-  if (warp == 10) {
+  if (warp == 2) {
     tmem_alloc(smem_u32(&s_tmem), kTmemCols);
     tmem_relinquish();
     tc_fence_before();
@@ -1115,149 +1157,154 @@ __global__ void __launch_bounds__(kThreads, 1)
   const bool some = make_item<kPPRows>(p, it, s_plan);   // uniform over the CTA
   tc_fence_after();
   if (!some) {   // no query rows here
-    if (warp == 10) tmem_dealloc(s_tmem, kTmemCols);
+    if (warp == 2) tmem_dealloc(s_tmem, kTmemCols);
     pdl_wait();
     return;
   }
   const int nx = it.nrows > kRows ? 2 : 1;   // query tiles present
   const uint32_t tmem = s_tmem;
 
-  if (warp == 0 || warp == 11) {
-    // ----------------------------------------------------------- TMA producers
-    // K (warp 0) and V (warp 11), each into its own ring; K slots free up as
-    // soon as both S MMAs of their tile are done, V slots after both P.V MMAs
-    const int which = warp == 0 ? 0 : 1;
-    if (lane == 0) {
-      prefetch_tmap(which ? &tm_v : &tm_k);
-      prefetch_tmap(which ? &tm_tv : &tm_tk);
-    }
-    const uint64_t pol = l2_policy_evict_first();
-    if (which == 0 && lane == 0 && p.q_tma) {
-      const uint32_t bar = smem_u32(&s_q_ready);
-      mbar_expect_tx(bar, static_cast<uint32_t>(nx * G::kQTile));
-      for (int x = 0; x < nx; ++x)
-#pragma unroll
-        for (int h = 0; h < G::kNH; ++h)
-          tma_load_3d(base + G::kQOff + x * G::kQTile + h * (kRows * 128), &tm_q, bar, h * 64,
-                      it.g * p.G, it.s0 + (it.r0 + x * kRows) / p.G, pol);
-    }
-    int chunk0 = -1;
-    bool pok = true;
-    for (int t = 0; t < it.ntiles; ++t) {
-      const int stage = t % S;
-      uint64_t* empty = which ? &s_v_empty[stage] : &s_k_empty[stage];
-      uint64_t* full = which ? &s_v_full[stage] : &s_k_full[stage];
-      if (!wait_all(empty, ((t / S) & 1) ^ 1u, budget) || aborted_warp(&s_abort)) {
-        pok = false;
-        break;
+  if (warp < 4) {
+    regs_dec<kPPIssueRegs>();
+    if (warp == 0 || warp == 3) {
+      // ----------------------------------------------------------- TMA producers
+      // K (warp 0) and V (warp 3), each into its own ring; K slots free up as
+      // soon as both S MMAs of their tile are done, V slots after both P.V MMAs
+      const int which = warp == 0 ? 0 : 1;
+      if (lane == 0) {
+        prefetch_tmap(which ? &tm_v : &tm_k);
+        prefetch_tmap(which ? &tm_tv : &tm_tk);
       }
-      const uint32_t dst = base + (which ? G::kVOff : G::kKOff) + stage * G::kKVTile;
-      if (p.page_size != 0 && t < it.nctx)
-        issue_paged_half<D>(p, it, t, dst, smem_u32(full), which ? &tm_v : &tm_k, pol,
-                            s_pages[which], chunk0, lane);
-      else if (lane == 0)
-        issue_half_tile<D>(p, it, t, dst, smem_u32(full), which ? &tm_v : &tm_k,
-                           which ? &tm_tv : &tm_tk, pol);
-      if (lane == 0) ++s_issued[which][stage];
-      __syncwarp();
-    }
-    if (!pok && lane == 0) {
-      note_timeout(p.status);
-      s_abort = 1;
-    }
-    // every copy issued has landed before the buffers are reused or left
-    // (the query tiles' too, which a wait that gave up may have left in flight)
-    if (lane == 0) {
-      for (int st = 0; st < S; ++st)
-        if (s_issued[which][st] > 0)
-          mbar_wait(smem_u32(which ? &s_v_full[st] : &s_k_full[st]),
-                    static_cast<uint32_t>((s_issued[which][st] - 1) & 1));
-      if (which == 0 && p.q_tma) mbar_wait(smem_u32(&s_q_ready), 0);
-    }
-    __syncwarp();
-  } else if (warp == 1 || warp == 10) {
-    // ------------------------------------------------------------ MMA issuers
-    // Two issuing threads, so that the one's barrier waits overlap the other's
-    // MMAs: warp 1 issues S_x(t) = Q_x K(t)^T, warp 10 O_x += P_x(t) V(t).
-    // While tile A's softmax works on key tile t, the tensor cores run
-    // O_B += P_B V(t-1) and S_B(t); while B's works, O_A += P_A V(t) and
-    // S_A(t+1).  Each commit tracks the issuing thread's own MMAs.
-    if (lane == 0) {
-      bool mok = true;
-      if (warp == 1) {
-        const uint32_t idesc_s = idesc_bf16(kRows, kKeys);   // S = Q K^T
-        mok = mbar_wait(smem_u32(&s_q_ready), 0, budget);
-        if (mok) tc_fence_after();
-        for (int t = 0; mok && t < it.ntiles; ++t) {
-          const int stage = t % S;
-          mok = mbar_wait(smem_u32(&s_k_full[stage]), (t / S) & 1, budget);
-          for (int x = 0; mok && x < nx; ++x) {
-            // tile x's S/P columns are free once O_x += P_x V of tile t-1 is done
-            if (t > 0) mok = mbar_wait(smem_u32(&s_pv_done[x]), (t - 1) & 1, budget);
-            if (!mok || s_abort) {
-              mok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t kst = base + G::kKOff + stage * G::kKVTile;
-            const uint32_t qst = base + G::kQOff + x * G::kQTile;
+      const uint64_t pol = l2_policy_evict_first();
+      if (which == 0 && lane == 0 && p.q_tma) {
+        const uint32_t bar = smem_u32(&s_q_ready);
+        mbar_expect_tx(bar, static_cast<uint32_t>(nx * G::kQTile));
+        for (int x = 0; x < nx; ++x)
 #pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) {
-              const int h = ks >> 2, kk = ks & 3;
-              tc_mma(tmem + (256u + 128u * static_cast<uint32_t>(x)),
-                     sw128_desc(qst + h * (kRows * 128) + 32 * kk),
-                     sw128_desc(kst + h * (kKeys * 128) + 32 * kk), idesc_s, ks > 0 ? 1u : 0u);
-            }
-            tc_commit(smem_u32(&s_s_full[x]));
-          }
-          // the last S of tile t releases K(t)
-          if (mok) tc_commit(smem_u32(&s_k_empty[stage]));
-        }
-      } else {
-        const uint32_t idesc_o = idesc_bf16(kRows, D, true);   // O += P V, V MN-major
-        for (int t = 0; mok && t < it.ntiles; ++t) {
-          const int stage = t % S;
-          mok = mbar_wait(smem_u32(&s_v_full[stage]), (t / S) & 1, budget);
-          for (int x = 0; mok && x < nx; ++x) {
-            // O_x += P_x(t) V(t) once tile x's softmax of key tile t is done
-            mok = mbar_wait(smem_u32(&s_p_full[x]), t & 1, budget);
-            if (!mok || s_abort) {
-              mok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t vst = base + G::kVOff + stage * G::kKVTile;
-#pragma unroll
-            for (int kk = 0; kk < kKeys / 16; ++kk)
-              tc_mma_ts(tmem + static_cast<uint32_t>(x * D),
-                        tmem + (256u + 128u * static_cast<uint32_t>(x)) + kk * 8,
-                        sw128_desc_mn(vst + kk * 2048, kKeys * 128, 1024), idesc_o,
-                        (t > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(smem_u32(&s_pv_done[x]));
-          }
-          // the last P.V of tile t releases V(t)
-          if (mok) tc_commit(smem_u32(&s_v_empty[stage]));
-        }
+          for (int h = 0; h < G::kNH; ++h)
+            tma_load_3d(base + G::kQOff + x * G::kQTile + h * (kRows * 128), &tm_q, bar, h * 64,
+                        it.g * p.G, it.s0 + (it.r0 + x * kRows) / p.G, pol);
       }
-      if (!mok) {
+      int chunk0 = -1;
+      bool pok = true;
+      for (int t = 0; t < it.ntiles; ++t) {
+        const int stage = t % S;
+        uint64_t* empty = which ? &s_v_empty[stage] : &s_k_empty[stage];
+        uint64_t* full = which ? &s_v_full[stage] : &s_k_full[stage];
+        if (!wait_all(empty, ((t / S) & 1) ^ 1u, budget) || aborted_warp(&s_abort)) {
+          pok = false;
+          break;
+        }
+        const uint32_t dst = base + (which ? G::kVOff : G::kKOff) + stage * G::kKVTile;
+        if (p.page_size != 0 && t < it.nctx)
+          issue_paged_half<D>(p, it, t, dst, smem_u32(full), which ? &tm_v : &tm_k, pol,
+                              s_pages[which], chunk0, lane);
+        else if (lane == 0)
+          issue_half_tile<D>(p, it, t, dst, smem_u32(full), which ? &tm_v : &tm_k,
+                             which ? &tm_tv : &tm_tk, pol);
+        if (lane == 0) ++s_issued[which][stage];
+        __syncwarp();
+      }
+      if (!pok && lane == 0) {
         note_timeout(p.status);
         s_abort = 1;
       }
-      // every MMA this thread issued has finished before TMEM or the buffers
-      // are reused
-      uint64_t* done = &s_mma_done[warp == 1 ? 0 : 1];
-      tc_commit(smem_u32(done));
-      mbar_wait(smem_u32(done), 0);
+      // every copy issued has landed before the buffers are reused or left
+      // (the query tiles' too, which a wait that gave up may have left in flight)
+      if (lane == 0) {
+        for (int st = 0; st < S; ++st)
+          if (s_issued[which][st] > 0)
+            mbar_wait(smem_u32(which ? &s_v_full[st] : &s_k_full[st]),
+                      static_cast<uint32_t>((s_issued[which][st] - 1) & 1));
+        if (which == 0 && p.q_tma) mbar_wait(smem_u32(&s_q_ready), 0);
+      }
+      __syncwarp();
+    } else {
+      // ------------------------------------------------------------ MMA issuers
+      // Two issuing threads, so that the one's barrier waits overlap the other's
+      // MMAs: warp 1 issues S_x(t) = Q_x K(t)^T, warp 2 O_x += P_x(t) V(t).
+      // While tile A's softmax works on key tile t, the tensor cores run
+      // O_B += P_B V(t-1) and S_B(t); while B's works, O_A += P_A V(t) and
+      // S_A(t+1).  Each commit tracks the issuing thread's own MMAs.
+      if (lane == 0) {
+        bool mok = true;
+        if (warp == 1) {
+          const uint32_t idesc_s = idesc_bf16(kRows, kKeys);   // S = Q K^T
+          mok = mbar_wait(smem_u32(&s_q_ready), 0, budget);
+          if (mok) tc_fence_after();
+          for (int t = 0; mok && t < it.ntiles; ++t) {
+            const int stage = t % S;
+            mok = mbar_wait(smem_u32(&s_k_full[stage]), (t / S) & 1, budget);
+            for (int x = 0; mok && x < nx; ++x) {
+              // the S columns are free once their last tile has been read: tile x's
+              // own, or (one buffer) that of the query tile before it
+              const int px = G::kSBufs == 2 ? x : (x == 0 ? nx - 1 : 0);
+              const int pt = px < x ? t : t - 1;
+              if (pt >= 0) mok = mbar_wait(smem_u32(&s_s_read[px]), pt & 1, budget);
+              if (!mok || s_abort) {
+                mok = false;
+                break;
+              }
+              tc_fence_after();
+              const uint32_t kst = base + G::kKOff + stage * G::kKVTile;
+              const uint32_t qst = base + G::kQOff + x * G::kQTile;
+#pragma unroll
+              for (int ks = 0; ks < D / 16; ++ks) {
+                const int h = ks >> 2, kk = ks & 3;
+                tc_mma(tmem + G::s_col(x), sw128_desc(qst + h * (kRows * 128) + 32 * kk),
+                       sw128_desc(kst + h * (kKeys * 128) + 32 * kk), idesc_s, ks > 0 ? 1u : 0u);
+              }
+              tc_commit(smem_u32(&s_s_full[x]));
+            }
+            // the last S of tile t releases K(t)
+            if (mok) tc_commit(smem_u32(&s_k_empty[stage]));
+          }
+        } else {
+          const uint32_t idesc_o = idesc_bf16(kRows, D, true);   // O += P V, V MN-major
+          for (int t = 0; mok && t < it.ntiles; ++t) {
+            const int stage = t % S;
+            mok = mbar_wait(smem_u32(&s_v_full[stage]), (t / S) & 1, budget);
+            for (int x = 0; mok && x < nx; ++x) {
+              // O_x += P_x(t) V(t) once tile x's softmax of key tile t is done
+              mok = mbar_wait(smem_u32(&s_p_full[x]), t & 1, budget);
+              if (!mok || s_abort) {
+                mok = false;
+                break;
+              }
+              tc_fence_after();
+              const uint32_t vst = base + G::kVOff + stage * G::kKVTile;
+#pragma unroll
+              for (int kk = 0; kk < kKeys / 16; ++kk)
+                tc_mma_ts(tmem + static_cast<uint32_t>(x * D), tmem + G::p_col(x) + kk * 8,
+                          sw128_desc_mn(vst + kk * 2048, kKeys * 128, 1024), idesc_o,
+                          (t > 0 || kk > 0) ? 1u : 0u);
+              tc_commit(smem_u32(&s_pv_done[x]));
+            }
+            // the last P.V of tile t releases V(t)
+            if (mok) tc_commit(smem_u32(&s_v_empty[stage]));
+          }
+        }
+        if (!mok) {
+          note_timeout(p.status);
+          s_abort = 1;
+        }
+        // every MMA this thread issued has finished before TMEM or the buffers
+        // are reused
+        uint64_t* done = &s_mma_done[warp == 1 ? 0 : 1];
+        tc_commit(smem_u32(done));
+        mbar_wait(smem_u32(done), 0);
+      }
+      __syncwarp();
     }
-    __syncwarp();
   } else {
+    regs_inc<kPPSoftmaxRegs>();
     // ------------------------------------------------------------ softmax of tile x
-    const int x = (warp - 2) >> 2;
+    const int x = (warp - 4) >> 2;
     const int row = (warp & 3) * 32 + lane;    // = TMEM lane = row of the tile
     const int rr = x * kRows + row;            // row of the item
     const bool mine = rr < it.nrows;
     const uint32_t lane_base = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-    const uint32_t sb = lane_base + (256u + 128u * static_cast<uint32_t>(x));
+    const uint32_t sb = lane_base + G::s_col(x), pb = lane_base + G::p_col(x);
     // the row's query -> shared memory, 128-byte swizzled like a TMA tile
     // (unless the query tiles come by TMA)
     if (!p.q_tma) {
@@ -1278,7 +1325,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&s_q_ready));
     }
-    tree_masks(p, it, s_par, s_anc);
+    tree_masks(p, it, threadIdx.x - 128, s_par, s_anc);
     uint64_t alo = 0, ahi = 0;
     if (mine) {
       const int node = (it.r0 + rr) / p.G;
@@ -1297,48 +1344,54 @@ __global__ void __launch_bounds__(kThreads, 1)
       ok = wait_all(&s_s_full[x], t & 1, budget) && !aborted_warp(&s_abort);
       if (!ok) break;
       tc_fence_after();
-      // pass 1: the row's max over the tile's keys (raw scores); only a
-      // ragged context tile and the tree tile need the key mask
-      const bool masked = tree || valid < kKeys;
-      float mt = -INFINITY;
+      // the row's scores -> registers, which frees the S columns for the next
+      // S; only a ragged context tile and the tree tile need the key mask
+      float xs[128];
+      tmem_ld128(sb, xs);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&s_s_read[x]));
+      if (tree || valid < kKeys) {
 #pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-        float xs[64];
-        tmem_ld64(sb + 64 * hf, xs);
-        if (masked) {
-          // the tree tile holds every node of the sequence (at most 128) from
-          // key 0: key k of this half is bit k of the half's ancestor word
-          const uint64_t am = tree ? (hf ? ahi : alo) : ~0ull;
+        for (int q = 0; q < 4; ++q) {   // 32 keys each, a bit per key
+          // the tree tile holds every node of the sequence (at most 128) from key 0
+          const int own = min(max(valid - 32 * q, 0), 32);
+          uint32_t w = own == 32 ? ~0u : (1u << own) - 1u;
+          if (tree) w &= static_cast<uint32_t>((q & 2 ? ahi : alo) >> (32 * (q & 1)));
 #pragma unroll
-          for (int k = 0; k < 64; ++k) {
-            const bool v = (64 * hf + k < valid) && ((am >> k) & 1ull);
-            xs[k] = v ? xs[k] : -INFINITY;
-          }
+          for (int k = 0; k < 32; ++k)
+            xs[32 * q + k] = (w >> k) & 1u ? xs[32 * q + k] : -INFINITY;
         }
-#pragma unroll
-        for (int k = 0; k < 64; k += 2) mt = fmaxf(fmaxf(mt, xs[k]), xs[k + 1]);
       }
+      float m4[4];   // four chains of maxima
+#pragma unroll
+      for (int q = 0; q < 4; ++q) m4[q] = fmaxf(xs[2 * q], xs[2 * q + 1]);
+#pragma unroll
+      for (int k = 8; k < 128; k += 8)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          m4[q] = fmaxf(fmaxf(m4[q], xs[k + 2 * q]), xs[k + 2 * q + 1]);
+      float mt = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
       mt *= c;
       const float mn = fmaxf(m_ref, mt);
       const bool had = m_ref != -INFINITY;
       const bool need = had ? (mn > m_ref + kRescaleLog2) : (mn != -INFINITY);
-      if (__any_sync(0xffffffffu, need && had)) {
-        // O holds earlier tiles of this row: rescale it once O += P V of tile
-        // t-1 is done
-        if (!wait_all(&s_pv_done[x], (t - 1) & 1, budget)) {
-          ok = false;
-          break;
-        }
+      // O += P V of tile t-1 is done: P may be written again, O rescaled
+      if (t > 0) {
+        ok = wait_all(&s_pv_done[x], (t - 1) & 1, budget);
+        if (!ok) break;
         tc_fence_after();
+      }
+      if (__any_sync(0xffffffffu, need && had)) {
         const float alpha = (need && had) ? exp2f(m_ref - mn) : 1.f;
 #pragma unroll 1
-        for (int cc = 0; cc < D / 32; ++cc) {
-          float o[32];
-          const uint32_t oc = lane_base + static_cast<uint32_t>(x * D) + 32 * cc;
-          tmem_ld32(oc, o);
+        for (int cc = 0; cc < D / 16; ++cc) {
+          uint32_t o[16];
+          const uint32_t oc = lane_base + static_cast<uint32_t>(x * D) + 16 * cc;
+          tmem_ld16(oc, o);
 #pragma unroll
-          for (int i = 0; i < 32; ++i) o[i] *= alpha;
-          tmem_st32(oc, o);
+          for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+          tmem_st16(oc, o);
         }
       }
       if (need) {
@@ -1346,26 +1399,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         m_ref = mn;
       }
       const float mu = (m_ref == -INFINITY) ? 0.f : m_ref;
-      // pass 2: P = exp2(s c - m) as bf16 pairs over the S columns already read
-      // (a loop: unrolled it holds both halves' values at the 168-register cap;
-      // 64 x 128 nodes at context 2048, paged, 340 -> 301 us with exp2_tile)
-#pragma unroll 1
-      for (int hf = 0; hf < 2; ++hf) {
-        float xs[64];
-        tmem_ld64(sb + 64 * hf, xs);
-        if (masked) {
-          // the tree tile holds every node of the sequence (at most 128) from
-          // key 0: key k of this half is bit k of the half's ancestor word
-          const uint64_t am = tree ? (hf ? ahi : alo) : ~0ull;
+      // P = exp2(s c - m) as bf16 pairs
 #pragma unroll
-          for (int k = 0; k < 64; ++k) {
-            const bool v = (64 * hf + k < valid) && ((am >> k) & 1ull);
-            xs[k] = v ? xs[k] : -INFINITY;
-          }
-        }
-        uint32_t pk[32];
-        l += exp2_tile(xs, c, mu, pk);
-        tmem_st32u(sb + 32 * hf, pk);
+      for (int q = 0; q < 4; ++q) {
+        uint32_t pk[16];
+        l += exp2_tile<32>(xs + 32 * q, c, mu, pk);
+        tmem_st16u(pb + 16 * q, pk);
       }
       if (valid < kKeys && x == 0) {
         // ragged tile: V rows past the last valid key may hold anything; zero
@@ -1377,7 +1416,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         uint8_t* vt = gbase + G::kVOff + stage * G::kKVTile;
         constexpr int kChunksPerRow = G::kNH * 8;
-        for (int i = threadIdx.x - 64; i < (kKeys - valid) * kChunksPerRow; i += 128) {
+        for (int i = threadIdx.x - 128; i < (kKeys - valid) * kChunksPerRow; i += 128) {
           const int r = valid + i / kChunksPerRow, rem = i % kChunksPerRow;
           *reinterpret_cast<uint4*>(vt + (rem >> 3) * (kKeys * 128) + r * 128 + (rem & 7) * 16) =
               make_uint4(0u, 0u, 0u, 0u);
@@ -1437,7 +1476,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 10) tmem_dealloc(tmem, kTmemCols);
+  if (warp == 2) tmem_dealloc(tmem, kTmemCols);
   pdl_wait();   // the next kernel's wait covers every earlier kernel
 }
 

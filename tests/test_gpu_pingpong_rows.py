@@ -1,0 +1,45 @@
+"""The ping-pong attention's two query tiles at the row counts where they
+change (one tile only, a full first tile, one row in the second, both full) in
+one ragged batch, against a plain PyTorch fp32 reference.  Keys grow along the
+context, so that the running maximum is raised, and O rescaled, more than once."""
+import pytest
+
+from test_gpu_attention_ragged import _call, _check_close, _inputs, _reference
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("D,page,Hq", [(128, 0, 32), (128, 16, 32), (64, 0, 32), (64, 64, 24)])
+def test_row_counts_of_the_two_query_tiles(D, page, Hq):
+    import torch
+    from paper_2609_02897_gb300 import asd
+    Hkv, B, N, cap = 8, 64, 128, 1024
+    nodes = [(1, 31, 32, 33, 43, 64, 127, 128)[b % 8] for b in range(B)]
+    ctx = [(0, 1, 127, 128, 129, 300, 640, 895)[(b // 8 + b) % 8] for b in range(B)]
+    full = _inputs(B, N, ctx, page, Hq, Hkv, D, cap, 5)
+    # a score's standard deviation rises from 1 to 8 over the cache
+    if page == 0:
+        full["k_cache"] *= torch.linspace(1, 8, cap, device="cuda").view(1, 1, cap, 1)
+    else:
+        of_page = torch.empty(B * cap // page, device="cuda")
+        of_page[full["page_table"].long()] = torch.linspace(1, 8, cap // page, device="cuda")
+        full["k_cache"] *= of_page.view(-1, 1, 1, 1)
+    # each sequence keeps its first nodes (a prefix of the binary tree is one)
+    rows = torch.cat([torch.arange(b * N, b * N + n) for b, n in enumerate(nodes)]).cuda()
+    d = dict(full)
+    for k in ("q", "tree_k", "tree_v", "parent"):
+        d[k] = full[k][rows].contiguous()
+    d["cu_nodes"] = torch.tensor([0] + nodes).cumsum(0).int().cuda()
+    T = sum(nodes)
+    dims = asd.make_dims(B, Hq, Hkv, D, 64, 64, asd.ASD_BF16, page, cap,
+                         B * cap // page if page else 0, N, N)
+    assert asd.asd_attention_variant(dims, T) == 3
+    out = _call(d, dims, asd.alloc_workspace(dims, T))
+    s = 0
+    for b, n in enumerate(nodes):
+        one = {k: d[k][s:s + n] for k in ("q", "tree_k", "tree_v")}
+        one["page_table"] = d["page_table"][b:b + 1] if page else None
+        for k in ("k_cache", "v_cache"):
+            one[k] = d[k] if page else d[k][b:b + 1]
+        _check_close(out[s:s + n], _reference(one, 1, n, ctx[b:b + 1], page, Hq, Hkv, D))
+        s += n
