@@ -520,12 +520,8 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
   }
 
   tree_masks(p, it, tid, s_par, s_anc);
-  uint64_t alo = 0, ahi = 0;
-  if (row < it.nrows) {
-    const int node = (it.r0 + row) / p.G;
-    alo = s_anc[node][0];
-    ahi = s_anc[node][1];
-  }
+  // ancestors among the keys of this half of the tree tile
+  const uint64_t anc = row < it.nrows ? s_anc[(it.r0 + row) / p.G][hf] : 0ull;
   const float c = p.scale_log2;
   float m_ref = -INFINITY, l = 0.f;
   bool ok = true, bad = false;
@@ -544,17 +540,23 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
       tc_fence_after();
       tmem_ld64(sb + 64 * hf, x);
       if (tree || valid < kKeys) {
-        // the tree tile holds every node of the sequence (at most 128) from
-        // key 0: key k of this half is bit k of the half's ancestor word
-        const uint64_t am = tree ? (hf ? ahi : alo) : ~0ull;
+        // a bit per key (a 64-bit shift and a comparison per key, and one chain
+        // of 32 maxima below: 16 ragged sequences of 20-100 nodes 71.0 us, now
+        // 68.9; 4 x 60 nodes at contexts to 3600 25.2 -> 24.6); the tree tile
+        // holds every node of the sequence, at most 128, from key 0
+        const int own = min(max(valid - 64 * hf, 0), 64);
+        uint64_t am = own == 64 ? ~0ull : (1ull << own) - 1ull;
+        if (tree) am &= anc;
+        const uint32_t w[2] = {static_cast<uint32_t>(am), static_cast<uint32_t>(am >> 32)};
 #pragma unroll
-        for (int k = 0; k < 64; ++k) {
-          const bool v = (64 * hf + k < valid) && ((am >> k) & 1ull);
-          x[k] = v ? x[k] : -INFINITY;
-        }
+        for (int k = 0; k < 64; ++k) x[k] = (w[k >> 5] >> (k & 31)) & 1u ? x[k] : -INFINITY;
       }
+      float m2[2] = {fmaxf(x[0], x[1]), fmaxf(x[2], x[3])};   // two chains of maxima
 #pragma unroll
-      for (int k = 0; k < 64; k += 2) mt = fmaxf(fmaxf(mt, x[k]), x[k + 1]);
+      for (int k = 4; k < 64; k += 4)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) m2[q] = fmaxf(fmaxf(m2[q], x[k + 2 * q]), x[k + 2 * q + 1]);
+      mt = fmaxf(m2[0], m2[1]);
       s_mx[e][hf][row] = mt;
     }
     // probe S of the next tile now (non-blocking), so that the barrier's
