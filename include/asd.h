@@ -322,8 +322,10 @@ int32_t asd_lm_head_variant(const asd_dims* dims, int32_t total_nodes, const voi
  * (a diagnostic query; no counterpart in the paper; nothing is launched): 1 the
  * bf16 split-KV kernel beside the LM head (up to 128 nodes), 2 the tensor-core
  * kernel with one 128-row query tile per CTA, 3 the tensor-core kernel with two
- * query tiles per CTA in ping-pong (when its 256-row items fill at least two
- * waves of CTAs), 4 the fp32 kernel, 0 for invalid arguments.
+ * query tiles per CTA in ping-pong (when the sequences have more than 128 query
+ * rows on average and the 256-row items fill 5/6 to 1 or more than 1.5 waves of
+ * CTAs, or 1 to 1.5 with pages of at most 32 tokens), 4 the fp32 kernel, 0 for
+ * invalid arguments.
  * Where the answer is 1, a step whose contexts turn out longer than the LM head
  * hides runs form 2 behind it instead (the device decides from ctx_len), and
  * asd_tree_attention by itself, without an LM head to share the SMs with,

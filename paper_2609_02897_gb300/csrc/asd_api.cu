@@ -148,7 +148,8 @@ WsLayout layout(const asd_dims& d, int T, int nsm) {
   // more than one 128-node tile: the LM head (wide kernel) leaves no room on
   // its SMs, attention runs after it on the tensor-core kernel, unsplit
   L.attn_tc = (d.dtype == ASD_BF16 && T > kAttnTcRows) ? 1 : 0;
-  if (L.attn_tc && attention_pingpong(d.batch, d.num_kv_heads, G, T, nsm)) L.attn_tc = 2;
+  if (L.attn_tc && attention_pingpong(d.batch, d.num_kv_heads, G, T, d.page_size, nsm))
+    L.attn_tc = 2;
   size_t off = 0;
   L.status = off;      off = align256(off + 16);
   L.seq_flags = off;   off = align256(off + 4 * static_cast<size_t>(d.batch));

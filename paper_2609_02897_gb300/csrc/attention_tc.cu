@@ -1490,13 +1490,27 @@ size_t attention_tc_smem_bytes(int head_dim, bool pingpong) {
   return 1024 + static_cast<size_t>(head_dim == 64 ? TcGeom<64>::kBytes : TcGeom<128>::kBytes);
 }
 
-bool attention_pingpong(int batch, int num_kv_heads, int G, int total_nodes, int nsm) {
-  // the ping-pong kernel does two query tiles per CTA: it pays once its items
-  // fill at least two waves of CTAs (measured: 1.2x the single-tile kernel's
-  // work per SM; with fewer items the single-tile kernel keeps more SMs busy)
+// A pair of query tiles takes 1.7 times as long as one tile on another SM does
+// (1.4 with small pages, where the copies of K and V count), so the line lies in
+// the waves of CTAs: measured with 8 KV heads, G = 4, 152 SMs, one tile against
+// two, contiguous unless said.
+//   above 1.5 waves of pairs: 16 x 128 nodes 90.0 / 77.0 us, 24 x 128 133.6 /
+//     114.6, 32 x 60 at contexts 1000-4000 109.7 / 96.1, 48 x 33 149.5 / 124.5
+//   1 to 1.5 (three waves of single tiles against two of pairs): 12 x 128
+//     68.0 / 75.7, pages of 64 75.0 / 77.5, of 32 79.9 / 77.7, of 16 90.1 / 78.2;
+//     24 x 60 with pages of 16 89.7 / 78.8
+//   up to 1: 8 x 128 nodes 45.8 / 39.0, ragged 16 sequences of 20-100 nodes
+//     (0.9 of a wave) 68.3 / 65.7, but 15 of them (0.78) 54.0 / 63.7: the single
+//     tiles' second wave is then short
+//   128 rows per sequence or fewer leave the second tile empty: 128 x 20 nodes
+//     153.8 / 157.6, 64 x 31 83.6 / 84.5
+bool attention_pingpong(int batch, int num_kv_heads, int G, int total_nodes, int page_size,
+                        int nsm) {
   const long long rows = static_cast<long long>(total_nodes) * G;
+  if (batch <= 0 || rows <= static_cast<long long>(batch) * kRows) return false;
   const long long items = static_cast<long long>(num_kv_heads) * ((rows + kPPRows - 1) / kPPRows);
-  return batch > 0 && items >= 2LL * nsm;
+  if (items > nsm && 2 * items <= 3LL * nsm) return page_size > 0 && page_size <= 32;
+  return 6 * items >= 5LL * nsm;
 }
 
 bool attention_q_tma_ok(int G) { return G >= 1 && kRows % G == 0; }

@@ -137,12 +137,13 @@ int attention_keys_per_tile();   // context keys per K/V tile = TMA box rows
 // tm_q (with p.q_tma, where attention_q_tma_ok(G)): a 3D map over
 // q [T, Hq, D] with boxes of 64 columns x G heads x kAttnTcRows / G nodes.
 // pingpong: the two-query-tile form (256 rows per CTA: one tile's MMAs run
-// during the other's softmax), chosen by attention_pingpong() when its items
-// fill at least two waves of CTAs.
+// during the other's softmax), chosen by attention_pingpong() by how many
+// waves of CTAs its items make.
 constexpr int kAttnTcRows = 128;   // query rows per CTA (per tile of the ping-pong form)
 constexpr int kAttnTcKeys = 128;   // keys per tile
 size_t attention_tc_smem_bytes(int head_dim, bool pingpong);
-bool attention_pingpong(int batch, int num_kv_heads, int G, int total_nodes, int nsm);
+bool attention_pingpong(int batch, int num_kv_heads, int G, int total_nodes, int page_size,
+                        int nsm);
 // Partial rows that the one-tile kernel can use to cut sequences into chunks
 // (0: the items of these dims and nodes fill the GPU anyway).
 long long attention_split_rows(const asd_dims& d, int total_nodes, int nsm);

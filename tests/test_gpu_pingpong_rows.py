@@ -1,7 +1,9 @@
 """The ping-pong attention's two query tiles at the row counts where they
 change (one tile only, a full first tile, one row in the second, both full) in
-one ragged batch, against a plain PyTorch fp32 reference.  Keys grow along the
-context, so that the running maximum is raised, and O rescaled, more than once."""
+one ragged batch, against a plain PyTorch fp32 reference, with several waves of
+items and with about one.  Keys grow along the context, so that the running
+maximum is raised, and O rescaled, more than once.  And which form a call takes
+on both sides of every line of the rule."""
 import pytest
 
 from test_gpu_attention_ragged import _call, _check_close, _inputs, _reference
@@ -9,11 +11,12 @@ from test_gpu_attention_ragged import _call, _check_close, _inputs, _reference
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("D,page,Hq", [(128, 0, 32), (128, 16, 32), (64, 0, 32), (64, 64, 24)])
-def test_row_counts_of_the_two_query_tiles(D, page, Hq):
+@pytest.mark.parametrize("B,D,page,Hq", [(64, 128, 0, 32), (64, 128, 16, 32), (64, 64, 0, 32),
+                                         (64, 64, 64, 24), (24, 128, 16, 32), (32, 64, 0, 32)])
+def test_row_counts_of_the_two_query_tiles(B, D, page, Hq):
     import torch
     from paper_2609_02897_gb300 import asd
-    Hkv, B, N, cap = 8, 64, 128, 1024
+    Hkv, N, cap = 8, 128, 1024
     nodes = [(1, 31, 32, 33, 43, 64, 127, 128)[b % 8] for b in range(B)]
     ctx = [(0, 1, 127, 128, 129, 300, 640, 895)[(b // 8 + b) % 8] for b in range(B)]
     full = _inputs(B, N, ctx, page, Hq, Hkv, D, cap, 5)
@@ -43,3 +46,22 @@ def test_row_counts_of_the_two_query_tiles(D, page, Hq):
             one[k] = d[k] if page else d[k][b:b + 1]
         _check_close(out[s:s + n], _reference(one, 1, n, ctx[b:b + 1], page, Hq, Hkv, D))
         s += n
+
+
+def test_which_form_a_call_takes():
+    import torch
+    from paper_2609_02897_gb300 import asd
+    nsm = torch.cuda.get_device_properties(0).multi_processor_count
+
+    def form(items, page=0, batch=1):
+        # one KV head and G = 2: an item is 128 nodes
+        dims = asd.make_dims(max(batch, items), 2, 1, 128, 64, 64, asd.ASD_BF16, page, 1024,
+                             64 if page else 0, 128, 8)
+        return asd.asd_attention_variant(dims, 128 * items)
+
+    low, half = -(-5 * nsm // 6), 3 * nsm // 2
+    assert [form(low - 1), form(low), form(nsm), form(nsm + 1), form(half), form(half + 1)] == \
+        [2, 3, 3, 2, 2, 3]
+    assert [form(low - 1, 16), form(nsm + 1, 32), form(half, 16), form(half, 64)] == [2, 3, 3, 2]
+    # 128 rows per sequence on average: the second query tile would stay empty
+    assert form(4 * nsm) == 3 and form(4 * nsm, batch=8 * nsm) == 2
