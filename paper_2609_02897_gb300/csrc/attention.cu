@@ -812,18 +812,20 @@ long long attention_co_tiles_max(const asd_dims& d, int n_parts, int nsm) {
 }
 
 int attention_co_tiles_limit(const asd_dims& d) {
-  // A tile takes the kernel about 1.2 us at D = 128 (0.9 at 64), the LM head
-  // streams W at about 6.4 TB/s, and the tensor-core kernel needs about a
-  // quarter of this one's time: it wins from 4/3 of the LM head's time on, and
-  // beside a short LM head from about the time that its own launches take.
-  // Steps of a Llama-3.1-8B-shaped LM head (limit 182 tiles), always this kernel
-  // before and the rule now: 60 nodes at context 24576 276 -> 218 us, 65536
-  // 628 -> 254; 8 x 8 nodes at 16384 349 -> 266, 32768 631 -> 339; under the
-  // limit (60 nodes at 16384: 205) the same.  Deciding on the device costs a
-  // step of short contexts in a roomy cache 1.5 to 5 us.
+  // Beside the LM head, which streams W at about 6.4 TB/s, a tile takes the
+  // kernel 1.2 us (contiguous), 1.6 (pages of 32 tokens or more) or 1.9 at
+  // D = 128 and starts late; the tensor-core kernel needs about a quarter of
+  // that behind the LM head.  Measured, this kernel against the rule's other
+  // side: LM head of 82 us, 11 x 4 nodes, 64 heads, at 53 tiles: contiguous 101.8
+  // / 114.5 us, pages of 64 123.2 / 116.5, of 16 138.9 / 120.0, at 39 tiles of
+  // 16-token pages 112.6 / 115.9.  LM head of 164 us: 60 nodes at 130 tiles
+  // contiguous 203.3 / 203.9, pages of 64 258.4 / 205.9, of 16 299.4 / 211.1; 11 x
+  // 4 nodes at 76 tiles, pages of 16, 200.0 / 205.4.  Deciding on the device
+  // costs a step of short contexts in a roomy cache 1.5 to 5 us.
   const double lm_us = 2.0 * d.vocab * static_cast<double>(d.hidden) / 6.4e6;
-  const double tile_us = d.head_dim == 128 ? 1.2 : 0.9;
-  return static_cast<int>(std::max(16.0, std::min(4.0 / 3.0 * lm_us / tile_us, 1e6)));
+  double tiles_per_us = d.page_size == 0 ? 0.8 : d.page_size >= kKeysPerTile ? 0.6 : 0.5;
+  if (d.head_dim == 64) tiles_per_us *= 4.0 / 3.0;   // a tile of half the bytes: 0.9 us, not 1.2
+  return static_cast<int>(std::max(16.0, std::min(tiles_per_us * lm_us, 1e6)));
 }
 
 static dim3 attn_grid(const AttnParams& p) {
