@@ -283,6 +283,7 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
   a.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(d.head_dim)));
   a.nsm = device_sm_count();
   a.co_tiles = -1;
+  a.p_two = c.L.attn_tc ? 0 : 1;
   if (d.dtype != ASD_BF16)
     return launch_attention_f32(a, c.st) == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
   // up to 128 nodes the mma.sync kernel runs beside the LM head of a verify

@@ -472,6 +472,44 @@ __device__ __forceinline__ float exp2_tile(const float* x, float c, float mu,
   return lo + hi;
 }
 
+// The same, P as the sum of two bf16 numbers.  Calls of up to 128 nodes hand half
+// of P to the tensor cores so (TWO below): the mma.sync kernel, which took them
+// before this one did, rescales to the running maximum of every 32 keys, which
+// makes the largest weights exact, and with P in one term this kernel's error
+// against 64 bits was up to 7 % above its.  Half of P in two terms leaves it 6 to
+// 14 % below; all of P 19 to 25 %, for twice the time.  8 nodes at context 32768:
+// one term 31.2 us, half 32.3, all 33.4; 128 nodes 90, 102, 117.
+// `hi` is cut off behind its 8 bits, `lo` the rest rounded to bf16, so that hi + lo is
+// within 2^-16 of P.  `lo` is taken from P (1 + 2^-20), which keeps it above zero
+// wherever P is: an infinite V then stays infinite (0 * inf would be NaN); the sum
+// is scaled likewise.
+constexpr float kTwoTermScale = 1.f + 0x1p-20f;
+template <int N>
+__device__ __forceinline__ float exp2_tile_two(const float* x, float c, float mu,
+                                               uint32_t (&hi)[N / 2], uint32_t (&lo)[N / 2]) {
+  const uint64_t c2 = pack_f32x2(c, c), nmu2 = pack_f32x2(-mu, -mu);
+  const uint64_t k2 = pack_f32x2(kTwoTermScale, kTwoTermScale);
+  uint64_t sum = 0ull;
+#pragma unroll
+  for (int k = 0; k < N; k += 2) {
+    float y0, y1;
+    unpack_f32x2(fma_f32x2(pack_f32x2(x[k], x[k + 1]), c2, nmu2), y0, y1);
+    const float p0 = ex2_approx(y0), p1 = ex2_approx(y1);
+    const uint64_t p2 = pack_f32x2(p0, p1);
+    sum = add_f32x2(sum, p2);
+    const uint32_t u0 = __float_as_uint(p0), u1 = __float_as_uint(p1);
+    hi[k / 2] = __byte_perm(u0, u1, 0x7632);
+    const uint64_t nhi2 = pack_f32x2(__uint_as_float((u0 & 0xffff0000u) ^ 0x80000000u),
+                                     __uint_as_float((u1 & 0xffff0000u) ^ 0x80000000u));
+    unpack_f32x2(fma_f32x2(p2, k2, nhi2), y0, y1);
+    __nv_bfloat162 h = __floats2bfloat162_rn(y0, y1);
+    lo[k / 2] = *reinterpret_cast<uint32_t*>(&h);
+  }
+  float a, b;
+  unpack_f32x2(sum, a, b);
+  return (a + b) * kTwoTermScale;
+}
+
 // Softmax warps (eight): warp w handles TMEM lane quarter w % 4 (its 32 query
 // rows, one thread per row) and half h = (w - 2) / 4 of every tile's 128 keys.
 // Per tile: read its 64 S columns, mask, exchange the row's partial max with
@@ -482,7 +520,7 @@ __device__ __forceinline__ float exp2_tile(const float* x, float c, float mu,
 // until the end.  Returns false (uniformly over the eight warps) when a
 // bounded wait gave up; otherwise m_out and l_out are the row's reference max
 // and sum, with O complete in TMEM.
-template <int D>
+template <int D, bool TWO>
 __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it, uint32_t tmem,
                                              uint8_t* gbase, int* s_par, uint64_t (*s_anc)[2],
                                              float (*s_mx)[2][kRows], float (*s_l)[kRows],
@@ -600,9 +638,18 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
       m_ref = mn;
     }
     const float mu = (m_ref == -INFINITY) ? 0.f : m_ref;
-    uint32_t pk[32];
-    l += exp2_tile<64>(x, c, mu, pk);
-    tmem_st32u(sb + 32 * hf, pk);
+    if (TWO) {   // the first 32 of this half's keys in two terms
+      uint32_t hi[16], lo[16], pk[16];
+      l += exp2_tile_two<32>(x, c, mu, hi, lo);
+      tmem_st16u(sb + 32 * hf, hi);
+      tmem_st16u(sb + kKeys / 2 + 16 * hf, lo);
+      l += exp2_tile<32>(x + 32, c, mu, pk);
+      tmem_st16u(sb + 32 * hf + 16, pk);
+    } else {
+      uint32_t pk[32];
+      l += exp2_tile<64>(x, c, mu, pk);
+      tmem_st32u(sb + 32 * hf, pk);
+    }
     if (valid < kKeys) {
       // ragged tile: V rows past the last valid key may hold anything; zero
       // them so that 0 * V stays 0, once the V tile has landed (it comes
@@ -654,7 +701,8 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
   return true;
 }
 
-template <int D>
+// TWO: half of P in two bf16 terms (AttnParams::p_two).
+template <int D, bool TWO>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                    const __grid_constant__ CUtensorMap tm_tk,
@@ -833,6 +881,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_mma_ts(tmem, tmem + kSCol0 + b * kKeys + kk * 8,
                       sw128_desc_mn(vst + kk * 2048, kKeys * 128, 1024), idesc_o,
                       (j > 0 || kk > 0) ? 1u : 0u);
+          if (TWO)   // second terms of keys 0-31 and 64-95
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              tc_mma_ts(tmem, tmem + kSCol0 + b * kKeys + kKeys / 2 + i * 8,
+                        sw128_desc_mn(vst + ((i & 1) + 4 * (i >> 1)) * 2048, kKeys * 128, 1024),
+                        idesc_o, 1u);
           tc_commit(smem_u32(&s_pv_done[b]));
           tc_commit(smem_u32(&s_v_empty[stage]));
         }
@@ -849,7 +903,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    ok = softmax_role<D>(p, it, tmem, gbase, s_par, s_anc, s_mx, s_l, &s_q_ready, s_s_full, s_p_full,
+    ok = softmax_role<D, TWO>(p, it, tmem, gbase, s_par, s_anc, s_mx, s_l, &s_q_ready, s_s_full, s_p_full,
                          s_pv_done, s_v_full, &s_abort, budget, m_row, l_row);
   }
 
@@ -1533,7 +1587,8 @@ cudaError_t launch_attention_tc(const AttnParams& p, const CUtensorMap& tm_k,
       std::max<long long>(blocks * p.Hkv, p.part_cap > 0 ? p.nsm : 0);
   if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
   auto* k = pingpong ? (p.D == 64 ? attn_pp_kernel<64> : attn_pp_kernel<128>)
-                     : (p.D == 64 ? attn_tc_kernel<64> : attn_tc_kernel<128>);
+           : p.p_two ? (p.D == 64 ? attn_tc_kernel<64, true> : attn_tc_kernel<128, true>)
+                     : (p.D == 64 ? attn_tc_kernel<64, false> : attn_tc_kernel<128, false>);
   err = set_smem_attrs(k, smem);
   if (err != cudaSuccess) return err;
   err = launch_pdl(k, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), smem, s, tm_k, tm_v, tm_tk,

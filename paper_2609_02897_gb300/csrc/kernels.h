@@ -86,6 +86,9 @@ struct AttnParams {
   // takes the step, beyond which the tensor-core kernel does after it (both
   // are launched and decide alike, attention_beside_lm_head); -1: no choice
   int co_tiles;
+  // one-tile tensor-core kernel: half of P goes to the P.V MMA in two bf16 terms
+  // (calls of up to 128 nodes, which another kernel took before)
+  int p_two;
   // one-tile tensor-core kernel: partial results of sequences cut into chunks
   long long part_cap;       // rows that part_o / part_ml hold (0: no splitting)
   float* part_o;            // [part_cap][D]: a chunk's unnormalised output row
