@@ -328,10 +328,11 @@ int32_t asd_lm_head_variant(const asd_dims* dims, int32_t total_nodes, const voi
  * invalid arguments.
  * Where the answer is 1, a step whose contexts turn out longer than the LM head
  * hides runs form 2 behind it instead (the device decides from ctx_len), and
- * asd_tree_attention by itself, without an LM head to share the SMs with,
- * always runs form 2 (same semantics, other roundings).  Form 2
- * may cut long contexts into chunks, whose length follows the batch's context
- * lengths.
+ * asd_tree_attention by itself, without an LM head to share the SMs with, runs
+ * form 2 as well unless many sequences with short contexts make it several items
+ * per SM (by the cache's capacity, or decided on the device); same semantics,
+ * other roundings.  Form 2 may cut long contexts into chunks, whose length
+ * follows the batch's context lengths.
  */
 int32_t asd_attention_variant(const asd_dims* dims, int32_t total_nodes);
 

@@ -287,15 +287,21 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
   if (d.dtype != ASD_BF16)
     return launch_attention_f32(a, c.st) == cudaSuccess ? ASD_OK : ASD_ERR_CUDA;
   // up to 128 nodes the mma.sync kernel runs beside the LM head of a verify
-  // step, unless the contexts may be longer than the LM head hides: then both
-  // kernels are launched and the context lengths decide which one works.
-  // With the SMs to itself the tensor-core kernel is the faster one at every
-  // size.
-  const bool beside = in_step && !c.L.attn_tc;
-  bool tc = !beside;
-  if (beside && attention_co_tiles_max(d, c.L.n_parts, a.nsm) > attention_co_tiles_limit(d)) {
-    a.co_tiles = attention_co_tiles_limit(d);
-    tc = true;
+  // step, unless the contexts may be longer than the LM head hides, and takes a
+  // call by itself that makes several items per SM, unless the contexts may be
+  // too long for that: then both kernels are launched and the context lengths
+  // decide which one works.
+  bool mma = false, tc = true;
+  if (in_step && !c.L.attn_tc) {
+    mma = true;
+    tc = attention_co_tiles_max(d, c.L.n_parts, a.nsm) > attention_co_tiles_limit(d);
+    if (tc) a.co_tiles = attention_co_tiles_limit(d);
+  } else if (!c.L.attn_tc) {
+    const AloneRule rule = attention_alone_rule(d, c.T, a.nsm);
+    mma = rule.tiles >= 0;
+    tc = !mma || rule.both;
+    if (rule.both) a.co_tiles = rule.tiles;
+    a.alone = 1;
   }
   // maps over the context cache's rows with boxes of `keys` rows at most
   auto cache_maps = [&](int keys, CUtensorMap* tk, CUtensorMap* tv) {
@@ -312,13 +318,21 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
     return make_tmap_bf16(tk, k_cache, d.head_dim, rows, static_cast<uint32_t>(box)) &&
            make_tmap_bf16(tv, v_cache, d.head_dim, rows, static_cast<uint32_t>(box));
   };
-  CUtensorMap tk, tv;
-  if (beside) {
-    if (!cache_maps(attention_keys_per_tile(), &tk, &tv) ||
-        launch_attention_bf16(a, tk, tv, c.st) != cudaSuccess)
-      return ASD_ERR_CUDA;
+  auto run_mma = [&]() {
+    CUtensorMap tk, tv;
+    return cache_maps(attention_keys_per_tile(), &tk, &tv) &&
+                   launch_attention_bf16(a, tk, tv, c.st) == cudaSuccess
+               ? ASD_OK
+               : ASD_ERR_CUDA;
+  };
+  // beside the LM head this kernel comes first; where both are launched for a call
+  // by itself it comes last, so that its CTAs, if they have no work, pass while the
+  // tensor-core kernel's last wave runs
+  if (mma && (in_step || !tc)) {
+    const asd_status st = run_mma();
+    if (st != ASD_OK || !tc) return st;
   }
-  if (!tc) return ASD_OK;
+  CUtensorMap tk, tv;
   CUtensorMap ttk, ttv, tq;
   if (!cache_maps(kAttnTcKeys, &tk, &tv) ||
       !make_tree_tmap_bf16(&ttk, tree_k, d.head_dim, d.num_kv_heads, c.T, kAttnTcKeys) ||
@@ -347,8 +361,9 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
       a.part_o = ws_at<float>(c.ws, rows_at + sizeof(float2) * static_cast<size_t>(a.part_cap));
     }
   }
-  return launch_attention_tc(a, tk, tv, ttk, ttv, tq, pingpong, c.st) == cudaSuccess ? ASD_OK
-                                                                                    : ASD_ERR_CUDA;
+  if (launch_attention_tc(a, tk, tv, ttk, ttv, tq, pingpong, c.st) != cudaSuccess)
+    return ASD_ERR_CUDA;
+  return mma && !in_step ? run_mma() : ASD_OK;
 }
 
 // True when `w` is device memory of the current device (the only memory the

@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(128) attn_bf16_kernel(const __grid_constant__ 
   // ancestor masks itself and keeps every access inside the caller's arrays
   // whatever the inputs hold (the preparation kernel reports malformed ones;
   // the outputs of such a sequence are then unspecified).
-  if (p.co_tiles >= 0 && !attention_beside_lm_head(p)) {   // the tensor-core kernel's step
+  if (p.co_tiles >= 0 && !attention_takes_mma(p)) {   // the tensor-core kernel's call
     pdl_wait();
     return;
   }
@@ -826,6 +826,41 @@ int attention_co_tiles_limit(const asd_dims& d) {
   double tiles_per_us = d.page_size == 0 ? 0.8 : d.page_size >= kKeysPerTile ? 0.6 : 0.5;
   if (d.head_dim == 64) tiles_per_us *= 4.0 / 3.0;   // a tile of half the bytes: 0.9 us, not 1.2
   return static_cast<int>(std::max(16.0, std::min(tiles_per_us * lm_us, 1e6)));
+}
+
+AloneRule attention_alone_rule(const asd_dims& d, int total_nodes, int nsm) {
+  // The tensor-core kernel has one CTA per SM, whose start takes it some 7 us, the
+  // mma.sync kernel four, of 5 us together.  With one item per SM at most the former
+  // wins at once; with k the latter does up to about (23 k - 18) / (k + 1.6) key
+  // tiles of 32, the tree's among them.  This kernel / the tensor-core one,
+  // contiguous, D = 128, by context:
+  //   20 x 4 nodes, 160 items    188: 18.1 / 20.1 us   250: 20.7 / 19.9
+  //   64 x 2, 512 items          250: 39.0 / 40.6      380: 51.2 / 47.4
+  //   128 x 1, 1024 items          1: 28.6 / 64.7      380: 77.5 / 84.7   760: 128 / 109
+  //   64 x 2, 2048 items (MHA)   500: 163 / 172        760: 223 / 202
+  // pages of 16: 20 x 4 120: 18.9 / 19.2, 188: 23.2 / 22.1; 128 x 1 250: 79.0 /
+  // 82.2, 380: 105 / 92.7.  D = 64: 20 x 4 380: 19.9 / 20.3, 500: 23.7 / 22.3;
+  // 128 x 1 760: 75.5 / 98.6, 1020: 94.9 / 113.
+  const int G = d.num_q_heads / d.num_kv_heads;
+  const long long rows = static_cast<long long>(total_nodes) * G;
+  const long long items =
+      d.num_kv_heads * std::max<long long>(d.batch, (rows + kAttnTcRows - 1) / kAttnTcRows);
+  if (items <= nsm) return {-1, false};
+  const double k = static_cast<double>((items + nsm - 1) / nsm);
+  const double by_cache = (d.page_size == 0 ? 1.0 : d.page_size >= kKeysPerTile ? 0.8 : 0.65) *
+                          (d.head_dim == 64 ? 2.0 : 1.0);
+  const int tiles = static_cast<int>(by_cache * (23.0 * k - 18.0) / (k + 1.6));
+  const long long most = (static_cast<long long>(d.ctx_max) + kKeysPerTile - 1) / kKeysPerTile +
+                         (d.max_nodes + kKeysPerTile - 1) / kKeysPerTile;
+  if (most <= tiles) return {tiles, false};
+  // A cache that holds more: the contexts decide, and the grid of the kernel that
+  // does not take the call costs 1 to 2 us (mma.sync) or 1.6 k us (tensor cores, off
+  // the limit).  Up to k = 2 that is what the choice would gain (20 x 4 nodes at
+  // context 60 in a cache of 8192: 17.3 us with the choice, 17.7 without).  128 x 1
+  // at context 120, 4096 slots: 53.9 us, 64 on the tensor cores; 1000: 128.0 us,
+  // 125.4 without the choice.
+  if (k < 3) return {-1, false};
+  return {static_cast<int>(by_cache * (17.0 * k - 18.0) / (k + 1.6)), true};
 }
 
 static dim3 attn_grid(const AttnParams& p) {

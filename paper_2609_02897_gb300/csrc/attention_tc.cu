@@ -148,6 +148,7 @@ struct PlanSmem {
   int chunks[kOrderMax];
   int cut_ctas[kMaxChunks];   // CTAs and partial rows when the longest sequence is
   int cut_part[kMaxChunks];   // cut into 1, 2, ... chunks
+  AloneTiles alone[kMaxNodes / 32];   // a call by itself: sums over 32 sequences each
   int seq, first, part0;   // the sequence of this CTA, its first CTA and partial row
 };
 
@@ -262,7 +263,27 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
       s.chunks[q] = 1;
       s.order[q] = make_int2(order_key(s.tiles[q], q), s.items[q]);
     }
+    const bool choice = p.alone && p.co_tiles >= 0;   // B <= 128: a sequence per thread
+    if (choice && threadIdx.x < kMaxNodes) {
+      const int q = threadIdx.x;
+      AloneTiles a{0, 0, 0};
+      if (q < p.B) a = alone_tiles(p, min(max(s.n[q], 0), kMaxNodes), s.ctx[q]);
+      a = {__reduce_max_sync(0xffffffffu, a.longest), __reduce_add_sync(0xffffffffu, a.total),
+           __reduce_add_sync(0xffffffffu, a.blocks)};
+      if ((q & 31) == 0) s.alone[q >> 5] = a;
+    }
     __syncthreads();
+    // The mma.sync kernel's call: decided here, where the extents are at hand,
+    // since in front of every CTA's set-up (attention_takes_mma) it cost the several
+    // waves of such a call 1.3 us each.
+    if (choice) {
+      AloneTiles a = s.alone[0];
+#pragma unroll
+      for (int w = 1; w < kMaxNodes / 32; ++w)
+        a = {max(a.longest, s.alone[w].longest), a.total + s.alone[w].total,
+             a.blocks + s.alone[w].blocks};
+      if (alone_takes_mma(p, a)) return false;
+    }
     if (p.part_cap > 0) {
       const int len = chunk_length(p, s);
       const float inv = __frcp_rn(static_cast<float>(len));
@@ -730,7 +751,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ PlanSmem s_plan;
 
   pdl_launch_dependents();
-  if (p.co_tiles >= 0 && attention_beside_lm_head(p)) {   // the mma.sync kernel's step
+  // the mma.sync kernel's step (a call by itself: make_item)
+  if (p.co_tiles >= 0 && !p.alone && attention_takes_mma(p)) {
     pdl_wait();
     return;
   }
@@ -1007,7 +1029,7 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const AttnPar
   const int w = (threadIdx.x >> 5) % kMergeWarps, rl = (threadIdx.x >> 5) / kMergeWarps;
   const int s0 = p.cu_nodes[b], n = p.cu_nodes[b + 1] - s0, R = n * p.G;
   pdl_wait();
-  if (p.co_tiles >= 0 && attention_beside_lm_head(p)) return;   // nothing was cut
+  if (p.co_tiles >= 0 && attention_takes_mma(p)) return;   // nothing was cut
   if (n <= 0 || n > kMaxNodes || s0 < 0 || s0 + n > p.T || static_cast<int>(blockIdx.x) * kMergeRows >= R)
     return;
   const int2 plan = __ldcg(p.plan + b);

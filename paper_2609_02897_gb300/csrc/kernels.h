@@ -81,11 +81,14 @@ struct AttnParams {
   float scale_log2;         // log2(e) / sqrt(D)
   int q_tma;                // tensor-core kernels: the query tiles by TMA (tm_q)
   int nsm;                  // SMs of the device
-  // steps of up to 128 nodes whose cache could hold more keys than the LM head
-  // hides: the 32-key tiles up to which the mma.sync kernel beside the LM head
-  // takes the step, beyond which the tensor-core kernel does after it (both
-  // are launched and decide alike, attention_beside_lm_head); -1: no choice
+  // bf16 calls of up to 128 nodes that the context lengths decide about: the
+  // 32-key tiles up to which the mma.sync kernel takes the call, beyond which the
+  // tensor-core kernel does (both are launched and decide alike,
+  // attention_takes_mma); -1: no choice.  A step whose cache could hold more keys
+  // than the LM head hides (attention_co_tiles_limit), or, with `alone`, a call
+  // without an LM head and with several items per SM (attention_alone_rule)
   int co_tiles;
+  int alone;
   // one-tile tensor-core kernel: half of P goes to the P.V MMA in two bf16 terms
   // (calls of up to 128 nodes, which another kernel took before)
   int p_two;
@@ -95,16 +98,41 @@ struct AttnParams {
   float2* part_ml;          // [part_cap]: its reference max (log2 domain) and sum
   int2* plan;               // [B]: first partial row and chunks of a sequence
 };
-// Whether this step's attention runs beside the LM head (p.co_tiles): the key
+// Whether the mma.sync kernel takes this call (p.co_tiles): in a step the key
 // tiles of its longest split, or an even share of all of them per SM, against
-// the limit.  Every lane of a warp calls it; the answer is uniform over the
-// grid.  B <= 128 here.
+// the limit; in a call by itself the mean of the key tiles over the query row
+// blocks, and half of the longest.  Every lane of a warp calls it; the answer is
+// uniform over the grid.  B <= 128 here; unrolled, so that the loads of all
+// sequences are in flight at once.
 constexpr int kCoKeys = 32, kCoRows = 64;   // keys per tile, query rows per CTA
-__device__ __forceinline__ bool attention_beside_lm_head(const AttnParams& p) {
-  int longest = 0, total = 0;
-  for (int q = threadIdx.x & 31; q < p.B; q += 32) {
+struct AloneTiles {   // sums of a call by itself
+  int longest, total, blocks;
+};
+// Sequence of n nodes and context ctx: query row blocks and key tiles.
+__device__ __forceinline__ AloneTiles alone_tiles(const AttnParams& p, int n, int ctx) {
+  const int rows = (n * p.G + kCoRows - 1) / kCoRows;
+  // key tiles cut off far beyond any limit and far from overflow
+  const int t = min((ctx + kCoKeys - 1) / kCoKeys + (n + kCoKeys - 1) / kCoKeys, 1 << 12);
+  return {t, rows * t, rows};
+}
+__device__ __forceinline__ bool alone_takes_mma(const AttnParams& p, const AloneTiles& a) {
+  return a.longest <= 2 * p.co_tiles && a.total <= p.co_tiles * a.blocks;
+}
+__device__ __forceinline__ bool attention_takes_mma(const AttnParams& p) {
+  int longest = 0, total = 0, blocks = 0;
+#pragma unroll
+  for (int k = 0; k < kMaxNodes / 32; ++k) {
+    const int q = (threadIdx.x & 31) + 32 * k;
+    if (q >= p.B) continue;
     const int n = min(max(p.cu_nodes[q + 1] - p.cu_nodes[q], 0), kMaxNodes);
     const int ctx = min(max(p.ctx_len[q], 0), p.ctx_max);
+    if (p.alone) {
+      const AloneTiles a = alone_tiles(p, n, ctx);
+      longest = max(longest, a.longest);
+      total += a.total;
+      blocks += a.blocks;
+      continue;
+    }
     const int tree = (n + kCoKeys - 1) / kCoKeys;
     const int tiles = (ctx + kCoKeys - 1) / kCoKeys;
     longest = max(longest, (tiles + p.n_parts - 1) / p.n_parts + tree);
@@ -115,7 +143,9 @@ __device__ __forceinline__ bool attention_beside_lm_head(const AttnParams& p) {
   }
   longest = __reduce_max_sync(0xffffffffu, longest);
   total = __reduce_add_sync(0xffffffffu, total);
-  return max(longest, total) <= p.co_tiles;
+  if (!p.alone) return max(longest, total) <= p.co_tiles;
+  blocks = __reduce_add_sync(0xffffffffu, blocks);
+  return alone_takes_mma(p, {longest, total, blocks});
 }
 // bf16 path: tensor-core (mma.sync) split-KV kernel fed by TMA; tm_k / tm_v are
 // 2D tensor maps over the context cache rows (box 64 columns x
@@ -129,6 +159,13 @@ int attention_row_blocks(int max_nodes, int G);
 // the cache's capacity, and up to how many of them it is the faster choice.
 long long attention_co_tiles_max(const asd_dims& d, int n_parts, int nsm);
 int attention_co_tiles_limit(const asd_dims& d);
+// The same limit for a call by itself (-1: the tensor-core kernel takes it), and
+// whether the contexts may exceed it, so that both kernels are launched.
+struct AloneRule {
+  int tiles;
+  bool both;
+};
+AloneRule attention_alone_rule(const asd_dims& d, int total_nodes, int nsm);
 int attention_keys_per_tile();   // context keys per K/V tile = TMA box rows
 // bf16 path on the 5th-generation tensor cores, where attention has the SMs to
 // itself (a standalone call, or a step of more than 128 tree nodes): one CTA
