@@ -149,6 +149,7 @@ struct PlanSmem {
   int cut_ctas[kMaxChunks];   // CTAs and partial rows when the longest sequence is
   int cut_part[kMaxChunks];   // cut into 1, 2, ... chunks
   AloneTiles alone[kMaxNodes / 32];   // a call by itself: sums over 32 sequences each
+  int past;                // items in all where they are more than the grid's CTAs, else 0
   int seq, first, part0;   // the sequence of this CTA, its first CTA and partial row
 };
 
@@ -226,6 +227,7 @@ template <int ROWS>
 __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSmem& s) {
   const int idx = blockIdx.x;
   int local, ctx, longest;   // longest: key tiles of the sequence's longest chunk
+  if (threadIdx.x == 0) s.past = 0;
   if (p.B > kOrderMax) {   // index order, unsplit
     const int rbmax = (p.max_nodes * p.G + ROWS - 1) / ROWS;
     it.b = idx / (rbmax * p.Hkv);
@@ -310,6 +312,7 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
         const int2 o = s.order[j];
         first += o.x > mine.x ? o.y : 0;
       }
+      if (first + mine.y > static_cast<int>(gridDim.x)) atomicMax(&s.past, first + mine.y);
       if (idx < first || idx >= first + mine.y) continue;
       if (p.part_cap > 0) {
         for (int j = 0; j < p.B; ++j) part += s.order[j].x > mine.x ? s.part[j] : 0;
@@ -352,6 +355,80 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
   it.key_base = t0 * kKeys;
   it.ctx = ctx - it.key_base;
   return true;
+}
+
+// The items past the grid, which has a CTA for every item of sequences that do
+// not overlap: a batch whose cu_nodes run backwards (reported as ASD_ERR_TREE) can
+// make more, and its well-formed sequences keep their outputs.  Plain loops over
+// the keys, a warp per query row, by the eight softmax warps (tid: thread among
+// them) of every CTA when it is done.
+template <int D, int ROWS>
+__device__ __forceinline__ void items_past_grid(const AttnParams& p, PlanSmem& s, int tid) {
+  constexpr int kV = D / 32;   // a lane's columns
+  const int lane = tid & 31;
+  const __nv_bfloat16* kc = static_cast<const __nv_bfloat16*>(p.k_cache);
+  const __nv_bfloat16* vc = static_cast<const __nv_bfloat16*>(p.v_cache);
+  for (int idx = gridDim.x + blockIdx.x; idx < s.past; idx += gridDim.x) {
+    softmax_sync();   // everyone is done with the last item's sequence
+    for (int q = tid; q < p.B; q += kSoftmaxThreads) {
+      int first = 0;
+      for (int j = 0; j < p.B; ++j) first += s.order[j].x > s.order[q].x ? s.order[j].y : 0;
+      if (idx < first || idx >= first + s.order[q].y) continue;
+      s.seq = q;
+      s.first = first;
+      if (idx == first && p.part_cap > 0) p.plan[q] = make_int2(0, 1);   // nothing to merge
+    }
+    softmax_sync();
+    const int b = s.seq, s0 = s.s0[b], R = s.n[b] * p.G, rb = (R + ROWS - 1) / ROWS;
+    const int g = (idx - s.first) / rb, r0 = (idx - s.first - g * rb) * ROWS;
+    for (int r = r0 + (tid >> 5); r < min(r0 + ROWS, R); r += kSoftmaxThreads / 32) {
+      const int node = r / p.G;
+      const size_t row = static_cast<size_t>(s0 + node) * p.Hq + g * p.G + (r - node * p.G);
+      float q[kV], o[kV], m = -INFINITY, l = 0.f;
+#pragma unroll
+      for (int k = 0; k < kV; ++k) {
+        q[k] = to_f32(static_cast<const __nv_bfloat16*>(p.q)[row * D + lane * kV + k]) * p.scale_log2;
+        o[k] = 0.f;
+      }
+      auto key = [&](const __nv_bfloat16* kr, const __nv_bfloat16* vr) {
+        float x = 0.f;
+#pragma unroll
+        for (int k = 0; k < kV; ++k) x = fmaf(q[k], to_f32(kr[lane * kV + k]), x);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        const float mn = fmaxf(m, x);
+        const float al = m == -INFINITY ? 0.f : exp2f(m - mn);
+        const float pe = x == -INFINITY ? 0.f : exp2f(x - mn);
+        l = l * al + pe;
+#pragma unroll
+        for (int k = 0; k < kV; ++k) o[k] = fmaf(pe, to_f32(vr[lane * kV + k]), o[k] * al);
+        m = mn;
+      };
+      for (int j = 0; j < s.ctx[b]; ++j) {
+        size_t at = (static_cast<size_t>(b) * p.Hkv + g) * p.ctx_max + j;
+        if (p.page_size) {
+          const int page = p.page_table[static_cast<size_t>(b) * p.pages_per_seq + j / p.page_size];
+          if (page < 0 || page >= p.num_pages) {
+            set_status(p.status, ASD_ERR_CTX_RANGE);
+            continue;
+          }
+          at = (static_cast<size_t>(page) * p.Hkv + g) * p.page_size + j % p.page_size;
+        }
+        key(kc + at * D, vc + at * D);
+      }
+      for (int u = node; u >= 0;) {   // the node and its ancestors
+        const size_t at = (static_cast<size_t>(s0 + u) * p.Hkv + g) * D;
+        key(static_cast<const __nv_bfloat16*>(p.tree_k) + at,
+            static_cast<const __nv_bfloat16*>(p.tree_v) + at);
+        const int pu = p.parent[s0 + u];
+        u = pu < u ? pu : -1;
+      }
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+      for (int k = 0; k < kV; ++k)
+        static_cast<__nv_bfloat16*>(p.out)[row * D + lane * kV + k] = from_f32<__nv_bfloat16>(o[k] * inv);
+    }
+  }
 }
 
 __device__ __forceinline__ size_t grow_of(const AttnParams& p, const Item& it, int r) {
@@ -1003,6 +1080,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   if (warp == 10) tmem_dealloc(tmem, kTmemCols);
+  if (s_plan.past > 0 && warp >= 2 && warp < 10)
+    items_past_grid<D, kRows>(p, s_plan, threadIdx.x - 64);
   pdl_wait();   // the next kernel's wait covers every earlier kernel
 }
 
@@ -1555,6 +1634,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   if (warp == 2) tmem_dealloc(tmem, kTmemCols);
+  if (s_plan.past > 0 && warp >= 4)   // warps 0-3 gave up the registers for it
+    items_past_grid<D, kPPRows>(p, s_plan, threadIdx.x - 128);
   pdl_wait();   // the next kernel's wait covers every earlier kernel
 }
 
@@ -1599,8 +1680,8 @@ cudaError_t launch_attention_tc(const AttnParams& p, const CUtensorMap& tm_k,
   if (p.D != 64 && p.D != 128) return cudaErrorInvalidValue;
   cudaError_t err;
   // row blocks: at most max_nodes * G rows of each of B sequences, and T * G
-  // rows of which every sequence may leave one block ragged; index order
-  // (B > kOrderMax) numbers the first form
+  // rows of which every sequence may leave one block ragged (sequences that overlap
+  // can make more: items_past_grid); index order (B > kOrderMax) numbers the first form
   const int rows = pingpong ? kPPRows : kRows;
   const long long full = static_cast<long long>((p.max_nodes * p.G + rows - 1) / rows) * p.B;
   const long long blocks =
