@@ -223,7 +223,8 @@ __device__ __forceinline__ int chunk_length(const AttnParams& p, PlanSmem& s) {
 // query rows (which read the same keys) innermost.  The hardware dispatches
 // CTAs in blockIdx order, so the longest run first and the short ones fill the
 // last wave.  False when the CTA has none.  Every thread of the CTA calls it (it synchronises the CTA).
-template <int ROWS>
+// CHOICE: the call may be the mma.sync kernel's (AttnParams::alone).
+template <int ROWS, bool CHOICE>
 __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSmem& s) {
   const int idx = blockIdx.x;
   int local, ctx, longest;   // longest: key tiles of the sequence's longest chunk
@@ -265,7 +266,7 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
       s.chunks[q] = 1;
       s.order[q] = make_int2(order_key(s.tiles[q], q), s.items[q]);
     }
-    const bool choice = p.alone && p.co_tiles >= 0;   // B <= 128: a sequence per thread
+    const bool choice = CHOICE && p.alone && p.co_tiles >= 0;   // B <= 128: a sequence per thread
     if (choice && threadIdx.x < kMaxNodes) {
       const int q = threadIdx.x;
       AloneTiles a{0, 0, 0};
@@ -799,7 +800,8 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
   return true;
 }
 
-// TWO: half of P in two bf16 terms (AttnParams::p_two).
+// TWO: half of P in two bf16 terms (AttnParams::p_two: a call of up to 128 nodes, which
+// alone may be the mma.sync kernel's).
 template <int D, bool TWO>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -829,7 +831,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   pdl_launch_dependents();
   // the mma.sync kernel's step (a call by itself: make_item)
-  if (p.co_tiles >= 0 && !p.alone && attention_takes_mma(p)) {
+  if (TWO && p.co_tiles >= 0 && !p.alone && attention_takes_mma(p)) {
     pdl_wait();
     return;
   }
@@ -875,7 +877,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
   }
   Item it;
-  const bool some = make_item<kRows>(p, it, s_plan);   // uniform over the CTA
+  const bool some = make_item<kRows, TWO>(p, it, s_plan);   // uniform over the CTA
   tc_fence_after();
   if (!some) {   // no query rows here
     if (warp == 10) tmem_dealloc(s_tmem, kTmemCols);
@@ -1311,7 +1313,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
   }
   Item it;
-  const bool some = make_item<kPPRows>(p, it, s_plan);   // uniform over the CTA
+  const bool some = make_item<kPPRows, false>(p, it, s_plan);   // uniform over the CTA
   tc_fence_after();
   if (!some) {   // no query rows here
     if (warp == 2) tmem_dealloc(s_tmem, kTmemCols);
