@@ -110,6 +110,14 @@ def tensor_peak():
         return 1900.0, "fallback"
 
 
+def check_replicas(args):
+    """Replicas on several GPUs run the headline workload as it is, whose 60 nodes
+    take the LM head's weight-streaming kernel: the wide kernel's clustered form
+    (from three tiles of 128 nodes on) multicasts and serves 1-GPU runs."""
+    if int(os.environ.get("WORLD_SIZE", "1")) > 1 and (args.config != CONFIG or args.batch):
+        raise SystemExit("several GPUs: only the headline workload (--config 2, no --batch) is run")
+
+
 def workload_config(wl):
     if CONFIG == 2:
         desc = ("llama3.1-8b-shaped verify step: batch 1, context 2048, 32 q / 8 kv heads, "
@@ -857,10 +865,7 @@ def main():
     if args.config != CONFIG or args.batch:
         args.no_cpu_baseline = True   # the oracle's full step is far too slow beyond the headline
         args.no_workloads = True
-    if int(os.environ.get("WORLD_SIZE", "1")) > 1 and args.config != CONFIG:
-        # replicas on several GPUs run the headline workload only: the wide LM
-        # head's clustered form (steps of more than 768 nodes) serves 1-GPU runs
-        raise SystemExit("several GPUs: only the headline workload (--config 2) is run")
+    check_replicas(args)
     CONFIG = args.config
     TAU = args.tau if args.tau is not None else synth.WORKLOADS[CONFIG]["tau"][0]
     if args.impl == "reference":

@@ -312,8 +312,9 @@ int32_t asd_abi_version(void);
  * kernel in clusters of two SMs that multicast W between them (three or four
  * 128-node tiles, or seven and more, and an even range count), 4 the fp32 kernel,
  * 0 for invalid arguments.  The clustered form multicasts from the calling
- * GPU's own memory only: when w_lm is not device memory of the current device
- * the call runs form 2.
+ * GPU's own memory only, and serves programs that use one GPU: when w_lm is not
+ * device memory of the current device, or the process sees several GPUs, the call
+ * runs form 2.
  */
 int32_t asd_lm_head_variant(const asd_dims* dims, int32_t total_nodes, const void* w_lm);
 

@@ -366,9 +366,15 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
   return mma && !in_step ? run_mma() : ASD_OK;
 }
 
-// True when `w` is device memory of the current device (the only memory the
-// clustered LM head may multicast from).
-bool on_this_device(const void* w) {
+// True when the clustered LM head may multicast from `w`: device memory of the
+// current device, in a process that sees no other GPU (a run on several GPUs takes
+// the unclustered form).
+bool may_multicast(const void* w) {
+  static const bool one_gpu = [] {
+    int n = 0;
+    return cudaGetDeviceCount(&n) == cudaSuccess && n == 1;
+  }();
+  if (!one_gpu) return false;
   int dev = 0;
   cudaPointerAttributes a{};
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
@@ -382,7 +388,7 @@ bool on_this_device(const void* w) {
 asd_status run_lmhead(const Ctx& c, const void* hidden, const void* w, float* l_draft) {
   const asd_dims& d = c.d;
   LmParams p{};
-  p.w_local = on_this_device(w) ? 1 : 0;
+  p.w_local = may_multicast(w) ? 1 : 0;
   p.hidden = hidden;
   p.w = w;
   p.child_start = ws_at<int32_t>(c.ws, c.L.child_start);
@@ -437,7 +443,7 @@ asd_status run_lmhead_lazy(const Ctx& c, const void* hidden, const void* w,
 
   LmParams p{};
   p.w = w;
-  p.w_local = on_this_device(w) ? 1 : 0;
+  p.w_local = may_multicast(w) ? 1 : 0;
   p.child_start = ws_at<int32_t>(c.ws, c.L.child_start);
   p.child_cnt = ws_at<int32_t>(c.ws, c.L.child_cnt);
   p.child_tok = ws_at<int32_t>(c.ws, c.L.child_tok);
@@ -554,7 +560,7 @@ int32_t asd_lm_head_variant(const asd_dims* dims, int32_t total_nodes, const voi
   LmParams p{};
   p.T = total_nodes;
   p.g_lm = lm_ranges(dims->vocab, nsm);
-  p.w_local = on_this_device(w_lm) ? 1 : 0;
+  p.w_local = may_multicast(w_lm) ? 1 : 0;
   p.t_dev = nullptr;
   if (dims->lm_head_schedule == ASD_LM_LAZY_LEVELS) return 2;   // a pass per launch
   return lmhead_bf16_variant(p);

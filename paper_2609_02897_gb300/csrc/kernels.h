@@ -214,8 +214,9 @@ struct LmParams {
   // belongs to node row_node[r].  Both null: T rows, row r = node r.
   const int* t_dev;
   const int32_t* row_node;
-  // 1: W is memory of the launching device, so the wide kernel may run in
-  // clusters of two that multicast W between their SMs (set by the host)
+  // 1: W is memory of the launching device, the only one this process sees, so the
+  // wide kernel may run in clusters of two that multicast W between their SMs (set
+  // by the host)
   int w_local;
 };
 constexpr int kLmStages = 3;       // 3 x 48 KB (a_rows <= 64): room for an attention CTA

@@ -990,7 +990,7 @@ int lmhead_bf16_variant(const LmParams& p) {
   // (each W stage is read once per cluster) and move their CTAs in lock step
   // through the rounds of node tiles.  The ranges must pair up, and the W
   // multicast reads this GPU's own memory only: a weight elsewhere (host or
-  // another device) runs unclustered.
+  // another device) and a process that sees several GPUs run unclustered.
   const int tiles = (p.T + kM - 1) / kM;
   if (p.g_lm % 2 != 0 || p.t_dev || !p.w_local) return 2;
   // W of 128256 x 4096, a cluster's round against unclustered ones: four tiles
