@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(192, 1)
 // the epilogue has drained it.
 //
 // CL = 2: the CTAs come in clusters of two that own two adjacent vocabulary
-// ranges together and share out the node tiles, four in a round (wide_slot).
+// ranges together and share out the node tiles, four in a round (WideRounds::slot).
 // Each CTA copies one of the two 128-row halves of every W stage and multicasts
 // it to both, so every SM pulls 48 KB per stage instead of 64 and W crosses HBM
 // once per four node tiles.  A stage is refilled only after both CTAs' MMAs have
@@ -467,11 +467,11 @@ struct WideRounds {
 // phase of its barriers.  A round with slot 0 alone alternates between the two,
 // so that one tile's drain overlaps the next tile's MMAs; its threads then wait
 // for phases of the other slot's barriers, which is sound while the two issuers
-// are within one tile of each other (a tile of at least kWideStages + 1 stages).
+// are within one tile of each other: a tile of more stages than the ring has.
 struct WideAcc {
   int cnt0 = 0, cnt1 = 0, flip = 0;   // uses so far of either accumulator
   bool may_flip;
-  __device__ __forceinline__ explicit WideAcc(int nkb) : may_flip(nkb > 3) {}
+  __device__ __forceinline__ explicit WideAcc(int nkb) : may_flip(nkb > kWideStages) {}
   // accumulator of slot j, `use`: how often it was used before
   __device__ __forceinline__ int of(int j, bool two, int& use) const {
     const int acc = j == 1 ? 1 : (two ? 0 : flip);

@@ -1,8 +1,9 @@
 """The wide LM head's sharing of node tiles between the CTAs of a cluster, where
 it can go wrong: every remainder of four tiles after none, one and two full
 rounds, odd and even numbers of 128-row vocabulary tiles per range (a 256-row
-tile then straddles two ranges), and hidden widths of one to four 64-element
-k-blocks (fewer stages than the ring, where the accumulators do not alternate).
+tile then straddles two ranges), and hidden widths of one, three and four
+64-element k-blocks (up to as many as the ring of three has stages the
+accumulators do not alternate, from four on they do).
 Bit-compared with the same rows computed by other tile counts: a row's
 statistics do not depend on the tile that holds it."""
 import pytest
