@@ -32,7 +32,8 @@ struct Geom {
   static constexpr int kTv = kThreads / kTn;         // and along the vocabulary
   static constexpr int kVp = kVt / kTv;              // a thread's vocabulary rows
   static constexpr int kNp = NT / kTn;               // and nodes
-  static constexpr int kStages = NT <= 16 ? 4 : 3;   // two CTAs per SM
+  static constexpr int kStages = NT <= 16 ? 4 : 3;
+  static constexpr int kCtas = NT <= 32 ? 2 : 1;     // per SM: 82 to 91 KB each, 119 for 64 nodes
   static constexpr int kStageFloats = (kVt + NT) * kLd;
   static constexpr size_t kBytes = sizeof(float) * kStages * kStageFloats;
 };
@@ -50,7 +51,7 @@ __device__ __forceinline__ void copy_async(float* dst, const float* src, bool in
 }
 
 template <int NT>
-__global__ void __launch_bounds__(kThreads, 2) lmhead_f32_kernel(const LmParams p) {
+__global__ void __launch_bounds__(kThreads, Geom<NT>::kCtas) lmhead_f32_kernel(const LmParams p) {
   using G = Geom<NT>;
   extern __shared__ __align__(16) float smem[];
   __shared__ float s_x[NT][kVt + 1];                 // logits of a chunk
