@@ -158,10 +158,16 @@ def _ptr(t: Optional[torch.Tensor]):
     return t.data_ptr()
 
 
+# The handle of torch.cuda.current_stream() without making a Stream object, where
+# this torch has the function (its name is not public).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
-        # the raw handle of torch.cuda.current_stream(), without the Stream object
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -271,8 +277,9 @@ ATTENTION_VARIANTS = {1: "attn_bf16_kernel", 2: "attn_tc_kernel", 3: "attn_pp_ke
 
 
 def asd_attention_variant(dims: Dims, total_nodes: int) -> int:
-    """Which tree-attention kernel a call runs (include/asd.h): 1-4, 0 for
-    invalid arguments."""
+    """Which tree-attention kernel a verify step runs (include/asd.h): 1-4, 0 for
+    invalid arguments.  Where it is 1, a step of long contexts and an attention
+    call by itself may run 2 instead."""
     return int(_lib.asd_attention_variant(ctypes.byref(dims), int(total_nodes)))
 
 
