@@ -29,11 +29,11 @@ def _alone(d, B, n, page, pages, cap, Hq, Hkv, D):
     return _call(d, dims, asd.alloc_workspace(dims, B * n))
 
 
-def _beside_lm_head(d, B, n, page, pages, cap, Hq, Hkv, D):
-    """attn_out of a step whose LM head (1 GB of weight) hides the attention."""
+def _beside_lm_head(d, B, n, page, pages, cap, Hq, Hkv, D, hidden=4096, vocab=128000):
+    """attn_out of a step; its LM head (by default 1 GB of weight) hides attention
+    of up to 0.8 key tiles a microsecond (contiguous, D = 128)."""
     import torch
     from paper_2609_02897_gb300 import asd
-    hidden, vocab = 4096, 128000
     dims = asd.make_dims(B, Hq, Hkv, D, hidden, vocab, asd.ASD_BF16, page, cap, pages, n, n)
     bf16 = dict(dtype=torch.bfloat16, device="cuda")
     step = asd.VerifyStep(dims, B * n).bind(
@@ -97,3 +97,31 @@ def test_a_large_cache_leaves_it_to_the_contexts(B, n, page, Hq, D):
     out = _alone(d, B, n, page, pages, cap, Hq, Hkv, D)
     exact = _exact(d, B, n, ctx, page, Hq, Hkv, D)
     assert float((out.double() - exact).norm() / exact.norm()) < BOUND   # 2.2e-3: mma.sync
+
+
+# (B, nodes, hidden, vocab, contexts at the limit, and one key beyond).  A tiny LM
+# head: 16 key tiles on the busiest SM, which are the longest split's (84 context
+# tiles in 6 splits, 2 of the tree).  One of 480 MB: 60 tiles, those of one
+# unsplit sequence among 40 (the others share out 1 tile per SM each).
+STEPS = [
+    (2, 40, 64, 200, [2688, 2688], [2688, 2689]),
+    (40, 3, 4096, 58600, [1] * 39 + [32 * 59], [1] * 39 + [32 * 59 + 1]),
+    (2, 40, 64, 200, [0, 5], [4000, 40]),
+]
+
+
+@pytest.mark.parametrize("case", range(len(STEPS)))
+def test_a_step_runs_the_kernel_its_contexts_call_for(case):
+    """Up to the limit the mma.sync kernel beside the LM head, with the bits of a
+    step whose LM head hides any context of the cache; beyond it the tensor-core
+    kernel, with those of an attention call by itself."""
+    B, n, hidden, vocab, at, beyond = STEPS[case]
+    Hq, Hkv, D, cap = 16, 4, 128, 4096 if B == 2 else 2048
+    for ctx, mma in ((at, True), (beyond, False)):
+        d = _inputs(B, n, ctx, 0, Hq, Hkv, D, cap, case)
+        alone = _alone(d, B, n, 0, 0, cap, Hq, Hkv, D)
+        out = _beside_lm_head(d, B, n, 0, 0, cap, Hq, Hkv, D, hidden, vocab).clone()
+        # the step has committed past the contexts, which no attention reads
+        hidden_by_lm = _beside_lm_head(d, B, n, 0, 0, cap, Hq, Hkv, D)
+        assert not _same(alone, hidden_by_lm)
+        assert _same(out, hidden_by_lm if mma else alone)

@@ -24,12 +24,18 @@ def test_rows_do_not_depend_on_their_tile(hidden, vocab):
     tokens = torch.randint(0, vocab, (most,), generator=g, device="cuda").int()
     parent = (torch.arange(most, dtype=torch.int32) % n - 1).cuda()     # chains of 8
 
+    ranges = min(torch.cuda.get_device_properties(0).multi_processor_count, 256, (vocab + 31) // 32)
+    clustered = torch.cuda.device_count() == 1 and ranges % 2 == 0
+
     def call(T):
         dims = asd.make_dims(T // n, 4, 4, 64, hidden, vocab, asd.ASD_BF16, 0, 64, 0, n, n)
         out = {k: torch.zeros(T, dtype=torch.float32, device="cuda")
                for k in ("row_max", "row_lse", "l_draft", "ratio")}
         out["row_argmax"] = torch.zeros(T, dtype=torch.int32, device="cuda")
         out["accept"] = torch.zeros(T, dtype=torch.uint8, device="cuda")
+        tiles = -(-T // 128)
+        assert asd.asd_lm_head_variant(dims, T, w) == \
+            (3 if clustered and (tiles in (3, 4) or tiles >= 7) else 2), tiles
         ws = asd.alloc_workspace(dims, T)
         cu = torch.arange(0, T + 1, n, dtype=torch.int32, device="cuda")
         asd.asd_lmhead_margin(dims, h[:T], w, tokens[:T], parent[:T], cu, 0.5, workspace=ws, **out)

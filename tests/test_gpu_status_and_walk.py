@@ -86,6 +86,50 @@ def test_walk_and_commit(B, rule):
     assert int(cout[B - 1]) == int(ctx[B - 1])
 
 
+@pytest.mark.parametrize("B", [8, 9, 16, 17])
+def test_walk_and_commit_in_a_captured_graph(B):
+    """The cluster launches, the non-portable sizes among them, and the kernel that
+    clears the status word beyond 16 sequences, recorded and replayed on other
+    inputs in the same buffers."""
+    import torch
+    from paper_2609_02897_gb300 import asd
+    first = _batch(B, 100 + B)
+    parent, _, _, _, _, cu = first
+    rng = np.random.default_rng(B)
+    T, Hkv, D, cap, max_path = int(cu[-1]), 2, 64, 64, 16
+    # the same trees, other verdicts
+    second = (parent, rng.integers(0, 50, T).astype(np.int32), (rng.random(T) < 0.6).astype(np.uint8),
+              rng.integers(0, 50, T).astype(np.int32), first[4], cu)
+    dims = asd.make_dims(B, 2, Hkv, D, 64, 50, asd.ASD_BF16, 0, cap, 0, 128, max_path)
+    ws = asd.alloc_workspace(dims, T)
+    dev = [torch.from_numpy(x.copy()).cuda() for x in first]
+    i32 = lambda *s: torch.zeros(s, dtype=torch.int32, device="cuda")  # noqa: E731
+    path, plen, bonus, npro, cout, ctx = i32(B, max_path), i32(B), i32(B), i32(B), i32(B), i32(B)
+    tk, tv = (torch.randn(T, Hkv, D, device="cuda").to(torch.bfloat16) for _ in range(2))
+    kc, vc = (torch.zeros(B, Hkv, cap, D, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+
+    def calls():
+        asd.asd_accept_path(dims, dev[0], dev[1], dev[2], dev[3], dev[5], path, plen, bonus, npro, ws,
+                            ratio=dev[4])
+        asd.asd_kv_compact(dims, tk, tv, dev[5], T, path, plen, ctx, None, kc, vc, cout, ws)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        calls()
+    for batch in (first, second):
+        for t, x in zip(dev, batch):
+            t.copy_(torch.from_numpy(x.copy()))
+        kc.zero_()
+        graph.replay()
+        assert asd.asd_get_device_status(ws) == 0
+        want, wlen, wbonus, _ = oracle.accept_path(parent, batch[2], batch[3], batch[1], cu, rule=0,
+                                                   ratio=batch[4])
+        assert plen.tolist() == list(wlen) and bonus.tolist() == list(wbonus) and cout.tolist() == list(wlen)
+        for b in range(B):
+            rows = torch.tensor([int(cu[b]) + u for u in want[b]], device="cuda")
+            assert torch.equal(kc[b, :, :len(rows)], tk[rows].transpose(0, 1))
+
+
 @pytest.mark.parametrize("B", [1, 8, 9, 32, 33, 40])
 def test_tree_preparation_reports_any_sequence(B):
     import torch

@@ -22,7 +22,7 @@ def dev():
 def test_cluster_form_only_for_a_weight_on_this_gpu(dev):
     import torch
     from paper_2609_02897_gb300 import asd
-    wl = synth.make_workload(5, small=True, overrides=dict(B=8))   # 1024 nodes: 4 tile pairs
+    wl = synth.make_workload(5, small=True, overrides=dict(B=8))   # 1024 nodes: 8 tiles of 128
     dims = dev.dims_of(wl)
     nsm = torch.cuda.get_device_properties(0).multi_processor_count
     ranges = max(1, min(nsm, 256, (wl.vocab + 31) // 32))
@@ -32,12 +32,18 @@ def test_cluster_form_only_for_a_weight_on_this_gpu(dev):
     assert asd.asd_lm_head_variant(dims, wl.T, w_dev) == (3 if ranges % 2 == 0 else 2)
     assert asd.asd_lm_head_variant(dims, wl.T, w_pinned) == 2
     assert asd.asd_lm_head_variant(dims, wl.T, w_pageable) == 2
-    # two tile pairs: clustered (with pairing ranges); three: unclustered (one
-    # CTA of a cluster would idle through the second round)
+    # clustered (with pairing ranges): three and four tiles of 128 nodes, and seven
+    # and more; two, five and six leave a CTA of the cluster too little to do
     assert asd.asd_lm_head_variant(dims, 512, w_dev) == (3 if ranges % 2 == 0 else 2)
     assert asd.asd_lm_head_variant(dims, 768, w_dev) == 2
     assert asd.asd_lm_head_variant(dims, 256, w_dev) == 2
-    # the lazy schedule's levels run the wide kernel unclustered
+    dims.batch = 10                               # up to ten tiles
+    for tiles in range(2, 11):
+        for nodes in (128 * tiles - 127, 128 * tiles):
+            assert asd.asd_lm_head_variant(dims, nodes, w_dev) == \
+                (3 if ranges % 2 == 0 and (tiles in (3, 4) or tiles >= 7) else 2), nodes
+    dims.batch = wl.B
+    # the lazy schedule's passes run the wide kernel unclustered
     dims.lm_head_schedule = asd.ASD_LM_LAZY_LEVELS
     assert asd.asd_lm_head_variant(dims, wl.T, w_dev) == 2
 
@@ -64,7 +70,8 @@ def test_attention_variant(dev):
     wl = synth.make_workload(5, small=True)        # 6 x 128 nodes, 2 KV heads, G = 4
     dims = dev.dims_of(wl)
     assert asd.asd_attention_variant(dims, wl.T) == 2
-    # the two-tile form once its 256-row items fill two waves of CTAs
+    # the two-tile form: its 256-row items make more than 1.5 waves of CTAs (the
+    # other lines of that rule: test_gpu_pingpong_rows.py)
     dims.batch = 4 * nsm
     items = dims.num_kv_heads * ((dims.batch * 128 * 4 + 255) // 256)
     assert items >= 2 * nsm
