@@ -759,9 +759,10 @@ asd_status asd_verify_step(const asd_dims* dims, const asd_verify_args* a, void*
   // The LM head goes first and takes one CTA per SM; the attention kernel
   // starts right behind it (it reads no output of the LM head).  Up to 128
   // nodes its CTAs share the SMs with the LM head's while the weights stream
-  // in, unless the contexts are longer than that hides; beyond that the wide LM head fills the SMs' shared memory and the
-  // tensor-core attention runs after it.  The lazy schedule also finalises
-  // the rows it computes, so the tail only walks.
+  // in, unless the contexts are longer than that hides; beyond that the wide LM
+  // head fills the SMs' shared memory and the tensor-core attention runs after
+  // it.  The lazy schedule also finalises the rows it computes, so the tail only
+  // walks.
   const bool lazy = c.d.lm_head_schedule == ASD_LM_LAZY_LEVELS;
   st = lazy ? run_lmhead_lazy(c, a->hidden, a->w_lm, a->parent, a->tokens, a->cu_nodes, a->tau,
                               a->row_max, a->row_argmax, a->row_lse, a->l_draft, a->ratio,

@@ -1,21 +1,21 @@
 // Tree attention of the verify pass (Sec. 2 "Verify": the target scores every
 // drafted node of the tree in one forward pass): the bf16 kernel that shares
-// the SMs with the LM head (verify steps of up to 128 nodes; larger steps and
-// standalone calls go to the tensor-core kernels in attention_tc.cu) and the
-// exact fp32 kernel.
+// the SMs with the LM head (verify steps of up to 128 nodes) and takes calls by
+// themselves of many short sequences (the rest goes to the tensor-core kernels in
+// attention_tc.cu), and the exact fp32 kernel.
 //
 // Work unit: one CTA per (row block, sequence x KV head, context split).  The
 // query rows of a (sequence, KV head) pair are its N nodes times the G query
 // heads that share the KV head (grouped-query attention), packed node-major:
 // row r -> node r / G, head g*G + r % G.  Split z covers context keys
-// [z*L, (z+1)*L), L from the sequence's own length (flash-decoding split-KV); the CTA of the sequence's last
-// non-empty split also covers the tree keys, where a node only sees its
-// ancestors (bitmasks derived in-kernel from the parent array).  The splits of one
-// (row block, sequence x KV head) form a thread-block cluster: each CTA keeps
-// its softmax-normalised partial output and log-sum-exp in shared memory, and
-// after a cluster barrier every CTA merges a slice of the rows by reading its
-// peers' partials through distributed shared memory.  No partial leaves the
-// cluster.
+// [z*L, (z+1)*L), L from the sequence's own length (flash-decoding split-KV); the
+// CTA of the sequence's last non-empty split also covers the tree keys, where a
+// node only sees its ancestors (bitmasks derived in-kernel from the parent array).
+// The splits of one (row block, sequence x KV head) form a thread-block cluster:
+// each CTA keeps its softmax-normalised partial output and log-sum-exp in shared
+// memory, and after a cluster barrier every CTA merges a slice of the rows by
+// reading its peers' partials through distributed shared memory.  No partial
+// leaves the cluster.
 #include <algorithm>
 #include <type_traits>
 
@@ -120,17 +120,6 @@ struct KeyRange {
   }
 };
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
-               ::: "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-
 // Address of the same shared-memory location in cluster CTA `rank`.
 __device__ __forceinline__ uint32_t peer_addr(uint32_t local, uint32_t rank) {
   uint32_t r;
@@ -167,9 +156,9 @@ __device__ __forceinline__ void cluster_merge(const AttnParams& p, const RowMap&
   constexpr int kC4 = D / 4;
   __shared__ float s_w[kRowsPerCta][kMaxAttnParts];
   __shared__ float s_inv[kRowsPerCta];
-  cluster_sync();
+  cluster_barrier();
   const int P = p.n_parts;
-  const uint32_t rank = cluster_rank();
+  const uint32_t rank = cta_rank_in_cluster();
   const int per = (nrows + P - 1) / P;
   const int rbeg = static_cast<int>(rank) * per;
   const int rend = min(nrows, rbeg + per);
@@ -216,7 +205,7 @@ __device__ __forceinline__ void cluster_merge(const AttnParams& p, const RowMap&
     out[2] = from_f32<OutT>(acc.z * inv);
     out[3] = from_f32<OutT>(acc.w * inv);
   }
-  cluster_sync();
+  cluster_barrier();
 }
 
 // ----------------------------------------------------------- bf16 tensor path
@@ -571,13 +560,6 @@ struct F32Geom {
   static_assert(4 * kTile >= kRowsPerCta * D, "the K/V ring holds the output rows at the end");
 };
 
-// 16 bytes of global memory -> shared memory, zeros unless `in`.
-__device__ __forceinline__ void copy16_async(float* dst, const float* src, bool in) {
-  const int n = in ? 16 : 0;
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n)
-               : "memory");
-}
-
 template <int D>
 __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const AttnParams p) {
   using G = F32Geom<D>;
@@ -639,15 +621,15 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const AttnParams 
       }
       const bool in = row >= 0;
       const long long at = in ? row * D + 4 * ch : 0;
-      copy16_async(smem_f + G::kK + stage * G::kTile + j * kLd + 4 * ch, (tree ? tk : kc) + at, in);
-      copy16_async(smem_f + G::kV + stage * G::kTile + j * kLd + 4 * ch, (tree ? tv : vc) + at, in);
+      copy_async<16>(smem_f + G::kK + stage * G::kTile + j * kLd + 4 * ch, (tree ? tk : kc) + at, in);
+      copy_async<16>(smem_f + G::kV + stage * G::kTile + j * kLd + 4 * ch, (tree ? tv : vc) + at, in);
       if (ch == 0) s_seen[stage][j] = in ? (tree ? 2 + u - nctx_keys : 1) : 0;
     }
   };
 
   for (int i = tid; i < nrows * (D / 4); i += kF32Threads) {
     const int r = i / (D / 4), ch = i - r * (D / 4);
-    copy16_async(smem_f + G::kQ + r * kLd + 4 * ch, qp + rm.grow(r) * D + 4 * ch, true);
+    copy_async<16>(smem_f + G::kQ + r * kLd + 4 * ch, qp + rm.grow(r) * D + 4 * ch, true);
   }
   if (ntiles > 0) load(0);
   asm volatile("cp.async.commit_group;" ::: "memory");

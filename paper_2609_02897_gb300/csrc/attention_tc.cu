@@ -1,13 +1,16 @@
 // Tree attention (Sec. 2 "Verify": the target scores every drafted node in
 // one forward pass) on the 5th-generation tensor cores, where the attention
-// kernel has the SMs to itself: a standalone attention call, or a step of more
-// than 128 tree nodes (the LM head then takes most of an SM's shared memory
-// and runs first).  bf16 in, fp32 accumulate.
+// kernel has the SMs to itself: a step of more than 128 tree nodes (the LM head
+// then takes most of an SM's shared memory and runs first); a smaller one whose
+// contexts are longer than its LM head hides, behind the LM head (decided on the
+// device, AttnParams::co_tiles); and an attention call by itself, unless many
+// short sequences are better off with the mma.sync kernel.  bf16 in, fp32
+// accumulate.
 //
 // Measured, a whole asd_tree_attention call: one sequence, 8 nodes, context
-// 32768 in a cache of 40960 slots 186.5 -> 36.9 us (134 MB of K/V; the
+// 32768 in a cache of 40960 slots 186.5 -> 32.3 us (134 MB of K/V; the
 // mma.sync kernel in 8 splits of the cache's capacity before), 4 sequences of
-// 60 nodes, contexts 901 to 3625 41.0 -> 32.4 us (unsplit before).
+// 60 nodes, contexts 901 to 3625 41.0 -> 24.8 us (unsplit before).
 //
 // Work item (one CTA): 128 query rows of one (sequence, KV head) pair and a
 // chunk of its keys: the whole context, or, when the items would leave SMs
@@ -16,12 +19,11 @@
 // (chunk_length: the host knows the cache's capacity only, which says little
 // about them), so a cache sized for many times the context splits like a tight
 // one.  A chunk leaves its unnormalised O, reference max and row sum in the
-// workspace, and attn_merge_kernel, a warp per query row, combines them.  The
-// CTAs take the chunks in decreasing order of work, so the longest start
-// first.  The rows of a pair are its N nodes times the G query heads that
+// workspace, and attn_merge_kernel, one warp or four per query row, combines
+// them.  The CTAs take the chunks in decreasing order of work, so the longest
+// start first.  The rows of a pair are its N nodes times the G query heads that
 // share the KV head, node-major (row r -> node r / G, head g*G + r % G); row r
-// lives in TMEM lane r.  Keys come in tiles of 128,
-// K and V through TMA rings of their own (128-byte swizzle; paged caches one
+// lives in TMEM lane r.  Keys come in tiles of 128, K and V through TMA rings of their own (128-byte swizzle; paged caches one
 // box per page; the tree K/V through a 3D map over [T, Hkv, D]), so a K slot
 // is refilled as soon as its S MMA is done rather than after the tile's P.V;
 // the last tile of a pair holds its tree keys, where a node sees only its
@@ -37,10 +39,11 @@
 //
 // The softmax keeps a per-row reference max m and rescales O only when the
 // running max exceeds m by more than 2^8 in the exp2 domain (P then stays
-// below 2^8 and the result equals that with the exact running max).  S/P is triple-buffered: S of tile
-// t+1 is ready when the softmax finishes tile t, and S of tile t+2 does not
-// wait for O += P V of tile t (with two buffers it did, which put the P.V,
-// its commit and the next S on the softmax's path every second tile).
+// below 2^8 and the result equals that with the exact running max, but for the
+// rounding of P: exp2_tile_two).  S/P is triple-buffered: S of tile t+1 is ready
+// when the softmax finishes tile t, and S of tile t+2 does not wait for O += P V of
+// tile t (with two buffers it did, which put the P.V, its commit and the next S on
+// the softmax's path every second tile).
 //
 // TMEM (512 columns): O [0, D), S/P [128, 256), [256, 384), [384, 512).
 // Shared memory: Q, a 3-stage K ring and a V ring (160 KB of rings for D =
@@ -222,7 +225,8 @@ __device__ __forceinline__ int chunk_length(const AttnParams& p, PlanSmem& s) {
 // length (ties by index), within one its KV heads, its chunks, its blocks of
 // query rows (which read the same keys) innermost.  The hardware dispatches
 // CTAs in blockIdx order, so the longest run first and the short ones fill the
-// last wave.  False when the CTA has none.  Every thread of the CTA calls it (it synchronises the CTA).
+// last wave.  False when the CTA has none.  Every thread of the CTA calls it (it
+// synchronises the CTA).
 // CHOICE: the call may be the mma.sync kernel's (AttnParams::alone).
 template <int ROWS, bool CHOICE>
 __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSmem& s) {
@@ -385,16 +389,18 @@ __device__ __forceinline__ void items_past_grid(const AttnParams& p, PlanSmem& s
     for (int r = r0 + (tid >> 5); r < min(r0 + ROWS, R); r += kSoftmaxThreads / 32) {
       const int node = r / p.G;
       const size_t row = static_cast<size_t>(s0 + node) * p.Hq + g * p.G + (r - node * p.G);
+      const __nv_bfloat16* qr = static_cast<const __nv_bfloat16*>(p.q) + row * D;
+      __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.out) + row * D;
       float q[kV], o[kV], m = -INFINITY, l = 0.f;
 #pragma unroll
       for (int k = 0; k < kV; ++k) {
-        q[k] = to_f32(static_cast<const __nv_bfloat16*>(p.q)[row * D + lane * kV + k]) * p.scale_log2;
+        q[k] = __bfloat162float(qr[lane * kV + k]) * p.scale_log2;
         o[k] = 0.f;
       }
       auto key = [&](const __nv_bfloat16* kr, const __nv_bfloat16* vr) {
         float x = 0.f;
 #pragma unroll
-        for (int k = 0; k < kV; ++k) x = fmaf(q[k], to_f32(kr[lane * kV + k]), x);
+        for (int k = 0; k < kV; ++k) x = fmaf(q[k], __bfloat162float(kr[lane * kV + k]), x);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
         const float mn = fmaxf(m, x);
@@ -402,7 +408,7 @@ __device__ __forceinline__ void items_past_grid(const AttnParams& p, PlanSmem& s
         const float pe = x == -INFINITY ? 0.f : exp2f(x - mn);
         l = l * al + pe;
 #pragma unroll
-        for (int k = 0; k < kV; ++k) o[k] = fmaf(pe, to_f32(vr[lane * kV + k]), o[k] * al);
+        for (int k = 0; k < kV; ++k) o[k] = fmaf(pe, __bfloat162float(vr[lane * kV + k]), o[k] * al);
         m = mn;
       };
       for (int j = 0; j < s.ctx[b]; ++j) {
@@ -427,7 +433,7 @@ __device__ __forceinline__ void items_past_grid(const AttnParams& p, PlanSmem& s
       const float inv = l > 0.f ? 1.f / l : 0.f;
 #pragma unroll
       for (int k = 0; k < kV; ++k)
-        static_cast<__nv_bfloat16*>(p.out)[row * D + lane * kV + k] = from_f32<__nv_bfloat16>(o[k] * inv);
+        out[lane * kV + k] = __float2bfloat16_rn(o[k] * inv);
     }
   }
 }

@@ -168,10 +168,10 @@ struct AloneRule {
 AloneRule attention_alone_rule(const asd_dims& d, int total_nodes, int nsm);
 int attention_keys_per_tile();   // context keys per K/V tile = TMA box rows
 // bf16 path on the 5th-generation tensor cores, where attention has the SMs to
-// itself (a standalone call, or a step of more than 128 tree nodes): one CTA
-// per (128 query rows, sequence x KV head, chunk of the keys), and a merge
-// kernel behind it where chunks are possible (p.part_cap > 0).  tm_k /
-// tm_v: 2D maps over the cache rows with boxes of 64 columns x
+// itself (a step of more than 128 tree nodes, or of fewer with long contexts, or a
+// call by itself): one CTA per (128 query rows, sequence x KV head, chunk of the
+// keys), and a merge kernel behind it where chunks are possible (p.part_cap > 0).
+// tm_k / tm_v: 2D maps over the cache rows with boxes of 64 columns x
 // min(kAttnTcKeys, rows per page) rows; tm_tk / tm_tv: 3D maps over the tree
 // K/V [T, Hkv, D] with boxes of 64 columns x 1 head x kAttnTcKeys nodes;
 // tm_q (with p.q_tma, where attention_q_tma_ok(G)): a 3D map over

@@ -38,18 +38,6 @@ struct Geom {
   static constexpr size_t kBytes = sizeof(float) * kStages * kStageFloats;
 };
 
-// `bytes` (4 or 16) of global memory -> shared memory, zeros unless `in`.
-template <int bytes>
-__device__ __forceinline__ void copy_async(float* dst, const float* src, bool in) {
-  const int n = in ? bytes : 0;
-  if (bytes == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n)
-                 : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n)
-                 : "memory");
-}
-
 template <int NT>
 __global__ void __launch_bounds__(kThreads, Geom<NT>::kCtas) lmhead_f32_kernel(const LmParams p) {
   using G = Geom<NT>;

@@ -356,17 +356,6 @@ constexpr uint32_t kWideTmemCols = kWideG * kWideN;  // 512
 constexpr int kTileGroups = kLmTileN / kLmBoxRows;   // range groups per packed tile
 constexpr int kWideThreads = 352;                    // producer, 2 MMA issuers, 2 epilogue groups
 
-__device__ __forceinline__ uint32_t cta_rank_in_cluster() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
-               ::: "memory");
-}
-
 // The shared::cluster address of this CTA's shared variable at `local` in the
 // CTA of cluster rank `rank`.
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t local, int rank) {

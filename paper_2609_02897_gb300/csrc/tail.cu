@@ -1,5 +1,6 @@
 // Per-sequence tail of the verify step, one CTA of 1024 threads per sequence
-// (thread i < N owns local node i; all 32 warps share the merge and the copy).  Three stages, selected by TailParams::mode:
+// (thread i < N owns local node i; all 32 warps share the merge and the copy).
+// Three stages, selected by TailParams::mode:
 //  finalize  merge the LM head's per-range partials of every row into
 //            row_max / row_argmax / row_lse and evaluate the margin rule for
 //            every drafted node: ratio = exp(l_draft - row_max[parent]) (Eq. 1),
@@ -51,8 +52,7 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const TailParams p) 
   if (p.clear_status) {
     pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) p.status[0] = p.status[1] = 0;
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
-                 ::: "memory");
+    cluster_barrier();
   }
   pdl_launch_dependents();
   const int b = blockIdx.x;
@@ -327,8 +327,8 @@ cudaError_t launch_tail(const TailParams& p, cudaStream_t s) {
 cudaError_t launch_tail_alone(TailParams p, cudaStream_t s) {
   // Up to 16 sequences as one cluster that clears the status word itself: the
   // host's launch of a kernel for it is what such a call costs most (walk and
-  // commit of 16 sequences, two calls 15.7 -> 13.6 us).  More, or a device that does not
-  // take the cluster, keep the kernel.
+  // commit of 16 sequences, two calls 15.7 -> 13.6 us).  More, or a device that
+  // does not take the cluster, keep the kernel.
   if (p.B <= kMaxTailCluster) {
     cudaError_t err = cudaSuccess;
     if (p.B > 8)

@@ -9,9 +9,9 @@
 // by side in a CTA.  Batches of up to kOneCta sequences take one CTA, which can
 // then clear the status word itself, and the call's kernels follow one another
 // by programmatic launches from the previous call's on: a memset in front of
-// the call cost it about 4 us (headline step 175.5 -> 171.4 us, attention of
-// one sequence at context 32768 36.9 -> 33.0 us).  Nothing waits for the later rounds of such a batch but the LM
-// head's first epilogue, some 10 us into the call.
+// the call cost it about 4 us (headline step 175.5 -> 171.4 us).  Nothing waits
+// for the later rounds of such a batch but the LM head's first epilogue, some 10
+// us into the call.
 #include <algorithm>
 
 #include "kernels.h"
