@@ -324,9 +324,10 @@ int32_t asd_lm_head_variant(const asd_dims* dims, int32_t total_nodes, const voi
  * bf16 split-KV kernel beside the LM head (up to 128 nodes), 2 the tensor-core
  * kernel with one 128-row query tile per CTA, 3 the tensor-core kernel with two
  * query tiles per CTA in ping-pong (when the sequences have more than 128 query
- * rows on average and the 256-row items fill 5/6 to 1 or more than 1.5 waves of
- * CTAs, or 1 to 1.5 with pages of at most 32 tokens), 4 the fp32 kernel, 0 for
- * invalid arguments.
+ * rows on average, few of their second tiles stay empty, and the 256-row items fill
+ * more than 1.5 waves of CTAs, or more than one with pages of at most 32 tokens, or
+ * 5/6 to one, where the device decides from ctx_len and runs form 2 if the longest
+ * context stands out), 4 the fp32 kernel, 0 for invalid arguments.
  * Where the answer is 1, a step whose contexts turn out longer than the LM head
  * hides runs form 2 behind it instead (the device decides from ctx_len), and
  * asd_tree_attention by itself, without an LM head to share the SMs with, runs

@@ -148,8 +148,12 @@ WsLayout layout(const asd_dims& d, int T, int nsm) {
   // more than one 128-node tile: the LM head (wide kernel) leaves no room on
   // its SMs, attention runs after it on the tensor-core kernel, unsplit
   L.attn_tc = (d.dtype == ASD_BF16 && T > kAttnTcRows) ? 1 : 0;
-  if (L.attn_tc && attention_pingpong(d.batch, d.num_kv_heads, G, T, d.page_size, nsm))
-    L.attn_tc = 2;
+  if (L.attn_tc)
+    switch (attention_pair_rule(d.batch, d.num_kv_heads, G, T, d.page_size, nsm)) {
+      case PairRule::kOneTile: break;
+      case PairRule::kPairs: L.attn_tc = 2; break;
+      case PairRule::kByContext: L.attn_tc = 3; break;
+    }
   size_t off = 0;
   L.status = off;      off = align256(off + 16);
   L.seq_flags = off;   off = align256(off + 4 * static_cast<size_t>(d.batch));
@@ -345,7 +349,8 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
     if (!make_q_tmap_bf16(&tq, q, d.head_dim, d.num_q_heads, c.T, a.G)) return ASD_ERR_CUDA;
     a.q_tma = 1;
   }
-  const bool pingpong = c.L.attn_tc == 2;
+  const bool pingpong = c.L.attn_tc >= 2;
+  if (c.L.attn_tc == 3) a.pair_ratio = attention_pair_ratio(d.page_size);
   if (!pingpong) {
     // a standalone call has no use for the LM head's partials either
     const size_t at = in_step ? c.L.at_part : c.L.lm_part;
@@ -362,6 +367,11 @@ asd_status run_attention(const Ctx& c, const void* q, const void* k_cache, const
     }
   }
   if (launch_attention_tc(a, tk, tv, ttk, ttv, tq, pingpong, c.st) != cudaSuccess)
+    return ASD_ERR_CUDA;
+  // decided by the context lengths: the one-tile form, unsplit at these sizes; if
+  // it has no work its CTAs pass on the SMs that the pairs leave free
+  if (c.L.attn_tc == 3 &&
+      launch_attention_tc(a, tk, tv, ttk, ttv, tq, false, c.st) != cudaSuccess)
     return ASD_ERR_CUDA;
   return mma && !in_step ? run_mma() : ASD_OK;
 }
@@ -549,7 +559,7 @@ int32_t asd_attention_variant(const asd_dims* dims, int32_t total_nodes) {
   const int nsm = device_sm_count();
   if (nsm <= 0) return 0;
   const WsLayout L = layout(*dims, total_nodes, nsm);
-  return L.attn_tc == 2 ? 3 : (L.attn_tc == 1 ? 2 : 1);
+  return L.attn_tc >= 2 ? 3 : (L.attn_tc == 1 ? 2 : 1);
 }
 
 int32_t asd_lm_head_variant(const asd_dims* dims, int32_t total_nodes, const void* w_lm) {

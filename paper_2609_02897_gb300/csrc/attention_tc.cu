@@ -127,6 +127,41 @@ __device__ __forceinline__ bool aborted_warp(volatile int* s_abort) {
   return __shfl_sync(0xffffffffu, *s_abort, 0) != 0;
 }
 
+// Whether a call of about one wave of pairs of query tiles is the ping-pong form's
+// (p.pair_ratio > 0: both forms are launched and decide alike).  Its pairs take 1.8
+// us a key tile together at D = 128 (1.5 at D = 64), and the call the longest pair's
+// time.  Of the one-tile form's items, one to two waves in decreasing order, an SM's
+// second starts as its first ends: the call takes the longest item, or 1.15 times
+// an even share of all, at 1.0 us a key tile (1.2 with pages of 32 tokens or more,
+// 1.4 with smaller ones; D = 64 0.85 and 1.1), and 4 us more than the pairs for the
+// second start.  The idle form's grid costs the call some 3 us.  One tile / pairs by
+// themselves, 8 KV heads, G = 4:
+//   16 x 64 nodes, context 2048 47.7 / 41.1 us, pages of 16 60.7 / 42.3, of 32 53.7 /
+//     42.1, D = 64 41.9 / 33.3; contexts 300-1000 30.4 / 26.0
+//   16 x 64, contexts 1000-6000 59.1 / 78.0, pages of 16 100.2 / 94.6, of 32 81.2 /
+//     95.8, D = 64 53.1 / 78.3; 9 x 128 67.7 / 89.3, D = 64 76.3 / 74.7
+// Every lane of a warp calls it; the answer is uniform over the grid.
+constexpr int kPairSeqs = 192;   // sequences at most (one pair each and KV head, one wave)
+__device__ __forceinline__ bool attention_takes_pairs(const AttnParams& p) {
+  int longest = 0, pairs = 0, work = 0;
+#pragma unroll
+  for (int k = 0; k < kPairSeqs / 32; ++k) {   // unrolled: all loads in flight at once
+    const int q = (threadIdx.x & 31) + 32 * k;
+    if (q >= p.B) continue;
+    const int n = min(max(p.cu_nodes[q + 1] - p.cu_nodes[q], 0), kMaxNodes);
+    const int ctx = min(max(p.ctx_len[q], 0), p.ctx_max);
+    const int t = n > 0 ? (ctx + kKeys - 1) / kKeys + 1 : 0, r = n * p.G;
+    longest = max(longest, t);
+    pairs += (r + 2 * kRows - 1) / (2 * kRows) * p.Hkv;
+    work += (r + kRows - 1) / kRows * p.Hkv * min(t, 1 << 20);
+  }
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  pairs = __reduce_add_sync(0xffffffffu, pairs);
+  work = __reduce_add_sync(0xffffffffu, work);
+  const float one = fmaxf(static_cast<float>(longest), 1.15f * static_cast<float>(work) / p.nsm);
+  return pairs <= p.nsm && static_cast<float>(longest) <= p.pair_ratio * one + 3.f;
+}
+
 struct Item {
   int b, g, s0, n, r0, nrows, R;
   int key_base;              // first context key of the chunk (a multiple of kKeys)
@@ -136,6 +171,12 @@ struct Item {
 };
 
 constexpr int kOrderMax = 256;   // batches ordered by work in-kernel (larger ones: index order)
+
+// Forms of the kernels compiled apart, since code that a call skips still costs it
+// up to 1 %: calls of up to 128 nodes hand half of P over in two bf16 terms and may
+// be the mma.sync kernel's (AttnParams::p_two, co_tiles); calls of about one wave of
+// pairs go to either form by their context lengths (pair_ratio).
+enum Mode { kPlain, kTwoTerms, kByContext };
 
 constexpr int kMaxChunks = 32;   // chunks per sequence: one lane of the merging warp each
 constexpr int kMergeOverhead = 3;   // cost of the merge in key tiles of ~1 us
@@ -227,12 +268,11 @@ __device__ __forceinline__ int chunk_length(const AttnParams& p, PlanSmem& s) {
 // CTAs in blockIdx order, so the longest run first and the short ones fill the
 // last wave.  False when the CTA has none.  Every thread of the CTA calls it (it
 // synchronises the CTA).
-// CHOICE: the call may be the mma.sync kernel's (AttnParams::alone).
-template <int ROWS, bool CHOICE>
+template <int ROWS, int MODE>
 __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSmem& s) {
   const int idx = blockIdx.x;
   int local, ctx, longest;   // longest: key tiles of the sequence's longest chunk
-  if (threadIdx.x == 0) s.past = 0;
+  if (ROWS == kRows && threadIdx.x == 0) s.past = 0;
   if (p.B > kOrderMax) {   // index order, unsplit
     const int rbmax = (p.max_nodes * p.G + ROWS - 1) / ROWS;
     it.b = idx / (rbmax * p.Hkv);
@@ -270,7 +310,8 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
       s.chunks[q] = 1;
       s.order[q] = make_int2(order_key(s.tiles[q], q), s.items[q]);
     }
-    const bool choice = CHOICE && p.alone && p.co_tiles >= 0;   // B <= 128: a sequence per thread
+    // B <= 128 here: a sequence per thread
+    const bool choice = MODE == kTwoTerms && p.alone && p.co_tiles >= 0;
     if (choice && threadIdx.x < kMaxNodes) {
       const int q = threadIdx.x;
       AloneTiles a{0, 0, 0};
@@ -317,7 +358,8 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
         const int2 o = s.order[j];
         first += o.x > mine.x ? o.y : 0;
       }
-      if (first + mine.y > static_cast<int>(gridDim.x)) atomicMax(&s.past, first + mine.y);
+      if (ROWS == kRows && first + mine.y > static_cast<int>(gridDim.x))
+        atomicMax(&s.past, first + mine.y);
       if (idx < first || idx >= first + mine.y) continue;
       if (p.part_cap > 0) {
         for (int j = 0; j < p.B; ++j) part += s.order[j].x > mine.x ? s.part[j] : 0;
@@ -362,12 +404,13 @@ __device__ __forceinline__ bool make_item(const AttnParams& p, Item& it, PlanSme
   return true;
 }
 
-// The items past the grid, which has a CTA for every item of sequences that do
-// not overlap: a batch whose cu_nodes run backwards (reported as ASD_ERR_TREE) can
-// make more, and its well-formed sequences keep their outputs.  Plain loops over
-// the keys, a warp per query row, by the eight softmax warps (tid: thread among
-// them) of every CTA when it is done.
-template <int D, int ROWS>
+// One-tile form: the items past the grid, which has a CTA for every item of
+// sequences that do not overlap.  A batch whose cu_nodes run backwards (reported as
+// ASD_ERR_TREE) can make more, and its well-formed sequences keep their outputs.
+// Plain loops over the keys, a warp per query row, by the eight softmax warps (tid:
+// thread among them) of every CTA when it is done.  (In the ping-pong form the
+// branch cost the tile loop 2 %; its grid covers every item instead.)
+template <int D>
 __device__ __forceinline__ void items_past_grid(const AttnParams& p, PlanSmem& s, int tid) {
   constexpr int kV = D / 32;   // a lane's columns
   const int lane = tid & 31;
@@ -384,9 +427,9 @@ __device__ __forceinline__ void items_past_grid(const AttnParams& p, PlanSmem& s
       if (idx == first && p.part_cap > 0) p.plan[q] = make_int2(0, 1);   // nothing to merge
     }
     softmax_sync();
-    const int b = s.seq, s0 = s.s0[b], R = s.n[b] * p.G, rb = (R + ROWS - 1) / ROWS;
-    const int g = (idx - s.first) / rb, r0 = (idx - s.first - g * rb) * ROWS;
-    for (int r = r0 + (tid >> 5); r < min(r0 + ROWS, R); r += kSoftmaxThreads / 32) {
+    const int b = s.seq, s0 = s.s0[b], R = s.n[b] * p.G, rb = (R + kRows - 1) / kRows;
+    const int g = (idx - s.first) / rb, r0 = (idx - s.first - g * rb) * kRows;
+    for (int r = r0 + (tid >> 5); r < min(r0 + kRows, R); r += kSoftmaxThreads / 32) {
       const int node = r / p.G;
       const size_t row = static_cast<size_t>(s0 + node) * p.Hq + g * p.G + (r - node * p.G);
       const __nv_bfloat16* qr = static_cast<const __nv_bfloat16*>(p.q) + row * D;
@@ -578,7 +621,7 @@ __device__ __forceinline__ float exp2_tile(const float* x, float c, float mu,
 }
 
 // The same, P as the sum of two bf16 numbers.  Calls of up to 128 nodes hand half
-// of P to the tensor cores so (TWO below): the mma.sync kernel, which took them
+// of P to the tensor cores so (kTwoTerms): the mma.sync kernel, which took them
 // before this one did, rescales to the running maximum of every 32 keys, which
 // makes the largest weights exact, and with P in one term this kernel's error
 // against 64 bits was up to 7 % above its.  Half of P in two terms leaves it 6 to
@@ -625,7 +668,7 @@ __device__ __forceinline__ float exp2_tile_two(const float* x, float c, float mu
 // until the end.  Returns false (uniformly over the eight warps) when a
 // bounded wait gave up; otherwise m_out and l_out are the row's reference max
 // and sum, with O complete in TMEM.
-template <int D, bool TWO>
+template <int D, int MODE>
 __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it, uint32_t tmem,
                                              uint8_t* gbase, int* s_par, uint64_t (*s_anc)[2],
                                              float (*s_mx)[2][kRows], float (*s_l)[kRows],
@@ -743,7 +786,7 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
       m_ref = mn;
     }
     const float mu = (m_ref == -INFINITY) ? 0.f : m_ref;
-    if (TWO) {   // the first 32 of this half's keys in two terms
+    if (MODE == kTwoTerms) {   // the first 32 of this half's keys
       uint32_t hi[16], lo[16], pk[16];
       l += exp2_tile_two<32>(x, c, mu, hi, lo);
       tmem_st16u(sb + 32 * hf, hi);
@@ -806,9 +849,7 @@ __device__ __forceinline__ bool softmax_role(const AttnParams& p, const Item& it
   return true;
 }
 
-// TWO: half of P in two bf16 terms (AttnParams::p_two: a call of up to 128 nodes, which
-// alone may be the mma.sync kernel's).
-template <int D, bool TWO>
+template <int D, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                    const __grid_constant__ CUtensorMap tm_tk,
@@ -836,8 +877,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ PlanSmem s_plan;
 
   pdl_launch_dependents();
+  if (MODE == kByContext && attention_takes_pairs(p)) {   // the ping-pong form's call
+    pdl_wait();
+    return;
+  }
   // the mma.sync kernel's step (a call by itself: make_item)
-  if (TWO && p.co_tiles >= 0 && !p.alone && attention_takes_mma(p)) {
+  if (MODE == kTwoTerms && p.co_tiles >= 0 && !p.alone && attention_takes_mma(p)) {
     pdl_wait();
     return;
   }
@@ -883,7 +928,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
   }
   Item it;
-  const bool some = make_item<kRows, TWO>(p, it, s_plan);   // uniform over the CTA
+  const bool some = make_item<kRows, MODE>(p, it, s_plan);   // uniform over the CTA
   tc_fence_after();
   if (!some) {   // no query rows here
     if (warp == 10) tmem_dealloc(s_tmem, kTmemCols);
@@ -988,7 +1033,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_mma_ts(tmem, tmem + kSCol0 + b * kKeys + kk * 8,
                       sw128_desc_mn(vst + kk * 2048, kKeys * 128, 1024), idesc_o,
                       (j > 0 || kk > 0) ? 1u : 0u);
-          if (TWO)   // second terms of keys 0-31 and 64-95
+          if (MODE == kTwoTerms)   // second terms of keys 0-31 and 64-95
 #pragma unroll
             for (int i = 0; i < 4; ++i)
               tc_mma_ts(tmem, tmem + kSCol0 + b * kKeys + kKeys / 2 + i * 8,
@@ -1010,7 +1055,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    ok = softmax_role<D, TWO>(p, it, tmem, gbase, s_par, s_anc, s_mx, s_l, &s_q_ready, s_s_full, s_p_full,
+    ok = softmax_role<D, MODE>(p, it, tmem, gbase, s_par, s_anc, s_mx, s_l, &s_q_ready, s_s_full, s_p_full,
                          s_pv_done, s_v_full, &s_abort, budget, m_row, l_row);
   }
 
@@ -1089,7 +1134,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   if (warp == 10) tmem_dealloc(tmem, kTmemCols);
   if (s_plan.past > 0 && warp >= 2 && warp < 10)
-    items_past_grid<D, kRows>(p, s_plan, threadIdx.x - 64);
+    items_past_grid<D>(p, s_plan, threadIdx.x - 64);
   pdl_wait();   // the next kernel's wait covers every earlier kernel
 }
 
@@ -1256,7 +1301,7 @@ __device__ __forceinline__ void regs_dec() {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
 }
 
-template <int D>
+template <int D, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_pp_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                    const __grid_constant__ CUtensorMap tm_tk,
@@ -1282,6 +1327,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ PlanSmem s_plan;
 
   pdl_launch_dependents();
+  if (MODE == kByContext && !attention_takes_pairs(p)) {   // the one-tile form's call
+    pdl_wait();
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long budget = wait_budget(p.wait_cycles);
 
@@ -1319,7 +1368,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
   }
   Item it;
-  const bool some = make_item<kPPRows, false>(p, it, s_plan);   // uniform over the CTA
+  const bool some = make_item<kPPRows, MODE>(p, it, s_plan);   // uniform over the CTA
   tc_fence_after();
   if (!some) {   // no query rows here
     if (warp == 2) tmem_dealloc(s_tmem, kTmemCols);
@@ -1642,8 +1691,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   if (warp == 2) tmem_dealloc(tmem, kTmemCols);
-  if (s_plan.past > 0 && warp >= 4)   // warps 0-3 gave up the registers for it
-    items_past_grid<D, kPPRows>(p, s_plan, threadIdx.x - 128);
   pdl_wait();   // the next kernel's wait covers every earlier kernel
 }
 
@@ -1660,22 +1707,37 @@ size_t attention_tc_smem_bytes(int head_dim, bool pingpong) {
 // the waves of CTAs: measured with 8 KV heads, G = 4, 152 SMs, one tile against
 // two, contiguous unless said.
 //   above 1.5 waves of pairs: 16 x 128 nodes 90.0 / 77.0 us, 24 x 128 133.6 /
-//     114.6, 32 x 60 at contexts 1000-4000 109.7 / 96.1, 48 x 33 149.5 / 124.5
+//     114.6, 32 x 60 at contexts 1000-6000 136 / 124, 48 x 33 149.5 / 124.5
 //   1 to 1.5 (three waves of single tiles against two of pairs): 12 x 128
 //     68.0 / 75.7, pages of 64 75.0 / 77.5, of 32 79.9 / 77.7, of 16 90.1 / 78.2;
-//     24 x 60 with pages of 16 89.7 / 78.8
-//   up to 1: 8 x 128 nodes 45.8 / 39.0, ragged 16 sequences of 20-100 nodes
-//     (0.9 of a wave) 68.3 / 65.7, but 15 of them (0.78) 54.0 / 63.7: the single
-//     tiles' second wave is then short
+//     20 x 60 (160 pairs) with pages of 16 89 / 78, at contexts 1000-6000 113 / 89
+//   up to 1: by the context lengths (attention_takes_pairs); below 5/6 of a wave the
+//     single tiles' second wave is short: 15 ragged sequences of 20-100 nodes (0.78
+//     of a wave) 54.0 / 63.7
 //   128 rows per sequence or fewer leave the second tile empty: 128 x 20 nodes
-//     153.8 / 157.6, 64 x 31 83.6 / 84.5
-bool attention_pingpong(int batch, int num_kv_heads, int G, int total_nodes, int page_size,
-                        int nsm) {
+//     153.8 / 157.6, 64 x 31 83.6 / 84.5; 257 to 384 rows make 3 tiles but 2 pairs
+//     (4 KV heads, G = 7): 32 x 40 71.1 / 86.2, 64 x 40 136.4 / 138.9
+// Pairs are counted for sequences of the average size; two waves of all rows are
+// enough whatever the sizes.
+PairRule attention_pair_rule(int batch, int num_kv_heads, int G, int total_nodes, int page_size,
+                             int nsm) {
   const long long rows = static_cast<long long>(total_nodes) * G;
-  if (batch <= 0 || rows <= static_cast<long long>(batch) * kRows) return false;
-  const long long items = static_cast<long long>(num_kv_heads) * ((rows + kPPRows - 1) / kPPRows);
-  if (items > nsm && 2 * items <= 3LL * nsm) return page_size > 0 && page_size <= 32;
-  return 6 * items >= 5LL * nsm;
+  if (batch <= 0 || rows <= static_cast<long long>(batch) * kRows) return PairRule::kOneTile;
+  const long long heads = num_kv_heads;
+  const long long least = heads * ((rows + kPPRows - 1) / kPPRows);
+  if (least >= 2LL * nsm) return PairRule::kPairs;
+  const long long avg = (rows + batch - 1) / batch;
+  const long long pairs = heads * batch * ((avg + kPPRows - 1) / kPPRows);
+  const long long tiles = heads * batch * ((avg + kRows - 1) / kRows);
+  const bool small = page_size > 0 && page_size <= 32;
+  if (10 * tiles < (small ? 14 : 17) * pairs || 6 * least < 5LL * nsm) return PairRule::kOneTile;
+  if (pairs <= nsm) return batch <= kPairSeqs ? PairRule::kByContext : PairRule::kOneTile;
+  return small || 2 * least > 3LL * nsm ? PairRule::kPairs : PairRule::kOneTile;
+}
+
+float attention_pair_ratio(int page_size) {
+  // a key tile of the one-tile form over a pair's (attention_takes_pairs)
+  return page_size == 0 ? 0.56f : page_size >= 32 ? 0.65f : 0.75f;
 }
 
 bool attention_q_tma_ok(int G) { return G >= 1 && kRows % G == 0; }
@@ -1687,19 +1749,28 @@ cudaError_t launch_attention_tc(const AttnParams& p, const CUtensorMap& tm_k,
   const size_t smem = attention_tc_smem_bytes(p.D, pingpong);
   if (p.D != 64 && p.D != 128) return cudaErrorInvalidValue;
   cudaError_t err;
-  // row blocks: at most max_nodes * G rows of each of B sequences, and T * G
-  // rows of which every sequence may leave one block ragged (sequences that overlap
-  // can make more: items_past_grid); index order (B > kOrderMax) numbers the first form
+  // row blocks: at most max_nodes * G rows of each of B sequences (index order, B >
+  // kOrderMax, numbers these; the ping-pong form's sequences are large, so that few
+  // of them lie idle), and T * G rows of which every sequence may leave one block
+  // ragged (sequences that overlap can make more: items_past_grid)
   const int rows = pingpong ? kPPRows : kRows;
   const long long full = static_cast<long long>((p.max_nodes * p.G + rows - 1) / rows) * p.B;
   const long long blocks =
-      p.B > kOrderMax ? full : std::min(full, static_cast<long long>(p.T) * p.G / rows + p.B);
+      p.B > kOrderMax || pingpong
+          ? full
+          : std::min(full, static_cast<long long>(p.T) * p.G / rows + p.B);
   const long long ctas =
       std::max<long long>(blocks * p.Hkv, p.part_cap > 0 ? p.nsm : 0);
   if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
-  auto* k = pingpong ? (p.D == 64 ? attn_pp_kernel<64> : attn_pp_kernel<128>)
-           : p.p_two ? (p.D == 64 ? attn_tc_kernel<64, true> : attn_tc_kernel<128, true>)
-                     : (p.D == 64 ? attn_tc_kernel<64, false> : attn_tc_kernel<128, false>);
+  const bool d64 = p.D == 64, by_context = p.pair_ratio > 0.f;
+  auto* k = d64 ? attn_tc_kernel<64, kPlain> : attn_tc_kernel<128, kPlain>;
+  if (pingpong)
+    k = by_context ? (d64 ? attn_pp_kernel<64, kByContext> : attn_pp_kernel<128, kByContext>)
+                   : (d64 ? attn_pp_kernel<64, kPlain> : attn_pp_kernel<128, kPlain>);
+  else if (by_context)
+    k = d64 ? attn_tc_kernel<64, kByContext> : attn_tc_kernel<128, kByContext>;
+  else if (p.p_two)
+    k = d64 ? attn_tc_kernel<64, kTwoTerms> : attn_tc_kernel<128, kTwoTerms>;
   err = set_smem_attrs(k, smem);
   if (err != cudaSuccess) return err;
   err = launch_pdl(k, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), smem, s, tm_k, tm_v, tm_tk,

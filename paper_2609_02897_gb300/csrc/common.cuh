@@ -51,8 +51,8 @@ struct WsLayout {
   size_t lz_h;         // bf16[2][lz_cap][hidden]: their hidden rows
   int lz_cap;          // T rounded up to 128
   int attn_tc;         // tensor-core attention (attention has the SMs to itself): 1 one
-                       // query tile per CTA, 2 two query tiles in ping-pong; 0: the bf16
-                       // mma.sync or the fp32 kernel
+                       // query tile per CTA, 2 two query tiles in ping-pong, 3 either, by
+                       // the context lengths; 0: the bf16 mma.sync or the fp32 kernel
 };
 
 // ---------------------------------------------------------------- device utils

@@ -89,6 +89,9 @@ struct AttnParams {
   // without an LM head and with several items per SM (attention_alone_rule)
   int co_tiles;
   int alone;
+  // calls that the context lengths decide between the two tensor-core forms about:
+  // attention_pair_ratio (0: no choice)
+  float pair_ratio;
   // one-tile tensor-core kernel: half of P goes to the P.V MMA in two bf16 terms
   // (calls of up to 128 nodes, which another kernel took before)
   int p_two;
@@ -177,13 +180,16 @@ int attention_keys_per_tile();   // context keys per K/V tile = TMA box rows
 // tm_q (with p.q_tma, where attention_q_tma_ok(G)): a 3D map over
 // q [T, Hq, D] with boxes of 64 columns x G heads x kAttnTcRows / G nodes.
 // pingpong: the two-query-tile form (256 rows per CTA: one tile's MMAs run
-// during the other's softmax), chosen by attention_pingpong() by how many
-// waves of CTAs its items make.
+// during the other's softmax), chosen by attention_pair_rule() by how many waves of
+// CTAs its items make, and about one wave by the context lengths: both forms are
+// then launched and decide alike.
 constexpr int kAttnTcRows = 128;   // query rows per CTA (per tile of the ping-pong form)
 constexpr int kAttnTcKeys = 128;   // keys per tile
 size_t attention_tc_smem_bytes(int head_dim, bool pingpong);
-bool attention_pingpong(int batch, int num_kv_heads, int G, int total_nodes, int page_size,
-                        int nsm);
+enum class PairRule { kOneTile, kPairs, kByContext };
+PairRule attention_pair_rule(int batch, int num_kv_heads, int G, int total_nodes, int page_size,
+                             int nsm);
+float attention_pair_ratio(int page_size);
 // Partial rows that the one-tile kernel can use to cut sequences into chunks
 // (0: the items of these dims and nodes fill the GPU anyway).
 long long attention_split_rows(const asd_dims& d, int total_nodes, int nsm);

@@ -65,3 +65,46 @@ def test_which_form_a_call_takes():
     assert [form(low - 1, 16), form(nsm + 1, 32), form(half, 16), form(half, 64)] == [2, 3, 3, 2]
     # 128 rows per sequence on average: the second query tile would stay empty
     assert form(4 * nsm) == 3 and form(4 * nsm, batch=8 * nsm) == 2
+
+    def of_nodes(n, batch, G):
+        dims = asd.make_dims(batch, G, 1, 128, 64, 64, asd.ASD_BF16, 0, 1024, 0, 128, 8)
+        return asd.asd_attention_variant(dims, n * batch)
+
+    # 100 nodes of G = 3 are 300 rows: three tiles, but two pairs, the second half
+    # empty; from two waves of all rows on pairs whatever the sizes
+    assert [of_nodes(100, 7 * nsm * 256 // 4 // 300, 3), of_nodes(100, 2 * nsm, 3)] == [2, 3]
+
+
+def test_about_one_wave_of_pairs_the_contexts_decide():
+    """Equal contexts run the two-tile form, a batch whose longest context stands
+    out single tiles, at both sides of the line; told by the bits of the same
+    sequences in a batch of fewer (single tiles) and of more (pairs)."""
+    import torch
+    from paper_2609_02897_gb300 import asd
+    Hq, Hkv, D, n, cap = 32, 8, 128, 128, 4096
+    nsm = torch.cuda.get_device_properties(0).multi_processor_count
+    mid, few, many = nsm // 16, 5 * nsm // 6 // 16 - 1, 3 * nsm // 2 // 16 + 1   # 16 pairs each
+    g = 1024 // 128 + 1              # key tiles of the others, the tree's among them
+    # the longest, t tiles: t <= 0.56 max(t, 1.15 work / nsm) + 3, 32 items each
+    line = max(t for t in range(g, 33)
+               if t <= 0.56 * max(t, 1.15 * 32 * (t + g * (mid - 1)) / nsm) + 3)
+    assert g < line < 32
+
+    def run(B, ctx):
+        d = dict(full, ctx_len=torch.tensor(ctx, dtype=torch.int32, device="cuda"))
+        for k in ("q", "tree_k", "tree_v", "parent"):
+            d[k] = full[k][:B * n].contiguous()
+        for k in ("k_cache", "v_cache"):
+            d[k] = full[k][:B].contiguous()
+        d["cu_nodes"] = torch.arange(0, B * n + 1, n, dtype=torch.int32, device="cuda")
+        dims = asd.make_dims(B, Hq, Hkv, D, 64, 64, asd.ASD_BF16, 0, cap, 0, n, n)
+        assert asd.asd_attention_variant(dims, B * n) == (2 if B == few else 3)
+        return _call(d, dims, asd.alloc_workspace(dims, B * n))[:few * n].view(torch.int16)
+
+    full = _inputs(many, n, [0] * many, 0, Hq, Hkv, D, cap, 3)
+    for longest, pairs in ((g, True), (line, True), (line + 1, False), (32, False)):
+        ctx = [1024] * many
+        ctx[1] = 128 * (longest - 1)
+        out, single, double = run(mid, ctx[:mid]), run(few, ctx[:few]), run(many, ctx)
+        assert not torch.equal(single, double)
+        assert torch.equal(out, double if pairs else single), (longest, pairs)
