@@ -14,8 +14,9 @@
 // the pass, writes what was reached, and lists the next pass.  Rows that were
 // computed ahead and not reached leave no trace.
 //
-// 32 sequences of 128 nodes at tau 1 (contexts of 2048 to 4096): three W passes
-// instead of eleven, the whole step 1723 -> 837 us.
+// 32 sequences of 128 nodes at tau 1 (contexts of 2048 to 4096): two or three W
+// passes by the inputs instead of nine to eleven, the whole step 1784 -> 837 us (the
+// same inputs, with three).
 //
 // The merge of the partials and the kappa rule are the tail kernel's, in the
 // same order, so every computed row and verdict is bit-identical to the
