@@ -23,11 +23,12 @@
 // them.  The CTAs take the chunks in decreasing order of work, so the longest
 // start first.  The rows of a pair are its N nodes times the G query heads that
 // share the KV head, node-major (row r -> node r / G, head g*G + r % G); row r
-// lives in TMEM lane r.  Keys come in tiles of 128, K and V through TMA rings of their own (128-byte swizzle; paged caches one
-// box per page; the tree K/V through a 3D map over [T, Hkv, D]), so a K slot
-// is refilled as soon as its S MMA is done rather than after the tile's P.V;
-// the last tile of a pair holds its tree keys, where a node sees only its
-// ancestors (bitmasks derived here from the parent array).
+// lives in TMEM lane r.  Keys come in tiles of 128, K and V through TMA rings of
+// their own (128-byte swizzle; paged caches one box per page; the tree K/V
+// through a 3D map over [T, Hkv, D]), so a K slot is refilled as soon as its S
+// MMA is done rather than after the tile's P.V; the last tile of a pair holds
+// its tree keys, where a node sees only its ancestors (bitmasks derived here
+// from the parent array).
 //
 //   Q             loaded once into shared memory by one TMA (G dividing 128:
 //                 boxes of G heads x 128/G nodes), else by the softmax warps
